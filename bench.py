@@ -49,8 +49,10 @@ MUFU_EX2_PER_S = 9.5e12
 
 # roofline bound of each kernel: (bound, which algorithmic quantity)
 KERNEL_BOUND = {
-    "mma_gemm": ("tensor", "flops"),
-    "simt_prep": ("alu", "flops"),
+    "tile_delta": ("tensor", "flops"),
+    "tile_out": ("tensor", "flops"),
+    "tile_bwd_q": ("tensor", "flops"),
+    "tile_bwd_k": ("tensor", "flops"),
     "tc_fwd": ("tensor", "flops"),
     "tc_bwd": ("tensor", "flops"),
     "tc_bwd_q": ("tensor", "flops"),

@@ -12,10 +12,9 @@ namespace prof {
 namespace {
 
 const char* kNames[K_COUNT] = {
-    "mma_gemm",    "simt_prep",     "simt_scan",      "simt_finalize", "simt_dstat",
-    "simt_vjp",    "simt_store",    "simt_reduce",    "simt_state",    "tc_fwd",
-    "tc_bwd",      "tc_delta",      "tc_scan",        "tc_bwd_q",      "tc_bwd_kv",
-    "tc_reduce",   "tc_selftest",   "tc_prep",        "stack_rows"};
+    "simt_prep",  "simt_scan",  "simt_reduce", "tc_fwd",      "tc_bwd",     "tc_delta",
+    "tc_scan",    "tc_bwd_q",   "tc_bwd_kv",   "tc_reduce",   "tc_selftest", "tc_prep",
+    "stack_rows", "tile_delta", "tile_out",    "tile_bwd_q",  "tile_bwd_k"};
 
 struct Rec {
   Kid k;

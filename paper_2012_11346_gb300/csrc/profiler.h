@@ -7,15 +7,9 @@ namespace prof {
 
 // Every kernel of the library, by name.
 enum Kid {
-  K_GEMM = 0,
-  K_PREP,
+  K_PREP = 0,
   K_SCAN,
-  K_FINALIZE,
-  K_DSTAT,
-  K_VJP,
-  K_STORE,
   K_REDUCE,
-  K_STATE,
   K_TC_FWD,
   K_TC_BWD,
   K_TC_DELTA,
@@ -26,6 +20,10 @@ enum Kid {
   K_TC_SELFTEST,
   K_TC_PREP,
   K_STACK,
+  K_TILE_DELTA,
+  K_TILE_OUT,
+  K_TILE_BWD_Q,
+  K_TILE_BWD_K,
   K_COUNT
 };
 

@@ -5,11 +5,13 @@
 namespace slim {
 namespace simt {
 
-size_t workspace_bytes(const Problem& p, bool bwd);
+// small: the least workspace the forward runs in (fwd takes any size from there
+// on, and sweeps fewer rows and chains at a time below the full size)
+size_t workspace_bytes(const Problem& p, bool bwd, bool small = false);
 
 slim_status fwd(const Problem& p, const void* q, const void* k, const void* v,
                 const float* omega, void* out, const StateOut& st, const StateInit& init,
-                void* workspace, cudaStream_t s);
+                void* workspace, size_t bytes, cudaStream_t s);
 
 slim_status bwd(const Problem& p, const void* q, const void* k, const void* v,
                 const float* omega, const void* out, const void* dout, const StateIn& st,

@@ -1,0 +1,1724 @@
+// Tile kernels of the fp32-compute path.
+//
+// A tile is 64 rows of one chain.  Operands are split once into bf16 pieces
+// (NX for a caller's rows: 1 for bf16, 3 for fp32; NS for everything computed:
+// 2 for bf16 problems, 3 for fp32 ones) when they enter shared memory or become
+// an MMA fragment, and every product of a tile stays in the CTA: nothing but
+// the tile's state, its g(K) and its results goes through global memory.
+// Products run as warp MMAs (m16n8k16): the pieces of a 64-row tile with
+// M = 256 features would leave no room for tcgen05's 128-row operand tiles, and
+// an accumulator that already sits in registers becomes the next product's
+// operand without a trip through shared memory.  m16n8k16 bf16 measured 600
+// TFLOP/s on a GB300 (1.86 PFLOP/s for tcgen05), with 3 (bf16) or 6 (fp32)
+// piece products per product: that rate bounds these kernels.
+#pragma once
+#include <math.h>
+
+#include "profiler.h"
+#include "simt_tiles.h"
+#include "warp_mma.cuh"
+
+namespace slim {
+namespace simt {
+
+constexpr int kThreads = 256;  // 8 warps
+constexpr int kChunk = 32;     // features staged at a time by the row kernels
+constexpr int kSmemMax = 232448;
+
+template <typename IO> struct Pieces;
+template <> struct Pieces<bf16> { static constexpr int NX = 1, NS = 2; };
+template <> struct Pieces<float> { static constexpr int NX = 3, NS = 3; };
+
+__device__ __forceinline__ void load8(const bf16* p, float (&v)[8]) {
+  const uint4 r = *reinterpret_cast<const uint4*>(p);
+  const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float2 f = unpack2(w[i]);
+    v[2 * i] = f.x;
+    v[2 * i + 1] = f.y;
+  }
+}
+__device__ __forceinline__ void load8(const float* p, float (&v)[8]) {
+  const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
+  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+// 8 consecutive values as NP pieces (piece stride ps)
+template <int NP>
+__device__ __forceinline__ void store_pieces8(bf16* dst, int ps, const float (&v)[8]) {
+  uint32_t w[4][NP];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) split_pair<NP>(v[2 * i], v[2 * i + 1], w[i]);
+#pragma unroll
+  for (int p = 0; p < NP; ++p)
+    *reinterpret_cast<uint4*>(dst + p * ps) = make_uint4(w[0][p], w[1][p], w[2][p], w[3][p]);
+}
+
+// a staged element's value (the sum of its pieces, exact for a caller's rows)
+template <int NP>
+__device__ __forceinline__ float staged(const bf16* p, int ps) {
+  float v = __bfloat162float(p[(NP - 1) * ps]);
+#pragma unroll
+  for (int i = NP - 2; i >= 0; --i) v += __bfloat162float(p[i * ps]);
+  return v;
+}
+
+// x . omega as a compensated dot product (FMA TwoProduct and TwoSum, about 48
+// bits; Ogita, Rump and Oishi's Dot2): decides ReLU's branch where the
+// projection's own error could.
+template <typename IO>
+__device__ __noinline__ float dot2(const IO* x, const float* om, int d) {
+  float sh = 0.f, sl = 0.f;
+  for (int j = 0; j < d; ++j) {
+    const float xw = Io<IO>::load(x, j), ow = om[j];
+    const float p = __fmul_rn(xw, ow), ep = __fmaf_rn(xw, ow, -p);
+    float t, e;
+    two_sum(sh, p, t, e);
+    sh = t;
+    sl = __fadd_rn(sl, __fadd_rn(e, ep));
+  }
+  return __fadd_rn(sh, sl);
+}
+
+// g(x)_f from the projection `dot` of row x (global, for ReLU's recheck).  The
+// recheck bound covers the accumulation of the 6 (3) piece products over d / 16
+// MMA steps, each step's truncation taken as 2^-23 of |omega| |x|, with a
+// factor of 2 to spare.
+template <typename IO>
+__device__ __forceinline__ float feature_value(const TileArgs& A, float dot, float half_norm, int f,
+                                               const IO* x, int d) {
+  if (A.feature == SLIM_FEAT_EXP) return expf(dot - half_norm) * A.inv_sqrt_m;
+  const float gamma = 4.f * (float)(d + 2) * 5.9604645e-08f;
+  if (fabsf(dot) <= gamma * A.om_norm[f] * sqrtf(2.f * half_norm))
+    dot = dot2<IO>(x, A.omega + (size_t)f * d, d);
+  return dot > 0.f ? dot * A.inv_sqrt_m : 0.f;
+}
+
+// A frame is the 64 rows a CTA works on: one tile of 48 or 64 rows, two of 32
+// or four of 16 (each padded from its A.pitch rows to A.rows).
+struct Frame {
+  int c, t0, left;  // chain, first tile, rows of the sequence from the frame's first on
+  size_t row0;      // first row in a caller tensor
+};
+__device__ __forceinline__ Frame frame_pos(const TileArgs& A, int frame) {
+  Frame f;
+  f.c = frame / A.nf;
+  f.t0 = frame % A.nf * A.per;
+  f.left = A.b - f.t0 * A.pitch;
+  f.row0 = (size_t)f.c * A.L + A.a + (size_t)f.t0 * A.pitch;
+  return f;
+}
+// caller row (from the frame's first) of frame row r, -1 for a padding row
+__device__ __forceinline__ int frame_row(const TileArgs& A, const Frame& f, int r) {
+  const int i = r >> A.shift, rr = r - (i << A.shift), x = i * A.pitch + rr;
+  return rr < A.pitch && x < f.left ? x : -1;
+}
+
+// The frame's rows of one caller tensor (src: its first row; padding rows are
+// zero) as pieces [NX][64][D + 8]; half_norm (when given): 0.5 |x|^2 per row.
+// D / 8 neighbouring lanes share a row.
+template <typename IO, int D>
+__device__ __forceinline__ void load_rows(const TileArgs& A, const Frame& f, const IO* src, bf16* dst,
+                                          float* half_norm) {
+  constexpr int NX = Pieces<IO>::NX, PD = D + 8, G = D / 8;
+  for (int e = threadIdx.x; e < kTile * G; e += kThreads) {
+    const int r = e / G, c8 = (e % G) * 8, x = frame_row(A, f, r);
+    float v[8] = {};
+    if (x >= 0) load8(src + (size_t)x * D + c8, v);
+    store_pieces8<NX>(dst + r * PD + c8, kTile * PD, v);
+    if (half_norm) {
+      float s = 0.f;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) s = fmaf(v[i], v[i], s);
+#pragma unroll
+      for (int o = 1; o < G; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (c8 == 0) half_norm[r] = 0.5f * s;
+    }
+  }
+}
+
+// ------------------------------------------------------------------ FMA projections
+// The forward's features (and the backward's of fp32 problems with d <= 32) come
+// from fp32 FMAs, one per term in j order: an MMA's truncating sum of 16 products
+// is a few times less exact, which the exponential passes on whole.  A CTA
+// projects 64 rows onto W = 64 or 32 features at a time; a thread has rows rt,
+// rt + 16, rt + 32, rt + 48 and W / 16 neighbouring features, 16 FMAs per
+// feature for every 4 + W / 16 16-byte (8-byte) shared-memory reads, which is
+// bound by the FMA issue rate for W = 64.
+template <int D>
+constexpr int fp_pitch() { return D + 4; }  // floats: 4 neighbouring rows fall into 4 bank groups
+
+// fp32 rows of a frame and their |x|^2 (summed as one warp's lanes do: strided
+// terms, then a butterfly); needs a __syncthreads before the rows are read.
+template <typename IO, int D>
+__device__ __forceinline__ void load_rows_fp(const TileArgs& A, const Frame& f, const IO* src, float* xs) {
+  constexpr int G = D / 8, XP = fp_pitch<D>();
+  for (int e = threadIdx.x; e < kTile * G; e += kThreads) {
+    const int r = e / G, c8 = (e % G) * 8, x = frame_row(A, f, r);
+    float v[8] = {};
+    if (x >= 0) load8(src + (size_t)x * D + c8, v);
+    float4* d = reinterpret_cast<float4*>(xs + r * XP + c8);
+    d[0] = make_float4(v[0], v[1], v[2], v[3]);
+    d[1] = make_float4(v[4], v[5], v[6], v[7]);
+  }
+}
+template <int D>
+__device__ __forceinline__ void row_norms(const float* xs, float* norm2) {
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  for (int r = warp; r < kTile; r += kThreads / 32) {
+    float s = 0.f;
+#pragma unroll
+    for (int j = lane; j < D; j += 32) s = fmaf(xs[r * fp_pitch<D>() + j], xs[r * fp_pitch<D>() + j], s);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) norm2[r] = s;
+  }
+}
+// W features of Omega, columns c0.. of its [M / 64][D][64] layout, to [D][W]
+template <int D, int W>
+__device__ __forceinline__ void stage_omega(float* dst, const float* om_t, int c0) {
+  const float* src = om_t + (size_t)(c0 / 64) * D * 64 + c0 % 64;
+  for (int e = threadIdx.x; e < D * W / 4; e += kThreads) {
+    const int j = e / (W / 4), q = (e % (W / 4)) * 4;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst + j * W + q)),
+                 "l"(src + (size_t)j * 64 + q)
+                 : "memory");
+  }
+}
+// x . omega as a compensated dot product (FMA TwoProduct and TwoSum, about 48
+// bits; Ogita, Rump and Oishi's Dot2): decides ReLU's branch where the
+// projection's own error could.
+static __device__ __noinline__ float dot2_staged(const float* x, const float* om, int stride, int d) {
+  float sh = 0.f, sl = 0.f;
+  for (int j = 0; j < d; ++j) {
+    const float xw = x[j], ow = om[j * stride];
+    const float p = __fmul_rn(xw, ow), ep = __fmaf_rn(xw, ow, -p);
+    float t, e;
+    two_sum(sh, p, t, e);
+    sh = t;
+    sl = __fadd_rn(sl, __fadd_rn(e, ep));
+  }
+  return __fadd_rn(sh, sl);
+}
+// g of the frame's 64 rows at features c0 .. c0 + W - 1 (0 in padding rows and
+// past M); put(row, feature offset, W / 16 values) stores them.
+// NI: the row groups (16 rows) to compute; the rest of the frame gets 0.
+template <int D, int W, int NI, typename Put>
+__device__ __forceinline__ void features_rows(const TileArgs& A, const Frame& f, const float* xs,
+                                            const float* norm2, const float* om, int c0, Put put) {
+  constexpr int XP = fp_pitch<D>(), NF = W / 16;
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int fq = ((warp & 1) * 8 + lane % 8) * NF, rt = (warp >> 1) * 4 + lane / 8;
+  float acc[NI][NF] = {};
+  if (A.feature == SLIM_FEAT_SQUARE) {
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+#pragma unroll
+      for (int n = 0; n < NF; ++n)
+        if (c0 + fq + n < D) {
+          const float x = xs[(rt + 16 * i) * XP + c0 + fq + n];
+          acc[i][n] = x * x;
+        }
+  } else {
+#pragma unroll 4
+    for (int j = 0; j < D; j += 4) {
+      float x[NI][4], o[4][NF];
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        const float4 v = *reinterpret_cast<const float4*>(xs + (rt + 16 * i) * XP + j);
+        x[i][0] = v.x; x[i][1] = v.y; x[i][2] = v.z; x[i][3] = v.w;
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (NF == 4) {
+          const float4 v = *reinterpret_cast<const float4*>(om + (j + k) * W + fq);
+          o[k][0] = v.x; o[k][1] = v.y; o[k][NF - 2] = v.z; o[k][NF - 1] = v.w;
+        } else {
+          const float2 v = *reinterpret_cast<const float2*>(om + (j + k) * W + fq);
+          o[k][0] = v.x; o[k][1] = v.y;
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int i = 0; i < NI; ++i)
+#pragma unroll
+          for (int n = 0; n < NF; ++n) acc[i][n] = fmaf(x[i][k], o[k][n], acc[i][n]);
+    }
+    // error bound of an fp32 dot product of length D, times a safety factor 2
+    const float gamma = 2.f * (float)(D + 2) * 5.9604645e-08f;
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      const int r = rt + 16 * i;
+      const bool ok = frame_row(A, f, r) >= 0;
+      const float n2 = norm2[r];
+#pragma unroll
+      for (int n = 0; n < NF; ++n) {
+        float v = 0.f;
+        if (ok && c0 + fq + n < A.M) {
+          v = acc[i][n];
+          if (A.feature == SLIM_FEAT_EXP) {
+            v = expf(v - 0.5f * n2) * A.inv_sqrt_m;
+          } else {
+            if (fabsf(v) <= gamma * A.om_norm[c0 + fq + n] * sqrtf(n2))
+              v = dot2_staged(xs + r * XP, om + fq + n, W, D);
+            v = v > 0.f ? v * A.inv_sqrt_m : 0.f;
+          }
+        }
+        acc[i][n] = v;
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < NI; ++i) put(rt + 16 * i, fq, acc[i]);
+  const float zero[NF] = {};
+#pragma unroll
+  for (int i = NI; i < 4; ++i) put(rt + 16 * i, fq, zero);
+}
+// A frame whose rows all lie in its first 16 (a few new rows on a running state)
+// projects those alone.
+template <int D, int W, typename Put>
+__device__ __forceinline__ void features_fp(const TileArgs& A, const Frame& f, const float* xs,
+                                            const float* norm2, const float* om, int c0, Put put) {
+  if (f.left <= (A.pitch < 16 ? A.pitch : 16))
+    features_rows<D, W, 1>(A, f, xs, norm2, om, c0, put);
+  else
+    features_rows<D, W, 4>(A, f, xs, norm2, om, c0, put);
+}
+
+constexpr int kPF = 64 + 8;  // row pitch of the forward's 64 x 64 chunk tiles
+
+// features_fp into pieces [NS][64][kPF]
+template <int D, int NS>
+__device__ __forceinline__ void features_to_pieces(const TileArgs& A, const Frame& f, const float* xs,
+                                                   const float* norm2, const float* om, int c0,
+                                                   bf16* dst) {
+  features_fp<D, 64>(A, f, xs, norm2, om, c0, [&](int r, int fo, const float(&v)[4]) {
+    uint32_t a[NS], b[NS];
+    split_pair<NS>(v[0], v[1], a);
+    split_pair<NS>(v[2], v[3], b);
+#pragma unroll
+    for (int p = 0; p < NS; ++p)
+      *reinterpret_cast<uint2*>(dst + (p * 64 + r) * kPF + fo) = make_uint2(a[p], b[p]);
+  });
+}
+
+// the fp32 value of staged pieces, smallest piece first
+template <int NP>
+__device__ __forceinline__ void add_pieces8(const bf16* p, int ps, float (&v)[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = 0.f;
+#pragma unroll
+  for (int q = NP - 1; q >= 0; --q) {
+    float w[8];
+    load8(p + q * ps, w);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] += w[i];
+  }
+}
+template <int NP>
+__device__ __forceinline__ float round_pieces(float x) {
+  float pc[NP];
+  split_bf16<NP>(x, pc);
+  float v = 0.f;
+#pragma unroll
+  for (int q = NP - 1; q >= 0; --q) v += pc[q];
+  return v;
+}
+// D += A b for one n8 block, A's pieces smallest first
+template <int NA>
+__device__ __forceinline__ void mma_n8(float (&d)[4], const uint32_t (&a)[NA][4], uint32_t b0, uint32_t b1) {
+#pragma unroll
+  for (int i = NA - 1; i >= 0; --i) mma16816(d, a[i], b0, b1);
+}
+constexpr uint32_t kOnes = 0x3f803f80u;  // two bf16 ones
+
+// ------------------------------------------------------------------ Delta_t
+// One CTA per frame: g(K) and, tile by tile, Delta_t = g(K)^T [V | 1].  Features
+// are taken 64 at a time: project (FMA pipe), split into pieces in shared memory,
+// then the tile products from there.  g(K)'s pieces are kept for the kernels that
+// read the frame's keys.  The z column (sum of g(K) over the tile's rows) is a
+// running fp32 sum in row order for d >= 64 and a column of ones in the MMAs
+// otherwise.
+// Forward and backward call this kernel on the same tiles, so the backward's
+// rollback subtracts exactly what the forward added.
+template <typename IO, int D>
+struct DeltaSmem {
+  static constexpr int NX = Pieces<IO>::NX, NS = Pieces<IO>::NS, PD = D + 8;
+  static constexpr int xs = kTile * fp_pitch<D>() * 4, om = D * 64 * 4, v = NX * kTile * PD * 2,
+                       ph = NS * 64 * kPF * 2;
+  static constexpr int bytes = xs + om + v + ph + kTile * 4;
+  static_assert(bytes <= kSmemMax, "shared memory");
+};
+
+template <typename IO, int D>
+__global__ void __launch_bounds__(kThreads, 2) k_delta(const __grid_constant__ TileArgs A) {
+  using S = DeltaSmem<IO, D>;
+  constexpr int NX = S::NX, NS = S::NS, PD = S::PD;
+  constexpr int CW = D >= 32 ? D / 2 : 16, NB = CW / 8;  // columns of a warp
+  extern __shared__ uint4 smem_raw[];
+  float* xs = reinterpret_cast<float*>(smem_raw);
+  float* om = xs + S::xs / 4;
+  bf16* Vs = reinterpret_cast<bf16*>(om + S::om / 4);
+  bf16* Ph = Vs + S::v / 2;
+  float* norm2 = reinterpret_cast<float*>(Ph + S::ph / 2);
+  pdl_wait();
+  pdl_launch();
+  const int frame = blockIdx.x;
+  const Frame f = frame_pos(A, frame);
+  const bool square = A.feature == SLIM_FEAT_SQUARE;
+  if (!square) {
+    stage_omega<D, 64>(om, A.om_t, 0);
+    cp_commit();
+  }
+  load_rows_fp<IO, D>(A, f, static_cast<const IO*>(A.k) + f.row0 * D, xs);
+  load_rows<IO, D>(A, f, static_cast<const IO*>(A.v) + f.row0 * D, Vs, nullptr);
+  __syncthreads();
+  row_norms<D>(xs, norm2);
+
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32, g = lane >> 2, t = lane & 3;
+  const int fb = warp & 3, h = warp >> 2;  // 16 features of the chunk, half of the columns
+  const int ksteps = A.rows / 16;          // k16 steps per tile
+  // two reduction groups (even and odd steps) for few features
+  const bool two = A.rows == 64 && (A.M == 32 || (A.M == 16 && NS == 3));
+  float* dl = A.delta + ((size_t)f.c * A.nt + f.t0) * A.E;
+  bf16* pk = A.phi_k ? A.phi_k + (size_t)frame * NS * 64 * A.M : nullptr;
+  const int ntl = min(A.per, A.nt - f.t0);  // tiles of this frame
+  for (int c0 = 0; c0 < A.M; c0 += 64) {
+    cp_wait<0>();
+    __syncthreads();
+    features_to_pieces<D, NS>(A, f, xs, norm2, om, c0, Ph);
+    __syncthreads();
+    if (!square && c0 + 64 < A.M) {
+      stage_omega<D, 64>(om, A.om_t, c0 + 64);
+      cp_commit();
+    }
+    const int nf = min(64, A.M - c0);
+    if (pk)
+      for (int e = tid; e < 64 * (nf / 8); e += kThreads) {
+        const int r = e / (nf / 8), c8 = (e % (nf / 8)) * 8;
+#pragma unroll
+        for (int p = 0; p < NS; ++p)
+          *reinterpret_cast<uint4*>(pk + ((size_t)p * 64 + r) * A.M + c0 + c8) =
+              *reinterpret_cast<const uint4*>(Ph + (p * 64 + r) * kPF + c8);
+      }
+    if (16 * fb < nf) {
+      const int f0 = c0 + 16 * fb + g;
+      float a0[NB][4] = {}, a1[NB][4] = {}, z0[4] = {}, z1[4] = {};
+#pragma unroll
+      for (int ks = 0; ks < 4; ++ks) {
+        const int i = 16 * ks >> A.shift, last = ks == ksteps * (i + 1) - 1;
+        if (ks >= ksteps * ntl) break;
+        uint32_t a[NS][4];
+        ld_at<NS>(a, Ph, 64 * kPF, kPF, 16 * fb, 16 * ks);
+        const bool g1 = two && (ks & 1);
+        if (D >= 32 || h == 0) {
+#pragma unroll
+          for (int nb = 0; nb < NB / 2; ++nb) {
+            uint32_t b[NX][4];
+            ld_bt<NX>(b, Vs, kTile * PD, PD, (D >= 32 ? CW * h : 0) + 16 * nb, 16 * ks);
+            if (g1)
+              mma_pieces<NS, NX>(a1[2 * nb], a1[2 * nb + 1], a, b);
+            else
+              mma_pieces<NS, NX>(a0[2 * nb], a0[2 * nb + 1], a, b);
+          }
+        }
+        if (D < 64 && h == 1) {
+          const uint32_t one = g == 0 ? kOnes : 0u;
+          if (g1)
+            mma_n8<NS>(z1, a, one, one);
+          else
+            mma_n8<NS>(z0, a, one, one);
+        }
+        if (last) {
+          float* dt = dl + (size_t)i * A.E;
+          if (D >= 32 || h == 0) {
+#pragma unroll
+            for (int nb = 0; nb < NB; ++nb) {
+              if (two)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) a0[nb][c] += a1[nb][c];
+              float* dst = dt + (size_t)f0 * D + (D >= 32 ? CW * h : 0) + 8 * nb + 2 * t;
+              *reinterpret_cast<float2*>(dst) = make_float2(a0[nb][0], a0[nb][1]);
+              *reinterpret_cast<float2*>(dst + 8 * D) = make_float2(a0[nb][2], a0[nb][3]);
+#pragma unroll
+              for (int c = 0; c < 4; ++c) a0[nb][c] = 0.f;
+            }
+          }
+          if (D < 64 && h == 1) {
+            if (two)
+#pragma unroll
+              for (int c = 0; c < 4; ++c) z0[c] += z1[c];
+            if (t == 0) {
+              dt[A.M * D + f0] = z0[0];
+              dt[A.M * D + f0 + 8] = z0[2];
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) z0[c] = 0.f;
+          }
+        }
+      }
+    }
+    if (D >= 64) {  // z: a lane sums two neighbouring features over one tile's rows
+      const int i = (warp - (c0 / 64) * A.per) & 7;  // the duty moves from warp to warp
+      if (i < ntl && 2 * lane < nf) {
+        const bf16* p = Ph + (size_t)i * A.rows * kPF + 2 * lane;
+        float s[2][2] = {};
+        for (int k0 = 0; k0 < A.rows; k0 += 16) {
+          const bool g1 = two && (k0 & 16);
+          float x = g1 ? s[1][0] : s[0][0], y = g1 ? s[1][1] : s[0][1];
+#pragma unroll
+          for (int k = 0; k < 16; ++k) {
+            float2 v = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int q = NS - 1; q >= 0; --q) {
+              const float2 w = unpack2(*reinterpret_cast<const uint32_t*>(p + (q * 64 + k0 + k) * kPF));
+              v.x += w.x;
+              v.y += w.y;
+            }
+            x += v.x;
+            y += v.y;
+          }
+          if (g1) {
+            s[1][0] = x;
+            s[1][1] = y;
+          } else {
+            s[0][0] = x;
+            s[0][1] = y;
+          }
+        }
+        if (two) {
+          s[0][0] += s[1][0];
+          s[0][1] += s[1][1];
+        }
+        *reinterpret_cast<float2*>(dl + (size_t)i * A.E + A.M * D + c0 + 2 * lane) = make_float2(s[0][0], s[0][1]);
+      }
+    }
+  }
+}
+
+// A chunk (up to R rows) of a state's S (fp32 rows of D) on its way to shared
+// memory as pieces: held in registers between load and store, so that the loads
+// overlap a chunk's products.
+template <int D, int R>
+struct StateChunk {
+  static constexpr int N = (R * D / 8 + kThreads - 1) / kThreads;
+  float v[N][8];
+  __device__ __forceinline__ void load(const float* S, int rows) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const int e = threadIdx.x + i * kThreads;
+      if (e < rows * (D / 8)) load8(S + (size_t)e * 8, v[i]);
+    }
+  }
+  template <int NP>
+  __device__ __forceinline__ void store(bf16* dst, int rows) const {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const int e = threadIdx.x + i * kThreads;
+      if (e < rows * (D / 8))
+        store_pieces8<NP>(dst + (e / (D / 8)) * (D + 8) + (e % (D / 8)) * 8, R * (D + 8), v[i]);
+    }
+  }
+};
+
+// `rows` rows of W bf16 (W % 8 == 0) in NP pieces, global row pitch gp and piece
+// stride gs, to shared memory (pitch sp, piece stride ss), asynchronously.
+template <int NP>
+__device__ __forceinline__ void stage_rows(bf16* dst, int ss, int sp, const bf16* src, size_t gs,
+                                           int gp, int rows, int W) {
+  const int u = W / 8, n = rows * u;
+  for (int e = threadIdx.x; e < n; e += kThreads) {
+    const int r = e / u, c8 = (e % u) * 8;
+#pragma unroll
+    for (int p = 0; p < NP; ++p) cp16(dst + p * ss + r * sp + c8, src + p * gs + (size_t)r * gp + c8);
+  }
+}
+
+__device__ __forceinline__ void store2(bf16* p, float x, float y) {
+  *reinterpret_cast<uint32_t*>(p) = pack2(x, y);
+}
+__device__ __forceinline__ void store2(float* p, float x, float y) {
+  *reinterpret_cast<float2*>(p) = make_float2(x, y);
+}
+
+// ------------------------------------------------------------------ readout
+// One CTA per frame: g(Q), A = tril(g(Q) g(K)^T) inside each tile, out = (g(Q) S +
+// A V) / (g(Q) z + A 1).  Warp (r, h) has rows 16 r .. 16 r + 15 and the h-th half
+// of every product's columns.  MODE 0: one tile of 48 or 64 rows, its state staged
+// in shared memory.  MODE 1 (two tiles of 32) and 2 (four of 16): every row group
+// has its own tile's state, read straight into MMA fragments; their products
+// sum the k16 steps in A.ks_* interleaved groups, added in order at the end.
+// The next chunk's Omega and state travel while this one's products run, its g(K)
+// while it is projected; FMA and tensor pipe overlap across the two CTAs of an SM.
+template <typename IO, int D, int MODE>
+struct OutSmem {
+  static constexpr int NX = Pieces<IO>::NX, NS = Pieces<IO>::NS, PD = D + 8;
+  static constexpr int xs = kTile * fp_pitch<D>() * 4, om = D * 64 * 4, ph = NS * 64 * kPF * 2,
+                       ps = MODE == 0 ? NS * 64 * PD * 2 : 0, zs = 4 * 64 * 4;
+  static constexpr int bytes = xs + om + 2 * ph + ps + zs + 2 * kTile * 4;
+  static_assert(NX * kTile * PD * 2 <= xs + om, "V in the projections' buffers");
+  static_assert(bytes <= kSmemMax, "shared memory");
+};
+
+template <typename IO, int D, int MODE>
+__global__ void __launch_bounds__(kThreads, D <= 64 ? 2 : 1)
+    k_out(const __grid_constant__ TileArgs A) {
+  using S = OutSmem<IO, D, MODE>;
+  constexpr int NX = S::NX, NS = S::NS, PD = S::PD;
+  constexpr int CW = D >= 32 ? D / 2 : 16, NB = CW / 8;       // columns of a warp
+  constexpr int GN = MODE == 0 ? 1 : MODE == 1 ? 2 : NS == 2 ? 4 : 2;  // most groups: readout
+  constexpr int GA = MODE == 0 ? 1 : MODE == 1 ? 2 : NS == 2 ? 8 : 4;  // scores
+  constexpr int KB = MODE == 0 ? 4 : MODE == 1 ? 2 : 1;       // n8 blocks of a warp's scores
+  constexpr bool ZM = D < 64;                                 // den as an MMA column
+  extern __shared__ uint4 smem_raw[];
+  float* xs = reinterpret_cast<float*>(smem_raw);
+  float* om = xs + S::xs / 4;
+  bf16* Ph = reinterpret_cast<bf16*>(om + S::om / 4);
+  bf16* Kp = Ph + S::ph / 2;
+  bf16* Ps = Kp + S::ph / 2;
+  float* zs = reinterpret_cast<float*>(Ps + S::ps / 2);  // [tile][64]: z rounded to the pieces
+  float* norm2 = zs + 4 * 64;
+  float* den_s = norm2 + kTile;
+  bf16* Vs = reinterpret_cast<bf16*>(xs);
+  pdl_wait();
+  pdl_launch();
+  const int frame = blockIdx.x;
+  const Frame f = frame_pos(A, frame);
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32, g = lane >> 2, t = lane & 3;
+  const int h = warp >> 2, r = warp & 3, r0 = 16 * r;
+  const int ti = MODE == 0 ? 0 : MODE == 1 ? r >> 1 : r;  // this warp's tile of the frame
+  const int ntl = min(A.per, A.nt - f.t0);
+  const size_t MD = (size_t)A.M * D;
+  const float* P0 = A.P + f.c * A.p_chain + f.t0 * A.p_tile;
+  const float* Pt = P0 + min(ti, ntl - 1) * A.p_tile;
+  const bf16* pk = A.phi_k + (size_t)frame * NS * 64 * A.M;
+  const bool square = A.feature == SLIM_FEAT_SQUARE;
+  const int cb = D >= 32 ? CW * h : 0;                    // first column
+  const bool cols = D >= 32 || h == 0;
+  // first key of this warp's scores, and whether any of them is unmasked
+  const int k0 = MODE == 0 ? 32 * h : MODE == 1 ? 32 * ti + 16 * h : r0;
+
+  StateChunk<D, 64> pc;
+  auto stage_keys = [&](int c0) {
+    if (A.causal)
+      stage_rows<NS>(Kp, 64 * kPF, kPF, pk + c0, (size_t)64 * A.M, A.M, 64, min(64, A.M - c0));
+    cp_commit();
+  };
+  auto stage_om = [&](int c0) {
+    if (!square) stage_omega<D, 64>(om, A.om_t, c0);
+    cp_commit();
+  };
+  stage_om(0);
+  stage_keys(0);
+  if (MODE == 0) pc.load(P0, min(64, A.M));
+  load_rows_fp<IO, D>(A, f, static_cast<const IO*>(A.q) + f.row0 * D, xs);
+  __syncthreads();
+  row_norms<D>(xs, norm2);
+  if (MODE == 0) pc.template store<NS>(Ps, min(64, A.M));
+
+  float num[GN][NB][4] = {}, sc[GA][KB][4] = {}, dz[GN][4] = {}, de[GN] = {};
+  // the warps with the fewest scores sum den for d >= 64, a row per lane
+  const int dr = warp == 4 ? lane : warp == 5 ? 32 + lane : -1;
+  const float* zrow = zs + (dr < 0 ? 0 : (MODE == 0 ? 0 : MODE == 1 ? dr / 32 : dr / 16) * 64);
+  for (int c0 = 0; c0 < A.M; c0 += 64) {
+    const int nf = min(64, A.M - c0);
+    cp_wait<1>();
+    __syncthreads();
+    features_to_pieces<D, NS>(A, f, xs, norm2, om, c0, Ph);
+    if (!ZM)
+      for (int e = tid; e < 64 * ntl; e += kThreads)
+        if (e % 64 < nf) zs[e] = round_pieces<NS>(P0[(e / 64) * A.p_tile + MD + c0 + e % 64]);
+    cp_wait<0>();
+    __syncthreads();
+    const bool more = c0 + 64 < A.M;
+    if (more) stage_om(c0 + 64);
+    if (MODE == 0 && more) pc.load(P0 + (size_t)(c0 + 64) * D, min(64, A.M - c0 - 64));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (16 * i >= nf) break;
+      const int step = c0 / 16 + i;
+      const int gn = GN == 1 ? 0 : step & (A.ks_n - 1), ga = GA == 1 ? 0 : step & (A.ks_a - 1);
+      uint32_t a[NS][4];
+      ld_a<NS>(a, Ph, 64 * kPF, kPF, r0, 16 * i);
+      const int m0 = c0 + 16 * i;
+      if (cols) {
+#pragma unroll
+        for (int nb = 0; nb < NB / 2; ++nb) {
+          uint32_t b[NS][4];
+          if (MODE == 0) {
+            ld_bt<NS>(b, Ps, 64 * PD, PD, cb + 16 * nb, 16 * i);
+          } else {
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+              const float* p = Pt + (size_t)(m0 + 2 * t) * D + cb + 16 * nb + 8 * q + g;
+              uint32_t w0[NS], w1[NS];
+              split_pair<NS>(p[0], p[D], w0);
+              split_pair<NS>(p[8 * D], p[9 * D], w1);
+#pragma unroll
+              for (int u = 0; u < NS; ++u) {
+                b[u][2 * q] = w0[u];
+                b[u][2 * q + 1] = w1[u];
+              }
+            }
+          }
+#pragma unroll
+          for (int q = 0; q < GN; ++q)
+            if (GN == 1 || q == gn) mma_pieces<NS, NS>(num[q][2 * nb], num[q][2 * nb + 1], a, b);
+        }
+      }
+      if (ZM && h == 1) {  // the z column
+        uint32_t w0[NS] = {}, w1[NS] = {};
+        if (g == 0) {
+          const float* z = Pt + MD + m0 + 2 * t;
+          split_pair<NS>(z[0], z[1], w0);
+          split_pair<NS>(z[8], z[9], w1);
+        }
+#pragma unroll
+        for (int q = 0; q < GN; ++q)
+          if (GN == 1 || q == gn) {
+#pragma unroll
+            for (int o = NS - 1; o >= 0; --o)
+#pragma unroll
+              for (int x = 0; x <= o; ++x) mma16816(dz[q], a[x], w0[o - x], w1[o - x]);
+          }
+      }
+      if (A.causal) {
+        if (MODE == 2) {
+          uint32_t b[NS][4];
+          ld_b<NS>(b, Kp, 64 * kPF, kPF, r0, 16 * i);
+#pragma unroll
+          for (int q = 0; q < GA; ++q)
+            if (q == ga) {
+#pragma unroll
+              for (int o = NS - 1; o >= 0; --o)
+#pragma unroll
+                for (int x = 0; x <= o; ++x)
+                  mma16816(sc[q][0], a[x], h ? b[o - x][2] : b[o - x][0], h ? b[o - x][3] : b[o - x][1]);
+            }
+        } else {
+#pragma unroll
+          for (int kb = 0; kb < KB / 2; ++kb)
+            if (k0 + 16 * kb <= r0) {  // later keys are masked
+              uint32_t b[NS][4];
+              ld_b<NS>(b, Kp, 64 * kPF, kPF, k0 + 16 * kb, 16 * i);
+#pragma unroll
+              for (int q = 0; q < GA; ++q)
+                if (GA == 1 || q == ga) mma_pieces<NS, NS>(sc[q][2 * kb], sc[q][(2 * kb + 1) % KB], a, b);
+            }
+        }
+      }
+      if (!ZM && dr >= 0) {  // den += g(q) z, feature after feature
+        float e = 0.f;
+#pragma unroll
+        for (int q = 0; q < GN; ++q)
+          if (q == gn) e = de[q];
+#pragma unroll
+        for (int k = 0; k < 16; k += 8) {
+          float x[8];
+          add_pieces8<NS>(Ph + dr * kPF + 16 * i + k, 64 * kPF, x);
+#pragma unroll
+          for (int u = 0; u < 8; ++u) e = fmaf(x[u], zrow[16 * i + k + u], e);
+        }
+#pragma unroll
+        for (int q = 0; q < GN; ++q)
+          if (q == gn) de[q] = e;
+      }
+    }
+    __syncthreads();
+    if (more) {
+      stage_keys(c0 + 64);
+      if (MODE == 0) pc.template store<NS>(Ps, min(64, A.M - c0 - 64));
+    }
+  }
+  // the groups' sums, in order
+#pragma unroll
+  for (int q = 1; q < GN; ++q)
+    if (q < A.ks_n) {
+#pragma unroll
+      for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) num[0][nb][c] += num[q][nb][c];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) dz[0][c] += dz[q][c];
+      de[0] += de[q];
+    }
+  if (A.causal) {
+    // masked scores as pieces (in g(Q)'s place), then A [V | 1]
+#pragma unroll
+    for (int q = 1; q < GA; ++q)
+      if (q < A.ks_a) {
+#pragma unroll
+        for (int kb = 0; kb < KB; ++kb)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) sc[0][kb][c] += sc[q][kb][c];
+      }
+#pragma unroll
+    for (int kb = 0; kb < KB; ++kb)
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        const int row = r0 + g + 8 * hf, key = k0 + (MODE == 2 ? 8 * h : 8 * kb) + 2 * t;
+        uint32_t w[NS];
+        split_pair<NS>(key <= row ? sc[0][kb][2 * hf] : 0.f, key + 1 <= row ? sc[0][kb][2 * hf + 1] : 0.f, w);
+#pragma unroll
+        for (int p = 0; p < NS; ++p)
+          *reinterpret_cast<uint32_t*>(Ph + (p * 64 + row) * kPF + key) = w[p];
+      }
+    load_rows<IO, D>(A, f, static_cast<const IO*>(A.v) + f.row0 * D, Vs, nullptr);
+    __syncthreads();
+    float av[NB][4] = {}, az[4] = {};
+#pragma unroll
+    for (int kb = 0; kb < 4; ++kb)
+      if (kb <= r && (MODE == 0 || kb == r || (MODE == 1 && kb == r - 1 && (r & 1)))) {
+        uint32_t a[NS][4];
+        ld_a<NS>(a, Ph, 64 * kPF, kPF, r0, 16 * kb);
+        if (cols) {
+#pragma unroll
+          for (int nb = 0; nb < NB / 2; ++nb) {
+            uint32_t b[NX][4];
+            ld_bt<NX>(b, Vs, kTile * PD, PD, cb + 16 * nb, 16 * kb);
+            mma_pieces<NS, NX>(av[2 * nb], av[2 * nb + 1], a, b);
+          }
+        }
+        if (ZM && h == 1) {
+          const uint32_t one = g == 0 ? kOnes : 0u;
+          mma_n8<NS>(az, a, one, one);
+        }
+      }
+#pragma unroll
+    for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) num[0][nb][c] = av[nb][c] + num[0][nb][c];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) dz[0][c] = az[c] + dz[0][c];
+    if (!ZM && dr >= 0) {
+      float e = 0.f;
+      const int kf = MODE == 0 ? 0 : dr >> A.shift << A.shift;  // the tile's first key
+      for (int k = kf; k <= dr; k += 8) {
+        float x[8];
+        add_pieces8<NS>(Ph + dr * kPF + k, 64 * kPF, x);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (k + u <= dr) e += x[u];
+      }
+      de[0] = e + de[0];
+    }
+  }
+  if (ZM) {
+    if (h == 1 && t == 0) {
+      den_s[r0 + g] = dz[0][0];
+      den_s[r0 + g + 8] = dz[0][2];
+    }
+  } else if (dr >= 0) {
+    den_s[dr] = de[0];
+  }
+  __syncthreads();
+  if (!cols) return;
+  IO* og = static_cast<IO*>(A.o) + f.row0 * D;
+#pragma unroll
+  for (int hf = 0; hf < 2; ++hf) {
+    const int row = r0 + g + 8 * hf, x = frame_row(A, f, row);
+    const float den = den_s[row];
+    if (x >= 0) {
+#pragma unroll
+      for (int nb = 0; nb < NB; ++nb)
+        store2(og + (size_t)x * D + cb + 8 * nb + 2 * t, den != 0.f ? num[0][nb][2 * hf] / den : 0.f,
+               den != 0.f ? num[0][nb][2 * hf + 1] / den : 0.f);
+    }
+  }
+}
+
+// ------------------------------------------------------------------ backward
+// The row kernels: warp (r, h) has rows 16 r .. 16 r + 15 of the frame and the h-th
+// 16 features of every staged chunk of 32; what the two halves sum over features
+// is added at the end.
+
+// Projections of 16 rows onto 16 staged features (rows f0.. of Om).
+template <typename IO, int D>
+__device__ __forceinline__ void project16(const bf16* Xs, int r0, const bf16* Om, int f0,
+                                          float (&acc)[2][4]) {
+  constexpr int NX = Pieces<IO>::NX, PD = D + 8;
+  float lo[2][4] = {};
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[i][c] = 0.f;
+#pragma unroll
+  for (int ks = 0; ks < D / 16; ++ks) {
+    uint32_t a[NX][4], b[3][4];
+    ld_a<NX>(a, Xs, kTile * PD, PD, r0, 16 * ks);
+    ld_b<3>(b, Om, kChunk * PD, PD, f0, 16 * ks);
+    mma_project<NX, 3>(acc[0], acc[1], lo[0], lo[1], a, b);
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[i][c] += lo[i][c];
+}
+
+// g(X) of a frame in the backward.  FP: from FMA projections (fp32 problems with
+// d <= 32, where they are the more exact and cheap); otherwise from MMAs.
+template <typename IO, int D>
+struct RowFeatures {
+  static constexpr int NX = Pieces<IO>::NX, PD = D + 8;
+  static constexpr bool FP = NX == 3 && D <= 32;
+  static constexpr int kPitch = kChunk + 4;
+  // shared memory of the FMA projections: rows, two chunks of Omega, a chunk of g(X)
+  static constexpr int xs = FP ? kTile * fp_pitch<D>() : 0, omf = FP ? D * kChunk : 0,
+                       ph = FP ? kTile * kPitch : 0, floats = xs + 2 * omf + ph;
+
+  // this warp's 16 rows at features fg .. fg + 15 (fl: the same features' offset in
+  // the chunk); x0, x1: caller rows of this thread's rows (-1: padding, g = 0)
+  static __device__ __forceinline__ void get(const TileArgs& A, const IO* xg, const bf16* Xs,
+                                             const float* hx, const bf16* Om, const float* phs, int r0,
+                                             int fl, int fg, int x0, int x1, float (&phi)[2][4]) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    if (FP) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          const float2 v = *reinterpret_cast<const float2*>(
+              phs + (r0 + g + 8 * hf) * kPitch + fl + 8 * i + 2 * t);
+          phi[i][2 * hf] = v.x;
+          phi[i][2 * hf + 1] = v.y;
+        }
+      return;
+    }
+    if (A.feature == SLIM_FEAT_SQUARE) {
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const float x = staged<NX>(
+              Xs + (r0 + g + 8 * (c >> 1)) * PD + fg + 8 * i + 2 * t + (c & 1), kTile * PD);
+          phi[i][c] = x * x;
+        }
+      return;
+    }
+    project16<IO, D>(Xs, r0, Om, fl, phi);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int r = r0 + g + 8 * (c >> 1), f = fg + 8 * i + 2 * t + (c & 1), x = c >> 1 ? x1 : x0;
+        phi[i][c] = x >= 0 ? feature_value<IO>(A, phi[i][c], hx[r], f, xg + (size_t)x * D, D) : 0.f;
+      }
+  }
+};
+
+// dOmega partials: CTA i of a backward launch adds the products of its tiles, in
+// the order it takes them, onto partial i.  Partials hold the accumulators as the
+// lanes do: 16 features x 16 columns are 2 x 32 float4 (slot_at), so that a warp
+// moves 512 contiguous bytes; k_domega puts them back in order.
+__device__ __forceinline__ size_t slot_at(int mb, int kd, int n16, int n8) {
+  return ((size_t)((mb * kd + n16) * 2 + n8) * 32 + (threadIdx.x & 31)) * 4;
+}
+__device__ __forceinline__ void slot_put(float* p, const float (&v)[4], bool first) {
+  if (first)
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  else
+    asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v[0]),
+                 "f"(v[1]), "f"(v[2]), "f"(v[3])
+                 : "memory");
+}
+// the pieces of a 16 x 16 block (as an A fragment) to rows r0.. of a row-major
+// tile, columns col0..
+template <int NP>
+__device__ __forceinline__ void put_block(bf16* dst, size_t ps, int pitch, int r0, int col0,
+                                          const uint32_t (&a)[NP][4]) {
+  const int lane = threadIdx.x & 31;
+  dst += (size_t)(r0 + (lane >> 2)) * pitch + col0 + 2 * (lane & 3);
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    bf16* d = dst + p * ps;
+    *reinterpret_cast<uint32_t*>(d) = a[p][0];
+    *reinterpret_cast<uint32_t*>(d + (size_t)8 * pitch) = a[p][1];
+    *reinterpret_cast<uint32_t*>(d + 8) = a[p][2];
+    *reinterpret_cast<uint32_t*>(d + (size_t)8 * pitch + 8) = a[p][3];
+  }
+}
+// u = dg (.) g'(x) of 16 rows x 16 features from dg and g (exp: g' = g; ReLU: 0 or
+// 1 / sqrt(M)), in place
+__device__ __forceinline__ void feature_vjp(const TileArgs& A, float (&dphi)[2][4],
+                                            const float (&phi)[2][4]) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      dphi[i][c] = A.feature == SLIM_FEAT_EXP ? dphi[i][c] * phi[i][c]
+                                              : (phi[i][c] > 0.f ? dphi[i][c] * A.inv_sqrt_m : 0.f);
+}
+// quadratic map: dX = 2 x (.) dg, straight to the caller's rows
+template <typename IO, int D>
+__device__ __forceinline__ void store_square_vjp(IO* dst, const bf16* Xs, int r0, int fg, int x0,
+                                                 int x1, const float (&dphi)[2][4]) {
+  constexpr int NX = Pieces<IO>::NX, PD = D + 8;
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+      const int row = hf ? x1 : x0, col = fg + 8 * i + 2 * t;
+      const bf16* x = Xs + (r0 + g + 8 * hf) * PD + col;
+      if (row >= 0)
+        store2(dst + (size_t)row * D + col, 2.f * staged<NX>(x, kTile * PD) * dphi[i][2 * hf],
+               2.f * staged<NX>(x + 1, kTile * PD) * dphi[i][2 * hf + 1]);
+    }
+}
+// dX = u Omega (- x sum u for the exponential map) of 16 rows, columns in D / 8 n8 blocks
+template <typename IO, int D>
+__device__ __forceinline__ void store_dx(const TileArgs& A, IO* dst, const bf16* Xs, int r0, int x0,
+                                         int x1, const float (&dx)[D / 8][4], float us0, float us1) {
+  constexpr int NX = Pieces<IO>::NX, PD = D + 8;
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const bool ex = A.feature == SLIM_FEAT_EXP;
+#pragma unroll
+  for (int hf = 0; hf < 2; ++hf) {
+    const int row = hf ? x1 : x0;
+    const float us = hf ? us1 : us0;
+    if (row >= 0) {
+#pragma unroll
+      for (int i = 0; i < D / 8; ++i) {
+        float x = dx[i][2 * hf], y = dx[i][2 * hf + 1];
+        if (ex) {
+          const bf16* xs = Xs + (r0 + g + 8 * hf) * PD + 8 * i + 2 * t;
+          x -= staged<NX>(xs, kTile * PD) * us;
+          y -= staged<NX>(xs + 1, kTile * PD) * us;
+        }
+        store2(dst + (size_t)row * D + 8 * i + 2 * t, x, y);
+      }
+    }
+  }
+}
+
+// CTAs that fit an SM by shared memory (228 KB, 1 KB of it per CTA)
+constexpr int ctas_per_sm(int bytes) { return 2 * (bytes + 1024) <= 233472 ? 2 : 1; }
+
+constexpr int kPT = kChunk + 8;  // row pitch of the 64 x 32 chunk tiles
+
+template <typename IO, int D>
+struct BwdQSmem {
+  static constexpr int NX = Pieces<IO>::NX, NS = Pieces<IO>::NS, PD = D + 8, PK = kTile + 8;
+  static constexpr int X = NX * kTile * PD, W = NS * kTile * PD, OM = 3 * kChunk * PD,
+                       PP = NS * kChunk * PD, KT = NS * kTile * kPT, R = OM + PP + KT,
+                       TQ = NS * kTile * kPT, DA = NS * kTile * PK;
+  static constexpr bool V_OWN = NX == 1;  // V has its own place, or takes the chunk's
+  static constexpr int bytes = (X + W + R + 2 * TQ + DA + (V_OWN ? X : 0)) * 2 + 4 * kTile * 4 + 4 * kChunk * 4 +
+                               RowFeatures<IO, D>::floats * 4;
+  static_assert(V_OWN || X <= R, "V in the chunk buffers");
+  static_assert(OM + KT <= 2 * TQ + DA, "second chunk buffer");
+  static_assert(128 * 34 * 4 <= 2 * TQ * 2, "score sums");
+  static_assert(128 * (D / 2 + 2) * 4 <= R * 2, "dq sums");
+  static_assert(bytes <= kSmemMax, "shared memory");
+};
+template <typename IO, int D>
+struct BwdKSmem {
+  static constexpr int NX = Pieces<IO>::NX, NS = Pieces<IO>::NS, PD = D + 8, PK = kTile + 8;
+  static constexpr int X = NX * kTile * PD, OM = 3 * kChunk * PD, GG = NS * kChunk * PD,
+                       TQ = NS * kTile * kPT, DA = NS * kTile * PK, W = NS * kTile * PD,
+                       R = OM + GG + 2 * TQ + DA;
+  static constexpr int bytes = (2 * X + R) * 2 + kTile * 4 + RowFeatures<IO, D>::floats * 4;
+  static_assert(DA + W <= R, "A and dnum in the chunk buffers");
+  static_assert(128 * (D + 2) * 4 <= R * 2, "dk, dv sums");
+  static_assert(bytes <= kSmemMax, "shared memory");
+};
+template <typename IO, int D>
+constexpr int bwd_occupancy() {
+  return ctas_per_sm(BwdQSmem<IO, D>::bytes) == 2 && ctas_per_sm(BwdKSmem<IO, D>::bytes) == 2 ? 2 : 1;
+}
+
+// Query side of a tile, from its state P_t:
+//   den = g(Q) z + A 1, dnum = dout / den, dden = -<dout, out> / den,
+//   dA = tril(dnum V^T + dden), dg(Q) = dnum S^T + dden z + dA g(K),
+//   Gd = g(Q)^T [dnum | dden], u = dg(Q) (.) g'(q), dq = u Omega - q sum u, dOmega += u^T q.
+// Two passes over the features: the first sums the denominators and A, which the
+// second needs.  g(Q), A, dA and dnum are left (as pieces) for the key side.
+template <typename IO, int D>
+__global__ void __launch_bounds__(kThreads, (bwd_occupancy<IO, D>()))
+    k_bwd_q(const __grid_constant__ TileArgs A) {
+  using S = BwdQSmem<IO, D>;
+  constexpr int NX = S::NX, NS = S::NS, PD = S::PD, PK = S::PK, KD = D / 16;
+  extern __shared__ uint4 smem_raw[];
+  bf16* Xs = reinterpret_cast<bf16*>(smem_raw);
+  bf16* Ws = Xs + S::X;
+  bf16* Om = Ws + S::W;
+  bf16* Ps = Om + S::OM;
+  bf16* Kt = Ps + S::PP;
+  bf16* Tq = Kt + S::KT;
+  bf16* Tu = Tq + S::TQ;
+  bf16* dAs = Tu + S::TQ;
+  bf16* Vs = S::V_OWN ? dAs + S::DA : Om;
+  float* hx = reinterpret_cast<float*>(dAs + S::DA + (S::V_OWN ? S::X : 0));
+  float* rd = hx + kTile;   // <dout, out>, then dden
+  float* dn = rd + kTile;   // den
+  float* gzs = dn + 2 * kTile;  // [4][kChunk]
+  using F = RowFeatures<IO, D>;
+  float* xf = gzs + 4 * kChunk;  // FMA projections
+  float* omf = xf + F::xs;
+  float* phs = omf + 2 * F::omf;
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32, g = lane >> 2, t = lane & 3;
+  const int h = warp >> 2, rb = warp & 3, r0 = 16 * rb, fl = 16 * h;
+  const bool square = A.feature == SLIM_FEAT_SQUARE;
+  const size_t MD = (size_t)A.M * D;
+  float* slot = A.slots + (size_t)blockIdx.x * MD;
+  pdl_wait();
+  pdl_launch();
+
+  for (int tile = blockIdx.x; tile < A.chains * A.nf; tile += gridDim.x) {
+    const Frame tp = frame_pos(A, tile);
+    const bool first = tile == (int)blockIdx.x;
+    const int x0 = frame_row(A, tp, r0 + g), x1 = frame_row(A, tp, r0 + g + 8);
+    const IO* qg = static_cast<const IO*>(A.q) + tp.row0 * D;
+    const IO* vg = static_cast<const IO*>(A.v) + tp.row0 * D;
+    const IO* dog = static_cast<const IO*>(A.dout) + tp.row0 * D;
+    const IO* og = static_cast<const IO*>(A.out) + tp.row0 * D;
+    const float* Pt = A.P + tp.c * A.p_chain + tp.t0 * A.p_tile;
+    const bf16* kt = A.phi_k + (size_t)tile * NS * A.M * kTile;
+    bf16* pq = A.phi_q + (size_t)tile * NS * A.M * kTile;
+    bf16* sA = A.sA + (size_t)tile * NS * kTile * kTile;
+    bf16* sdA = A.sdA + (size_t)tile * NS * kTile * kTile;
+    bf16* sW = A.sW + (size_t)tile * NS * kTile * D;
+    float* gd = A.gdelta + (size_t)tile * A.E;
+
+    auto stage = [&](int c0, bf16* om, bf16* ktp, float* of) {
+      const int nf = min(kChunk, A.M - c0);
+      if (!square)
+        stage_rows<3>(om, kChunk * PD, PD, A.om_row + (size_t)c0 * D, MD, D, nf, D);
+      if (A.causal)
+        stage_rows<NS>(ktp, kTile * kPT, kPT, kt + c0, (size_t)A.M * kTile, A.M, kTile, nf);
+      if (F::FP && !square) stage_omega<D, kChunk>(of, A.om_t, c0);
+      cp_commit();
+    };
+    // g(Q) of a chunk by FMAs (ends with a barrier)
+    auto project_fp = [&](int c0, const float* of) {
+      features_fp<D, kChunk>(A, tp, xf, dn + kTile, of, c0,
+                             [&](int r, int fo, const float(&v)[2]) {
+                               *reinterpret_cast<float2*>(phs + r * F::kPitch + fo) = make_float2(v[0], v[1]);
+                             });
+      __syncthreads();
+    };
+    // pass 1's chunks alternate between the chunk buffers and the T | dA space
+    bf16* om2 = Tq;
+    bf16* kt2 = Tq + S::OM;
+    stage(0, Om, Kt, omf);
+    load_rows<IO, D>(A, tp, qg, Xs, hx);
+    if (F::FP) load_rows_fp<IO, D>(A, tp, qg, xf);
+    if (S::V_OWN) load_rows<IO, D>(A, tp, vg, Vs, nullptr);
+    for (int e = tid; e < kTile * (D / 8); e += kThreads) {
+      const int r = e / (D / 8), c8 = (e % (D / 8)) * 8;
+      const int x = frame_row(A, tp, r);
+      float s = 0.f;
+      if (x >= 0) {
+        float a[8], b[8];
+        load8(dog + (size_t)x * D + c8, a);
+        load8(og + (size_t)x * D + c8, b);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) s = fmaf(a[i], b[i], s);
+      }
+#pragma unroll
+      for (int o = 1; o < D / 8; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (c8 == 0) rd[r] = s;
+    }
+    cp_wait<0>();
+    __syncthreads();
+    if (F::FP) {
+      row_norms<D>(xf, dn + kTile);
+      __syncthreads();
+    }
+
+    // pass 1: g(Q), A, den
+    float den0 = 0.f, den1 = 0.f;
+    {
+      float sc[8][4] = {};
+      int cur = 0;
+      for (int c0 = 0; c0 < A.M; c0 += kChunk) {
+        if (c0 + kChunk < A.M) stage(c0 + kChunk, cur ? Om : om2, cur ? Kt : kt2, cur ? omf : omf + F::omf);
+        const bf16* om = cur ? om2 : Om;
+        const bf16* ktp = cur ? kt2 : Kt;
+        if (F::FP) project_fp(c0, cur ? omf + F::omf : omf);
+        const int fg = c0 + fl;
+        if (fg < A.M) {
+          float phi[2][4];
+          F::get(A, qg, Xs, hx, om, phs, r0, fl, fg, x0, x1, phi);
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const float2 z = *reinterpret_cast<const float2*>(Pt + MD + fg + 8 * i + 2 * t);
+            den0 = fmaf(phi[i][0], z.x, fmaf(phi[i][1], z.y, den0));
+            den1 = fmaf(phi[i][2], z.x, fmaf(phi[i][3], z.y, den1));
+          }
+          if (A.causal) {
+            uint32_t a[NS][4];
+            acc_to_a<NS>(a, phi[0], phi[1]);
+            put_block<NS>(pq, (size_t)kTile * A.M, A.M, r0, fg, a);
+#pragma unroll
+            for (int kb = 0; kb < 4; ++kb)
+              if (kb <= rb) {
+                uint32_t b[NS][4];
+                ld_b<NS>(b, ktp, kTile * kPT, kPT, 16 * kb, fl);
+                mma_sum<NS, NS>(sc[2 * kb], sc[2 * kb + 1], a, b);
+              }
+          }
+        }
+        cp_wait<0>();
+        __syncthreads();
+        cur ^= 1;
+      }
+      den0 = quad_sum(den0);
+      den1 = quad_sum(den1);
+      float* red = reinterpret_cast<float*>(Tq) + (tid & 127);
+      if (h == 1) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) red[(4 * i + c) * 128] = sc[i][c];
+        red[32 * 128] = den0;
+        red[33 * 128] = den1;
+      }
+      __syncthreads();
+      if (S::V_OWN) {  // the chunk buffers are free: pass 2's first chunk
+        stage(0, Om, Kt, omf);
+      } else {
+        load_rows<IO, D>(A, tp, vg, Vs, nullptr);
+      }
+      if (h == 0) {
+        den0 += red[32 * 128];
+        den1 += red[33 * 128];
+        if (A.causal) {
+          float a0 = 0.f, a1 = 0.f;
+#pragma unroll
+          for (int kb = 0; kb < 4; ++kb)
+            if (kb <= rb) {
+#pragma unroll
+              for (int i = 2 * kb; i < 2 * kb + 2; ++i)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                  const int row = r0 + g + 8 * (c >> 1), key = 8 * i + 2 * t + (c & 1);
+                  const float v = sc[i][c] + red[(4 * i + c) * 128];
+                  sc[i][c] = key <= row ? v : 0.f;
+                }
+              a0 += sc[2 * kb][0] + sc[2 * kb][1] + sc[2 * kb + 1][0] + sc[2 * kb + 1][1];
+              a1 += sc[2 * kb][2] + sc[2 * kb][3] + sc[2 * kb + 1][2] + sc[2 * kb + 1][3];
+              uint32_t a[NS][4];
+              acc_to_a<NS>(a, sc[2 * kb], sc[2 * kb + 1]);
+              put_block<NS>(sA, kTile * kTile, kTile, r0, 16 * kb, a);
+            }
+          den0 += quad_sum(a0);
+          den1 += quad_sum(a1);
+        }
+        if (t == 0) {
+          dn[r0 + g] = den0;
+          dn[r0 + g + 8] = den1;
+        }
+      }
+    }
+    __syncthreads();
+
+    // W = dnum (pieces), dden
+    for (int e = tid; e < kTile * (D / 8); e += kThreads) {
+      const int r = e / (D / 8), c8 = (e % (D / 8)) * 8;
+      const int x = frame_row(A, tp, r);
+      const float den = dn[r];
+      float v[8] = {};
+      if (x >= 0 && den != 0.f) {
+        load8(dog + (size_t)x * D + c8, v);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = v[i] / den;
+      }
+      store_pieces8<NS>(Ws + r * PD + c8, kTile * PD, v);
+      if (A.causal) store_pieces8<NS>(sW + r * D + c8, kTile * D, v);
+    }
+    if (tid < kTile) {
+      const float den = dn[tid];
+      rd[tid] = frame_row(A, tp, tid) >= 0 && den != 0.f ? -rd[tid] / den : 0.f;
+    }
+    __syncthreads();
+    const float dd0 = rd[r0 + g], dd1 = rd[r0 + g + 8];
+
+    if (A.causal) {  // dA, a half's warp taking every other block of 16 keys
+#pragma unroll
+      for (int kb = 0; kb < 4; ++kb)
+        if (kb <= rb && (kb & 1) == h) {
+          float d[2][4] = {};
+#pragma unroll
+          for (int ks = 0; ks < KD; ++ks) {
+            uint32_t a[NS][4], b[NX][4];
+            ld_a<NS>(a, Ws, kTile * PD, PD, r0, 16 * ks);
+            ld_b<NX>(b, Vs, kTile * PD, PD, 16 * kb, 16 * ks);
+            mma_sum<NS, NX>(d[0], d[1], a, b);
+          }
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              const int row = r0 + g + 8 * (c >> 1), key = 16 * kb + 8 * i + 2 * t + (c & 1);
+              d[i][c] = key <= row ? d[i][c] + (c >> 1 ? dd1 : dd0) : 0.f;
+            }
+          uint32_t a[NS][4];
+          acc_to_a<NS>(a, d[0], d[1]);
+          put_block<NS>(dAs, kTile * PK, PK, r0, 16 * kb, a);
+          put_block<NS>(sdA, kTile * kTile, kTile, r0, 16 * kb, a);
+        }
+    }
+    StateChunk<D, kChunk> pc;
+    if (!S::V_OWN) {
+      __syncthreads();  // V read: the chunk buffers are free
+      stage(0, Om, Kt, omf);
+    }
+    pc.load(Pt, min(kChunk, A.M));
+    pc.template store<NS>(Ps, min(kChunk, A.M));
+    cp_wait<0>();
+    __syncthreads();
+
+    // pass 2
+    float dq[D / 8][4] = {}, us0 = 0.f, us1 = 0.f;
+    for (int c0 = 0; c0 < A.M; c0 += kChunk) {
+      const int fg = c0 + fl;
+      if (F::FP) project_fp(c0, omf);
+      if (fg < A.M) {
+        float phi[2][4], dp[2][4] = {};
+        F::get(A, qg, Xs, hx, Om, phs, r0, fl, fg, x0, x1, phi);
+#pragma unroll
+        for (int ks = 0; ks < KD; ++ks) {
+          uint32_t a[NS][4], b[NS][4];
+          ld_a<NS>(a, Ws, kTile * PD, PD, r0, 16 * ks);
+          ld_b<NS>(b, Ps, kChunk * PD, PD, fl, 16 * ks);
+          mma_sum<NS, NS>(dp[0], dp[1], a, b);
+        }
+        if (A.causal) {
+#pragma unroll
+          for (int kb = 0; kb < 4; ++kb)
+            if (kb <= rb) {
+              uint32_t a[NS][4], b[NS][4];
+              ld_a<NS>(a, dAs, kTile * PK, PK, r0, 16 * kb);
+              ld_bt<NS>(b, Kt, kTile * kPT, kPT, fl, 16 * kb);
+              mma_sum<NS, NS>(dp[0], dp[1], a, b);
+            }
+        }
+        uint32_t a[NS][4];
+        acc_to_a<NS>(a, phi[0], phi[1]);
+        put_block<NS>(Tq, kTile * kPT, kPT, r0, fl, a);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const float2 z = *reinterpret_cast<const float2*>(Pt + MD + fg + 8 * i + 2 * t);
+          dp[i][0] = fmaf(dd0, z.x, dp[i][0]);
+          dp[i][1] = fmaf(dd0, z.y, dp[i][1]);
+          dp[i][2] = fmaf(dd1, z.x, dp[i][2]);
+          dp[i][3] = fmaf(dd1, z.y, dp[i][3]);
+          // g_z's share: sum over this warp's rows of g(Q) dden
+          float s0 = fmaf(phi[i][0], dd0, phi[i][2] * dd1), s1 = fmaf(phi[i][1], dd0, phi[i][3] * dd1);
+#pragma unroll
+          for (int o = 4; o < 32; o <<= 1) {
+            s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+          }
+          if (g == 0) {
+            gzs[rb * kChunk + fl + 8 * i + 2 * t] = s0;
+            gzs[rb * kChunk + fl + 8 * i + 2 * t + 1] = s1;
+          }
+        }
+        if (square) {
+          store_square_vjp<IO, D>(static_cast<IO*>(A.dq) + tp.row0 * D, Xs, r0, fg, x0, x1, dp);
+        } else {
+          feature_vjp(A, dp, phi);
+          us0 += dp[0][0] + dp[0][1] + dp[1][0] + dp[1][1];
+          us1 += dp[0][2] + dp[0][3] + dp[1][2] + dp[1][3];
+          acc_to_a<NS>(a, dp[0], dp[1]);
+          put_block<NS>(Tu, kTile * kPT, kPT, r0, fl, a);
+#pragma unroll
+          for (int nb = 0; nb < KD; ++nb) {
+            uint32_t b[NS][4];
+            ld_bt<NS>(b, Om, kChunk * PD, PD, 16 * nb, fl);
+            mma_sum<NS, NS>(dq[2 * nb], dq[2 * nb + 1], a, b);
+          }
+        }
+      }
+      __syncthreads();
+      const bool more = c0 + kChunk < A.M;
+      if (more) {
+        stage(c0 + kChunk, Om, Kt, omf);
+        pc.load(Pt + (size_t)(c0 + kChunk) * D, min(kChunk, A.M - c0 - kChunk));
+      }
+      // warps 0-3: Gd = g(Q)^T dnum; warps 4-7: dOmega += u^T q; each 16 features x
+      // half of the columns (all of them for d = 16)
+      const int mb = (warp >> 1) & 1, ng = warp & 1;
+      constexpr int NU = KD >= 2 ? KD / 2 : 1;
+      if (c0 + 16 * mb < A.M && (KD >= 2 || ng == 0) && (h == 0 || !square)) {
+        float o[2 * NU][4] = {};
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) {
+          uint32_t a[NS][4];
+          ld_at<NS>(a, h ? Tu : Tq, kTile * kPT, kPT, 16 * mb, 16 * ks);
+#pragma unroll
+          for (int nu = 0; nu < NU; ++nu) {
+            const int n0 = 16 * (ng * NU + nu);
+            if (h == 0) {
+              uint32_t b[NS][4];
+              ld_bt<NS>(b, Ws, kTile * PD, PD, n0, 16 * ks);
+              mma_sum<NS, NS>(o[2 * nu], o[2 * nu + 1], a, b);
+            } else {
+              uint32_t b[NX][4];
+              ld_bt<NX>(b, Xs, kTile * PD, PD, n0, 16 * ks);
+              mma_sum<NS, NX>(o[2 * nu], o[2 * nu + 1], a, b);
+            }
+          }
+        }
+#pragma unroll
+        for (int nu = 0; nu < NU; ++nu)
+#pragma unroll
+          for (int n8 = 0; n8 < 2; ++n8) {
+            const float(&v)[4] = o[2 * nu + n8];
+            if (h == 0) {
+              float* dst = gd + (size_t)(c0 + 16 * mb + g) * D + 16 * (ng * NU + nu) + 8 * n8 + 2 * t;
+              *reinterpret_cast<float2*>(dst) = make_float2(v[0], v[1]);
+              *reinterpret_cast<float2*>(dst + 8 * D) = make_float2(v[2], v[3]);
+            } else {
+              slot_put(slot + slot_at(c0 / 16 + mb, KD, ng * NU + nu, n8), v, first);
+            }
+          }
+      }
+      if (tid < kChunk && c0 + tid < A.M)
+        gd[MD + c0 + tid] = (gzs[tid] + gzs[kChunk + tid]) + (gzs[2 * kChunk + tid] + gzs[3 * kChunk + tid]);
+      if (more) pc.template store<NS>(Ps, min(kChunk, A.M - c0 - kChunk));
+      cp_wait<0>();
+      __syncthreads();
+    }
+    if (!square) {
+      us0 = quad_sum(us0);
+      us1 = quad_sum(us1);
+      float* red = reinterpret_cast<float*>(Om) + (tid & 127);
+      if (h == 1) {
+#pragma unroll
+        for (int i = 0; i < D / 8; ++i)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) red[(4 * i + c) * 128] = dq[i][c];
+        red[(D / 2) * 128] = us0;
+        red[(D / 2 + 1) * 128] = us1;
+      }
+      __syncthreads();
+      if (h == 0) {
+#pragma unroll
+        for (int i = 0; i < D / 8; ++i)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) dq[i][c] += red[(4 * i + c) * 128];
+        store_dx<IO, D>(A, static_cast<IO*>(A.dq) + tp.row0 * D, Xs, r0, x0, x1, dq,
+                        us0 + red[(D / 2) * 128], us1 + red[(D / 2 + 1) * 128]);
+      }
+    }
+    __syncthreads();  // before the next tile's loads
+  }
+}
+
+// Key / value side of a tile, from its state gradient G_t and the query side's
+// g(Q), A, dA and dnum:
+//   dg(K) = V G_S^T + g_z + dA^T g(Q), dV = g(K) G_S + A^T dnum,
+//   u = dg(K) (.) g'(k), dk = u Omega - k sum u, dOmega += u^T k.
+template <typename IO, int D>
+__global__ void __launch_bounds__(kThreads, (bwd_occupancy<IO, D>()))
+    k_bwd_k(const __grid_constant__ TileArgs A) {
+  using S = BwdKSmem<IO, D>;
+  constexpr int NX = S::NX, NS = S::NS, PD = S::PD, PK = S::PK, KD = D / 16;
+  extern __shared__ uint4 smem_raw[];
+  bf16* Ks = reinterpret_cast<bf16*>(smem_raw);
+  bf16* Vs = Ks + S::X;
+  bf16* Om = Vs + S::X;
+  bf16* Gs = Om + S::OM;
+  bf16* Qs = Gs + S::GG;
+  bf16* Tu = Qs + S::TQ;
+  bf16* dAs = Tu + S::TQ;
+  float* hx = reinterpret_cast<float*>(dAs + S::DA);
+  using F = RowFeatures<IO, D>;
+  float* xf = hx + kTile;  // FMA projections (one chunk of Omega; the other's space holds |x|^2)
+  float* omf = xf + F::xs;
+  float* norm2 = omf + F::omf;
+  float* phs = omf + 2 * F::omf;
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32, g = lane >> 2, t = lane & 3;
+  const int h = warp >> 2, rb = warp & 3, r0 = 16 * rb, fl = 16 * h;
+  const bool square = A.feature == SLIM_FEAT_SQUARE;
+  const size_t MD = (size_t)A.M * D;
+  float* slot = A.slots + (size_t)blockIdx.x * MD;
+  pdl_wait();
+  pdl_launch();
+
+  for (int tile = blockIdx.x; tile < A.chains * A.nf; tile += gridDim.x) {
+    const Frame tp = frame_pos(A, tile);
+    const int x0 = frame_row(A, tp, r0 + g), x1 = frame_row(A, tp, r0 + g + 8);
+    const IO* kg = static_cast<const IO*>(A.k) + tp.row0 * D;
+    const float* Gt = A.G + tp.c * A.g_chain + tp.t0 / A.per * A.g_tile;
+    const bf16* pq = A.phi_q + (size_t)tile * NS * A.M * kTile;
+    const bf16* sA = A.sA + (size_t)tile * NS * kTile * kTile;
+    const bf16* sdA = A.sdA + (size_t)tile * NS * kTile * kTile;
+    const bf16* sW = A.sW + (size_t)tile * NS * kTile * D;
+
+    StateChunk<D, kChunk> gc;
+    auto stage = [&](int c0) {
+      const int nf = min(kChunk, A.M - c0);
+      if (!square)
+        stage_rows<3>(Om, kChunk * PD, PD, A.om_row + (size_t)c0 * D, MD, D, nf, D);
+      if (A.causal)
+        stage_rows<NS>(Qs, kTile * kPT, kPT, pq + c0, (size_t)kTile * A.M, A.M, kTile, nf);
+      if (F::FP && !square) stage_omega<D, kChunk>(omf, A.om_t, c0);
+      cp_commit();
+      gc.load(Gt + (size_t)c0 * D, nf);
+    };
+    if (A.causal) stage_rows<NS>(dAs, kTile * PK, PK, sdA, kTile * kTile, kTile, kTile, kTile);
+    stage(0);
+    load_rows<IO, D>(A, tp, kg, Ks, hx);
+    if (F::FP) load_rows_fp<IO, D>(A, tp, kg, xf);
+    load_rows<IO, D>(A, tp, static_cast<const IO*>(A.v) + tp.row0 * D, Vs, nullptr);
+    gc.template store<NS>(Gs, min(kChunk, A.M));
+    cp_wait<0>();
+    __syncthreads();
+    if (F::FP) {
+      row_norms<D>(xf, norm2);
+      __syncthreads();
+    }
+
+    float dk[D / 8][4] = {}, dv[D / 8][4] = {}, us0 = 0.f, us1 = 0.f;
+    for (int c0 = 0; c0 < A.M; c0 += kChunk) {
+      const int fg = c0 + fl;
+      if (F::FP) {
+        features_fp<D, kChunk>(A, tp, xf, norm2, omf, c0, [&](int r, int fo, const float(&v)[2]) {
+          *reinterpret_cast<float2*>(phs + r * F::kPitch + fo) = make_float2(v[0], v[1]);
+        });
+        __syncthreads();
+      }
+      if (fg < A.M) {
+        float phi[2][4], dp[2][4] = {};
+        F::get(A, kg, Ks, hx, Om, phs, r0, fl, fg, x0, x1, phi);
+#pragma unroll
+        for (int ks = 0; ks < KD; ++ks) {
+          uint32_t a[NX][4], b[NS][4];
+          ld_a<NX>(a, Vs, kTile * PD, PD, r0, 16 * ks);
+          ld_b<NS>(b, Gs, kChunk * PD, PD, fl, 16 * ks);
+          mma_sum<NX, NS>(dp[0], dp[1], a, b);
+        }
+        if (A.causal) {
+#pragma unroll
+          for (int kb = 0; kb < 4; ++kb)
+            if (kb >= rb) {  // rows before these keys do not read them
+              uint32_t a[NS][4], b[NS][4];
+              ld_at<NS>(a, dAs, kTile * PK, PK, r0, 16 * kb);
+              ld_bt<NS>(b, Qs, kTile * kPT, kPT, fl, 16 * kb);
+              mma_sum<NS, NS>(dp[0], dp[1], a, b);
+            }
+        }
+        uint32_t a[NS][4];
+        acc_to_a<NS>(a, phi[0], phi[1]);
+#pragma unroll
+        for (int nb = 0; nb < KD; ++nb) {
+          uint32_t b[NS][4];
+          ld_bt<NS>(b, Gs, kChunk * PD, PD, 16 * nb, fl);
+          mma_sum<NS, NS>(dv[2 * nb], dv[2 * nb + 1], a, b);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const float2 z = *reinterpret_cast<const float2*>(Gt + MD + fg + 8 * i + 2 * t);
+          dp[i][0] += z.x;
+          dp[i][1] += z.y;
+          dp[i][2] += z.x;
+          dp[i][3] += z.y;
+        }
+        if (square) {
+          store_square_vjp<IO, D>(static_cast<IO*>(A.dk) + tp.row0 * D, Ks, r0, fg, x0, x1, dp);
+        } else {
+          feature_vjp(A, dp, phi);
+          us0 += dp[0][0] + dp[0][1] + dp[1][0] + dp[1][1];
+          us1 += dp[0][2] + dp[0][3] + dp[1][2] + dp[1][3];
+          acc_to_a<NS>(a, dp[0], dp[1]);
+          put_block<NS>(Tu, kTile * kPT, kPT, r0, fl, a);
+#pragma unroll
+          for (int nb = 0; nb < KD; ++nb) {
+            uint32_t b[NS][4];
+            ld_bt<NS>(b, Om, kChunk * PD, PD, 16 * nb, fl);
+            mma_sum<NS, NS>(dk[2 * nb], dk[2 * nb + 1], a, b);
+          }
+        }
+      }
+      __syncthreads();
+      const bool more = c0 + kChunk < A.M;
+      if (more) stage(c0 + kChunk);
+      if (!square) {
+        for (int u = warp; u < 2 * KD; u += kThreads / 32) {  // 16 features x 16 columns
+          const int mb = u & 1, n16 = u >> 1;
+          if (c0 + 16 * mb < A.M) {
+            float o[2][4] = {};
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks) {
+              uint32_t a[NS][4], b[NX][4];
+              ld_at<NS>(a, Tu, kTile * kPT, kPT, 16 * mb, 16 * ks);
+              ld_bt<NX>(b, Ks, kTile * PD, PD, 16 * n16, 16 * ks);
+              mma_sum<NS, NX>(o[0], o[1], a, b);
+            }
+#pragma unroll
+            for (int n8 = 0; n8 < 2; ++n8)
+              slot_put(slot + slot_at(c0 / 16 + mb, KD, n16, n8), o[n8],
+                       A.slots_new && tile == (int)blockIdx.x);
+          }
+        }
+      }
+      if (more) gc.template store<NS>(Gs, min(kChunk, A.M - c0 - kChunk));
+      cp_wait<0>();
+      __syncthreads();
+    }
+    if (A.causal) {  // dV += A^T dnum, a half's warps taking every other block of 16 rows
+      bf16* As = Om;
+      bf16* Ws = Om + S::DA;
+      stage_rows<NS>(As, kTile * PK, PK, sA, kTile * kTile, kTile, kTile, kTile);
+      stage_rows<NS>(Ws, kTile * PD, PD, sW, kTile * D, D, kTile, D);
+      cp_commit();
+      cp_wait<0>();
+      __syncthreads();
+#pragma unroll
+      for (int kb = 0; kb < 4; ++kb)
+        if (kb >= rb && (kb & 1) == h) {
+          uint32_t a[NS][4];
+          ld_at<NS>(a, As, kTile * PK, PK, r0, 16 * kb);
+#pragma unroll
+          for (int nb = 0; nb < KD; ++nb) {
+            uint32_t b[NS][4];
+            ld_bt<NS>(b, Ws, kTile * PD, PD, 16 * nb, 16 * kb);
+            mma_sum<NS, NS>(dv[2 * nb], dv[2 * nb + 1], a, b);
+          }
+        }
+      __syncthreads();
+    }
+    // half 0 finishes dk, half 1 dv, each with the other's sums
+    us0 = quad_sum(us0);
+    us1 = quad_sum(us1);
+    float* rk = reinterpret_cast<float*>(Om) + (tid & 127);
+    float* rv = rk + (D / 2 + 2) * 128;
+#pragma unroll
+    for (int i = 0; i < D / 8; ++i)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        if (h == 1)
+          rk[(4 * i + c) * 128] = dk[i][c];
+        else
+          rv[(4 * i + c) * 128] = dv[i][c];
+      }
+    if (h == 1) {
+      rk[(D / 2) * 128] = us0;
+      rk[(D / 2 + 1) * 128] = us1;
+    }
+    __syncthreads();
+    if (h == 0) {
+      if (!square) {
+#pragma unroll
+        for (int i = 0; i < D / 8; ++i)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) dk[i][c] += rk[(4 * i + c) * 128];
+        store_dx<IO, D>(A, static_cast<IO*>(A.dk) + tp.row0 * D, Ks, r0, x0, x1, dk,
+                        us0 + rk[(D / 2) * 128], us1 + rk[(D / 2 + 1) * 128]);
+      }
+    } else {
+      IO* dvg = static_cast<IO*>(A.dv) + tp.row0 * D;
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        const int row = hf ? x1 : x0;
+        if (row >= 0) {
+#pragma unroll
+          for (int i = 0; i < D / 8; ++i)
+            store2(dvg + (size_t)row * D + 8 * i + 2 * t, dv[i][2 * hf] + rv[(4 * i + 2 * hf) * 128],
+                   dv[i][2 * hf + 1] + rv[(4 * i + 2 * hf + 1) * 128]);
+        }
+      }
+    }
+    __syncthreads();  // before the next tile's loads
+  }
+}
+
+// ------------------------------------------------------------------ launches
+// One-time, per-device shared-memory limit of a kernel, then a launch as a
+// programmatic dependent of the kernel before it in the stream.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem,
+                       cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+template <typename IO, int D, int K>
+cudaError_t smem_limit(const void* kern, int bytes) {
+  static bool set_flags[kMaxDevices] = {};
+  bool* set = device_flag(set_flags);
+  if (set == nullptr) return cudaErrorInvalidDevice;
+  if (*set) return cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) *set = true;
+  return e;
+}
+
+template <typename IO, int D>
+cudaError_t run_delta(const TileArgs& A, cudaStream_t s) {
+  constexpr int smem = DeltaSmem<IO, D>::bytes;
+  cudaError_t e = smem_limit<IO, D, 0>((const void*)k_delta<IO, D>, smem);
+  if (e != cudaSuccess) return e;
+  const double rows = (double)A.chains * A.b;
+  const double proj = A.feature == SLIM_FEAT_SQUARE ? 0.0 : 2.0;
+  prof::Scope ps(prof::K_TILE_DELTA, s, (2.0 + proj) * rows * D * A.M, 2.0 * rows * D * sizeof(IO));
+  return launch_pdl(k_delta<IO, D>, (unsigned)(A.chains * A.nf), kThreads, smem, s, A);
+}
+template <typename IO, int D, int MODE>
+cudaError_t run_out_mode(const TileArgs& A, cudaStream_t s) {
+  constexpr int smem = OutSmem<IO, D, MODE>::bytes;
+  cudaError_t e = smem_limit<IO, D, 4 + MODE>((const void*)k_out<IO, D, MODE>, smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_out<IO, D, MODE>, (unsigned)(A.chains * A.nf), kThreads, smem, s, A);
+}
+template <typename IO, int D>
+cudaError_t run_out(const TileArgs& A, cudaStream_t s) {
+  const double rows = (double)A.chains * A.b;
+  const double proj = A.feature == SLIM_FEAT_SQUARE ? 0.0 : 2.0;
+  prof::Scope ps(prof::K_TILE_OUT, s, (2.0 + proj) * rows * D * A.M,
+                 (A.causal ? 3.0 : 2.0) * rows * D * sizeof(IO));
+  return A.rows == 16   ? run_out_mode<IO, D, 2>(A, s)
+         : A.rows == 32 ? run_out_mode<IO, D, 1>(A, s)
+                        : run_out_mode<IO, D, 0>(A, s);
+}
+template <typename IO, int D>
+constexpr int slot_count() {
+  return kSms * bwd_occupancy<IO, D>();
+}
+template <typename IO, int D>
+unsigned bwd_grid(const TileArgs& A) {
+  const long long tiles = (long long)A.chains * A.nf;
+  return (unsigned)(tiles < slot_count<IO, D>() ? tiles : slot_count<IO, D>());
+}
+template <typename IO, int D>
+cudaError_t run_bwd_q(const TileArgs& A, cudaStream_t s) {
+  constexpr int smem = BwdQSmem<IO, D>::bytes;
+  cudaError_t e = smem_limit<IO, D, 2>((const void*)k_bwd_q<IO, D>, smem);
+  if (e != cudaSuccess) return e;
+  const double rows = (double)A.chains * A.b;
+  const double proj = A.feature == SLIM_FEAT_SQUARE ? 0.0 : 6.0;  // g(Q), dq, dOmega
+  prof::Scope ps(prof::K_TILE_BWD_Q, s, (4.0 + proj) * rows * D * A.M, 5.0 * rows * D * sizeof(IO));
+  return launch_pdl(k_bwd_q<IO, D>, bwd_grid<IO, D>(A), kThreads, smem, s, A);
+}
+template <typename IO, int D>
+cudaError_t run_bwd_k(const TileArgs& A, cudaStream_t s) {
+  constexpr int smem = BwdKSmem<IO, D>::bytes;
+  cudaError_t e = smem_limit<IO, D, 3>((const void*)k_bwd_k<IO, D>, smem);
+  if (e != cudaSuccess) return e;
+  const double rows = (double)A.chains * A.b;
+  const double proj = A.feature == SLIM_FEAT_SQUARE ? 0.0 : 4.0;  // dk, dOmega
+  prof::Scope ps(prof::K_TILE_BWD_K, s, (4.0 + proj) * rows * D * A.M, 4.0 * rows * D * sizeof(IO));
+  return launch_pdl(k_bwd_k<IO, D>, bwd_grid<IO, D>(A), kThreads, smem, s, A);
+}
+
+template <typename IO, int D>
+constexpr TileKernels tile_set() {
+  return TileKernels{run_delta<IO, D>, run_out<IO, D>, run_bwd_q<IO, D>, run_bwd_k<IO, D>,
+                     slot_count<IO, D>()};
+}
+
+}  // namespace simt
+}  // namespace slim

@@ -56,12 +56,12 @@ bool use_tc(const Problem& p) {
   return slim::tc::supports(p);
 }
 
-size_t ws_bytes(const Problem& p, bool bwd) {
-  return use_tc(p) ? slim::tc::workspace_bytes(p, bwd) : slim::simt::workspace_bytes(p, bwd);
+size_t ws_bytes(const Problem& p, bool bwd, bool small = false) {
+  return use_tc(p) ? slim::tc::workspace_bytes(p, bwd) : slim::simt::workspace_bytes(p, bwd, small);
 }
 
-slim_status check_workspace(const Problem& p, bool bwd, void* ws, size_t bytes) {
-  const size_t need = ws_bytes(p, bwd);
+slim_status check_workspace(const Problem& p, bool bwd, void* ws, size_t bytes, bool small = false) {
+  const size_t need = ws_bytes(p, bwd, small);
   if (need == 0) return SLIM_OK;
   if (ws == nullptr || bytes < need) return SLIM_ERR_WORKSPACE;
   if ((reinterpret_cast<uintptr_t>(ws) & 255u) != 0) return SLIM_ERR_INVALID_ARG;
@@ -78,13 +78,15 @@ cudaError_t copy_or_zero(float* dst, const float* src, size_t n, cudaStream_t s)
 
 // The forward sweep behind slim_fwd, slim_fwd_from and slim_fwd_noalloc.
 // report: the non-blocking timeout report of report.cu (off for the
-// allocation-free entry point).
+// allocation-free entry point).  small: a workspace below the size
+// slim_fwd_workspace_size gives is taken too, down to the least the sweep runs
+// in (the allocation-free entry point's fixed scratch).
 slim_status forward(const void* q, const void* k, const void* v, const float* omega, int B,
                     int H, int L, int d, int M, int C, slim_dtype dtype, slim_feature feature,
                     const float* S_init, const float* z_init, const float* S_init_lo,
                     const float* z_init_lo, void* out, float* S_state, float* z_state,
                     float* S_state_lo, float* z_state_lo, void* workspace,
-                    size_t workspace_bytes, cudaStream_t s, bool report) {
+                    size_t workspace_bytes, cudaStream_t s, bool report, bool small) {
   Problem p;
   slim_status st = check_problem(B, H, L, d, M, C, dtype, feature, &p);
   if (st != SLIM_OK) return st;
@@ -98,7 +100,7 @@ slim_status forward(const void* q, const void* k, const void* v, const float* om
   if (omega == nullptr && feature != SLIM_FEAT_SQUARE) return SLIM_ERR_INVALID_ARG;
   if (!pair_ok(S_init, z_init) || (S_init == nullptr && (S_init_lo || z_init_lo)))
     return SLIM_ERR_INVALID_ARG;
-  st = check_workspace(p, false, workspace, workspace_bytes);
+  st = check_workspace(p, false, workspace, workspace_bytes, small);
   if (st != SLIM_OK) return st;
   cudaStream_t s_ = s;
   if (L == 0) {
@@ -121,7 +123,7 @@ slim_status forward(const void* q, const void* k, const void* v, const float* om
   const slim::StateOut so{S_state, z_state, S_state_lo, z_state_lo};
   const slim::StateInit si{S_init, z_init, S_init_lo, z_init_lo};
   if (tc) return slim::tc::fwd(p, q, k, v, omega, out, so, si, counter, workspace, s_);
-  return slim::simt::fwd(p, q, k, v, omega, out, so, si, workspace, s_);
+  return slim::simt::fwd(p, q, k, v, omega, out, so, si, workspace, workspace_bytes, s_);
 }
 
 slim_status backward(const void* q, const void* k, const void* v, const float* omega,
@@ -168,6 +170,17 @@ slim_status backward(const void* q, const void* k, const void* v, const float* o
 }  // namespace
 
 namespace slim {
+// The least workspace the forward runs in (slim_fwd_workspace_size, or less
+// where that asks for more rows per launch sequence than it must).
+slim_status fwd_least_workspace(int B, int H, int L, int d, int M, int C, slim_dtype dtype,
+                                slim_feature feature, size_t* bytes) {
+  Problem p;
+  slim_status st = check_problem(B, H, L, d, M, C, dtype, feature, &p);
+  if (st != SLIM_OK) return st;
+  *bytes = ws_bytes(p, false, true);
+  return SLIM_OK;
+}
+
 // slim_fwd without the timeout report (for the allocation-free entry point,
 // which must not pin memory on its first call).
 slim_status fwd_unreported(const void* q, const void* k, const void* v, const float* omega,
@@ -177,7 +190,7 @@ slim_status fwd_unreported(const void* q, const void* k, const void* v, const fl
                            size_t workspace_bytes, cudaStream_t stream) {
   return forward(q, k, v, omega, B, H, L, d, M, C, dtype, feature, nullptr, nullptr, nullptr,
                  nullptr, out, S_state, z_state, S_state_lo, z_state_lo, workspace,
-                 workspace_bytes, stream, false);
+                 workspace_bytes, stream, false, true);
 }
 }  // namespace slim
 
@@ -223,7 +236,7 @@ slim_status slim_fwd(const void* q, const void* k, const void* v, const float* o
                      float* z_state_lo, void* workspace, size_t workspace_bytes, void* stream) {
   return forward(q, k, v, omega, B, H, L, d, M, C, dtype, feature, nullptr, nullptr, nullptr,
                  nullptr, out, S_state, z_state, S_state_lo, z_state_lo, workspace,
-                 workspace_bytes, static_cast<cudaStream_t>(stream), true);
+                 workspace_bytes, static_cast<cudaStream_t>(stream), true, false);
 }
 
 slim_status slim_fwd_from(const void* q, const void* k, const void* v, const float* omega, int B,
@@ -234,7 +247,7 @@ slim_status slim_fwd_from(const void* q, const void* k, const void* v, const flo
                           void* workspace, size_t workspace_bytes, void* stream) {
   return forward(q, k, v, omega, B, H, L, d, M, C, dtype, feature, S_init, z_init, S_init_lo,
                  z_init_lo, out, S_state, z_state, S_state_lo, z_state_lo, workspace,
-                 workspace_bytes, static_cast<cudaStream_t>(stream), true);
+                 workspace_bytes, static_cast<cudaStream_t>(stream), true, false);
 }
 
 slim_status slim_bwd(const void* q, const void* k, const void* v, const float* omega,
