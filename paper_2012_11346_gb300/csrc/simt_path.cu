@@ -37,6 +37,7 @@
 
 #include "common.cuh"
 #include "simt_path.h"
+#include "simt_short.h"
 #include "simt_tiles.h"
 
 namespace slim {
@@ -359,10 +360,19 @@ size_t workspace_bytes(const Problem& p, bool bwd, bool small) {
 
 // With less workspace than workspace_bytes asks for, the fewest rows per
 // sequence, and as many chains at a time as fit.
-slim_status fwd(const Problem& p, const void* q, const void* k, const void* v,
+slim_status fwd(const Problem& p, const void* q_ptr, const void* k, const void* v,
                 const float* omega, void* out, const StateOut& st, const StateInit& init,
                 void* workspace, size_t bytes, cudaStream_t s) {
   int batch = p.chains();
+  if (p.L <= kShortMax && p.C >= p.L) {
+    // a few rows on a running state: one launch (a frame of the general kernels
+    // holds 64 rows; measured 70 us for one row of 64 chains there, 13 us here)
+    const Seq q = sequence(p, 1, true);
+    const TileArgs A = seq_args(p, q, SeqWs{}, q_ptr, k, v, omega);
+    SLIM_TRY(launch_short(p, A.ks_n, A.ks_a, q_ptr, k, v, omega, out, st, init,
+                          static_cast<int*>(workspace), s));
+    return SLIM_OK;
+  }
   const bool small = bytes < fwd_bytes(p, batch, false);
   if (small) {
     const size_t one = fwd_bytes(p, 1, true), two = fwd_bytes(p, 2, true);
@@ -375,7 +385,7 @@ slim_status fwd(const Problem& p, const void* q, const void* k, const void* v,
   }
   for (int c0 = 0; c0 < p.chains(); c0 += batch) {
     const int n = p.chains() - c0 < batch ? p.chains() - c0 : batch;
-    const slim_status r = fwd_chains(p, c0, sequence(p, n, small), q, k, v, omega, out, st, init,
+    const slim_status r = fwd_chains(p, c0, sequence(p, n, small), q_ptr, k, v, omega, out, st, init,
                                      workspace, s);
     if (r != SLIM_OK) return r;
   }

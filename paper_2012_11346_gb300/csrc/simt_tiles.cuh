@@ -12,56 +12,14 @@
 // TFLOP/s on a GB300 (1.86 PFLOP/s for tcgen05), with 3 (bf16) or 6 (fp32)
 // piece products per product: that rate bounds these kernels.
 #pragma once
-#include <math.h>
-
-#include "profiler.h"
 #include "simt_tiles.h"
-#include "warp_mma.cuh"
+#include "tile_math.cuh"
 
 namespace slim {
 namespace simt {
 
-constexpr int kThreads = 256;  // 8 warps
 constexpr int kChunk = 32;     // features staged at a time by the row kernels
 constexpr int kSmemMax = 232448;
-
-template <typename IO> struct Pieces;
-template <> struct Pieces<bf16> { static constexpr int NX = 1, NS = 2; };
-template <> struct Pieces<float> { static constexpr int NX = 3, NS = 3; };
-
-__device__ __forceinline__ void load8(const bf16* p, float (&v)[8]) {
-  const uint4 r = *reinterpret_cast<const uint4*>(p);
-  const uint32_t w[4] = {r.x, r.y, r.z, r.w};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const float2 f = unpack2(w[i]);
-    v[2 * i] = f.x;
-    v[2 * i + 1] = f.y;
-  }
-}
-__device__ __forceinline__ void load8(const float* p, float (&v)[8]) {
-  const float4 a = reinterpret_cast<const float4*>(p)[0], b = reinterpret_cast<const float4*>(p)[1];
-  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
-}
-// 8 consecutive values as NP pieces (piece stride ps)
-template <int NP>
-__device__ __forceinline__ void store_pieces8(bf16* dst, int ps, const float (&v)[8]) {
-  uint32_t w[4][NP];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) split_pair<NP>(v[2 * i], v[2 * i + 1], w[i]);
-#pragma unroll
-  for (int p = 0; p < NP; ++p)
-    *reinterpret_cast<uint4*>(dst + p * ps) = make_uint4(w[0][p], w[1][p], w[2][p], w[3][p]);
-}
-
-// a staged element's value (the sum of its pieces, exact for a caller's rows)
-template <int NP>
-__device__ __forceinline__ float staged(const bf16* p, int ps) {
-  float v = __bfloat162float(p[(NP - 1) * ps]);
-#pragma unroll
-  for (int i = NP - 2; i >= 0; --i) v += __bfloat162float(p[i * ps]);
-  return v;
-}
 
 // x . omega as a compensated dot product (FMA TwoProduct and TwoSum, about 48
 // bits; Ogita, Rump and Oishi's Dot2): decides ReLU's branch where the
@@ -164,14 +122,9 @@ __device__ __forceinline__ void load_rows_fp(const TileArgs& A, const Frame& f, 
 }
 template <int D>
 __device__ __forceinline__ void row_norms(const float* xs, float* norm2) {
-  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-  for (int r = warp; r < kTile; r += kThreads / 32) {
-    float s = 0.f;
-#pragma unroll
-    for (int j = lane; j < D; j += 32) s = fmaf(xs[r * fp_pitch<D>() + j], xs[r * fp_pitch<D>() + j], s);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) norm2[r] = s;
+  for (int r = threadIdx.x / 32; r < kTile; r += kThreads / 32) {
+    const float s = warp_norm2<D>(xs + r * fp_pitch<D>());
+    if (threadIdx.x % 32 == 0) norm2[r] = s;
   }
 }
 // W features of Omega, columns c0.. of its [M / 64][D][64] layout, to [D][W]
@@ -184,21 +137,6 @@ __device__ __forceinline__ void stage_omega(float* dst, const float* om_t, int c
                  "l"(src + (size_t)j * 64 + q)
                  : "memory");
   }
-}
-// x . omega as a compensated dot product (FMA TwoProduct and TwoSum, about 48
-// bits; Ogita, Rump and Oishi's Dot2): decides ReLU's branch where the
-// projection's own error could.
-static __device__ __noinline__ float dot2_staged(const float* x, const float* om, int stride, int d) {
-  float sh = 0.f, sl = 0.f;
-  for (int j = 0; j < d; ++j) {
-    const float xw = x[j], ow = om[j * stride];
-    const float p = __fmul_rn(xw, ow), ep = __fmaf_rn(xw, ow, -p);
-    float t, e;
-    two_sum(sh, p, t, e);
-    sh = t;
-    sl = __fadd_rn(sl, __fadd_rn(e, ep));
-  }
-  return __fadd_rn(sh, sl);
 }
 // g of the frame's 64 rows at features c0 .. c0 + W - 1 (0 in padding rows and
 // past M); put(row, feature offset, W / 16 values) stores them.
@@ -245,8 +183,6 @@ __device__ __forceinline__ void features_rows(const TileArgs& A, const Frame& f,
 #pragma unroll
           for (int n = 0; n < NF; ++n) acc[i][n] = fmaf(x[i][k], o[k][n], acc[i][n]);
     }
-    // error bound of an fp32 dot product of length D, times a safety factor 2
-    const float gamma = 2.f * (float)(D + 2) * 5.9604645e-08f;
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
       const int r = rt + 16 * i;
@@ -254,18 +190,11 @@ __device__ __forceinline__ void features_rows(const TileArgs& A, const Frame& f,
       const float n2 = norm2[r];
 #pragma unroll
       for (int n = 0; n < NF; ++n) {
-        float v = 0.f;
-        if (ok && c0 + fq + n < A.M) {
-          v = acc[i][n];
-          if (A.feature == SLIM_FEAT_EXP) {
-            v = expf(v - 0.5f * n2) * A.inv_sqrt_m;
-          } else {
-            if (fabsf(v) <= gamma * A.om_norm[c0 + fq + n] * sqrtf(n2))
-              v = dot2_staged(xs + r * XP, om + fq + n, W, D);
-            v = v > 0.f ? v * A.inv_sqrt_m : 0.f;
-          }
-        }
-        acc[i][n] = v;
+        const int m = c0 + fq + n;
+        acc[i][n] = ok && m < A.M
+                        ? feature_fp<D>(A.feature, acc[i][n], n2, A.feature == SLIM_FEAT_RELU ? A.om_norm[m] : 0.f,
+                                        A.inv_sqrt_m, xs + r * XP, om + fq + n, W)
+                        : 0.f;
       }
     }
   }
@@ -302,36 +231,6 @@ __device__ __forceinline__ void features_to_pieces(const TileArgs& A, const Fram
       *reinterpret_cast<uint2*>(dst + (p * 64 + r) * kPF + fo) = make_uint2(a[p], b[p]);
   });
 }
-
-// the fp32 value of staged pieces, smallest piece first
-template <int NP>
-__device__ __forceinline__ void add_pieces8(const bf16* p, int ps, float (&v)[8]) {
-#pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = 0.f;
-#pragma unroll
-  for (int q = NP - 1; q >= 0; --q) {
-    float w[8];
-    load8(p + q * ps, w);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] += w[i];
-  }
-}
-template <int NP>
-__device__ __forceinline__ float round_pieces(float x) {
-  float pc[NP];
-  split_bf16<NP>(x, pc);
-  float v = 0.f;
-#pragma unroll
-  for (int q = NP - 1; q >= 0; --q) v += pc[q];
-  return v;
-}
-// D += A b for one n8 block, A's pieces smallest first
-template <int NA>
-__device__ __forceinline__ void mma_n8(float (&d)[4], const uint32_t (&a)[NA][4], uint32_t b0, uint32_t b1) {
-#pragma unroll
-  for (int i = NA - 1; i >= 0; --i) mma16816(d, a[i], b0, b1);
-}
-constexpr uint32_t kOnes = 0x3f803f80u;  // two bf16 ones
 
 // ------------------------------------------------------------------ Delta_t
 // One CTA per frame: g(K) and, tile by tile, Delta_t = g(K)^T [V | 1].  Features
@@ -533,13 +432,6 @@ __device__ __forceinline__ void stage_rows(bf16* dst, int ss, int sp, const bf16
 #pragma unroll
     for (int p = 0; p < NP; ++p) cp16(dst + p * ss + r * sp + c8, src + p * gs + (size_t)r * gp + c8);
   }
-}
-
-__device__ __forceinline__ void store2(bf16* p, float x, float y) {
-  *reinterpret_cast<uint32_t*>(p) = pack2(x, y);
-}
-__device__ __forceinline__ void store2(float* p, float x, float y) {
-  *reinterpret_cast<float2*>(p) = make_float2(x, y);
 }
 
 // ------------------------------------------------------------------ readout
@@ -1629,23 +1521,7 @@ __global__ void __launch_bounds__(kThreads, (bwd_occupancy<IO, D>()))
 }
 
 // ------------------------------------------------------------------ launches
-// One-time, per-device shared-memory limit of a kernel, then a launch as a
-// programmatic dependent of the kernel before it in the stream.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem,
-                       cudaStream_t s, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, args...);
-}
+// One-time, per-device shared-memory limit of a kernel.
 template <typename IO, int D, int K>
 cudaError_t smem_limit(const void* kern, int bytes) {
   static bool set_flags[kMaxDevices] = {};

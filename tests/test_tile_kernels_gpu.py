@@ -57,3 +57,40 @@ def test_noalloc_sweeps_chains_in_batches(cuda_device):
     torch.cuda.synchronize()
     for a, b in zip(got, ref):
         assert torch.equal(a, b)
+
+
+SHORT = [
+    # (rows per call, d, M, dtype, feature)
+    (1, 64, 256, "bf16", "exp"),
+    (3, 16, 48, "f32", "relu"),
+    (16, 32, 112, "bf16", "relu"),
+    (16, 128, 256, "f32", "exp"),
+    (7, 128, 128, "bf16", "square"),
+    (13, 64, 144, "f32", "exp"),
+]
+
+
+@pytest.mark.parametrize("r,d,M,dtype,feature", SHORT)
+def test_short_calls_equal_short_slices(cuda_device, r, d, M, dtype, feature):
+    """Calls of r <= 16 rows on a running state (one launch each, the state
+    updated in place) against one call with slices of r rows on the general
+    kernels: the same bits in out, the state and its residuals."""
+    n = 5
+    w = W.Workload("short", 2, 3, n * r, d, M, r, dtype, feature,
+                   "uniform" if feature == "relu" else "normal", "iid", seed=33)
+    x = W.make_inputs(w, device=cuda_device)
+    om = None if feature == "square" else x["omega"]
+    ref = slim.forward(x["q"], x["k"], x["v"], om, r, feature, residuals=True)
+    S, z, S_lo, z_lo = (torch.zeros_like(t) for t in ref[1:])
+    ws = torch.empty(slim.workspace_size(2, 3, r, d, M, r, x["q"].dtype, feature, False),
+                     dtype=torch.uint8, device=cuda_device)
+    for i in range(n):
+        q, k, v = (x[t][:, :, i * r:(i + 1) * r].contiguous() for t in ("q", "k", "v"))
+        out = torch.empty_like(q)
+        before = slim.launch_count()
+        slim.forward_into(q, k, v, om, 1000, feature, out, S, z, ws, S_lo=S_lo, z_lo=z_lo,
+                          S_init=S, z_init=z, S_init_lo=S_lo, z_init_lo=z_lo)
+        assert slim.launch_count() == before + 1
+        assert torch.equal(out, ref[0][:, :, i * r:(i + 1) * r]), i
+    for got, want in zip((S, z, S_lo, z_lo), ref[1:]):
+        assert torch.equal(got, want)
