@@ -59,11 +59,18 @@ constexpr int kShortRows = 1024; // rows per chain of a sequence of slices below
 
 struct Seq {
   int chains, d, M, E;
+  int slice;             // rows of a slice (of a tile when that is shorter than 64)
   int tile, pitch, per;  // a tile's padded rows and its rows; tiles per frame
   int rows, nt, nf, N;   // rows per sequence, tiles and frames per chain, sequences
   int ns;                // pieces per computed operand
   int slots;             // dOmega partials of a backward launch
 };
+
+// tiles of the first `rows` rows of a sequence (tiles start anew in every slice)
+int tiles_of(int rows, int slice, int pitch) {
+  const int per = (slice + pitch - 1) / pitch;
+  return rows / slice * per + (rows % slice + pitch - 1) / pitch;
+}
 
 // chains: how many are swept together.  small: the fewest rows per sequence; the
 // tiles are the same either way.
@@ -85,11 +92,13 @@ Seq sequence(const Problem& p, int chains, bool small) {
     const long long frame = (long long)q.per * q.pitch, half = kSeqFrames / 2 / chains;
     const long long least = (kShortRows + frame - 1) / frame;
     rows = frame * (small ? 1 : (half > least ? half : least));
-  } else if (Cs % kTile == 0 && !small && fill * kTile > Cs) {
-    rows = fill * kTile / Cs * Cs;
+  } else if (!small) {
+    const long long slices = fill / ((Cs + kTile - 1) / kTile);
+    if (slices > 1) rows = slices * Cs;
   }
   q.rows = (int)(rows < p.L ? rows : p.L);
-  q.nt = (q.rows + q.pitch - 1) / q.pitch;
+  q.slice = Cs < kTile ? q.pitch : Cs;
+  q.nt = tiles_of(q.rows, q.slice, q.pitch);
   q.nf = (q.nt + q.per - 1) / q.per;
   q.N = p.L == 0 ? 0 : (p.L + q.rows - 1) / q.rows;
   const long long frames = (long long)q.chains * q.nf;
@@ -154,6 +163,8 @@ TileArgs seq_args(const Problem& p, const Seq& q, const SeqWs& w, const void* qp
   A.chains = q.chains;
   A.rows = q.tile;
   A.pitch = q.pitch;
+  A.slice = q.slice;
+  A.slice_tiles = (q.slice + q.pitch - 1) / q.pitch;
   A.per = q.per;
   A.shift = q.per == 4 ? 4 : q.per == 2 ? 5 : 6;
   // reduction groups of short tiles' products over the features: as many as have
@@ -176,7 +187,7 @@ TileArgs seq_args(const Problem& p, const Seq& q, const SeqWs& w, const void* qp
 void seq_rows(TileArgs& A, const Problem& p, const Seq& q, int n) {
   A.a = n * q.rows;
   A.b = p.L - A.a < q.rows ? p.L - A.a : q.rows;
-  A.nt = (A.b + A.pitch - 1) / A.pitch;
+  A.nt = tiles_of(A.b, q.slice, q.pitch);
   A.nf = (A.nt + A.per - 1) / A.per;
   A.P = A.delta;
   A.p_chain = (long long)A.nt * q.E;

@@ -55,15 +55,18 @@ __device__ __forceinline__ float feature_value(const TileArgs& A, float dot, flo
 // A frame is the 64 rows a CTA works on: one tile of 48 or 64 rows, two of 32
 // or four of 16 (each padded from its A.pitch rows to A.rows).
 struct Frame {
-  int c, t0, left;  // chain, first tile, rows of the sequence from the frame's first on
+  int c, t0, left;  // chain, first tile, rows of the slice (of the sequence when a frame has
+                    // several tiles) from the frame's first on
   size_t row0;      // first row in a caller tensor
 };
 __device__ __forceinline__ Frame frame_pos(const TileArgs& A, int frame) {
   Frame f;
   f.c = frame / A.nf;
   f.t0 = frame % A.nf * A.per;
-  f.left = A.b - f.t0 * A.pitch;
-  f.row0 = (size_t)f.c * A.L + A.a + (size_t)f.t0 * A.pitch;
+  const int sl = f.t0 / A.slice_tiles, w = (f.t0 - sl * A.slice_tiles) * A.pitch, off = sl * A.slice + w;
+  f.left = A.b - off;
+  if (A.per == 1) f.left = min(f.left, A.slice - w);
+  f.row0 = (size_t)f.c * A.L + A.a + off;
   return f;
 }
 // caller row (from the frame's first) of frame row r, -1 for a padding row

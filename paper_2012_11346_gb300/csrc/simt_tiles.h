@@ -8,8 +8,8 @@ namespace simt {
 constexpr int kTile = 64;  // rows of a frame, and of the largest tile
 constexpr int kSms = 152;  // streaming multiprocessors of a GB300
 
-// One launch sequence: rows [a, a + b) of every chain, cut into nt tiles of `pitch`
-// rows per chain; a frame is `per` consecutive tiles, frame i = chain * nf + i.  A
+// One launch sequence: rows [a, a + b) of every chain, cut into nt tiles of up to
+// `pitch` rows per chain; a frame is `per` consecutive tiles, frame i = chain * nf + i.  A
 // state (S, z) is E = M d + M floats, S row-major [M][d], then z.
 struct TileArgs {
   const void *q, *k, *v, *out, *dout;  // caller tensors [chains][L][d]
@@ -34,6 +34,7 @@ struct TileArgs {
   int L, M, E, a, b, chains;
   int rows, pitch, per;        // a tile's rows in a frame (16, 32, 48 or 64) and in the sequence; tiles per frame
   int shift;                   // frame row >> shift: the tile of the frame
+  int slice, slice_tiles;      // rows and tiles of a slice (tiles start anew in every slice)
   int nt, nf;                  // tiles and frames per chain
   int ks_n, ks_a;              // reduction groups of the readout's and the scores' k16 steps (rows < 48)
   int feature, causal;
