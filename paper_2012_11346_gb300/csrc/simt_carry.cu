@@ -1,8 +1,7 @@
 // The fp32-compute path's small kernels: Omega's operand pieces, and the state
 // carried over the tiles of a launch sequence.
-#include "profiler.h"
 #include "simt_tiles.h"
-#include "warp_mma.cuh"
+#include "tile_math.cuh"
 
 namespace slim {
 namespace simt {
@@ -53,113 +52,126 @@ cudaError_t launch_setup(cudaStream_t s, const float* omega, int M, int d, float
   return cudaGetLastError();
 }
 
-// One thread per (chain, 4 consecutive state elements): the tiles are loaded
-// KB at a time so that their latencies overlap, then folded in order into the
-// value/error pair (TwoSum), so that rolling back by subtraction (eq. 17) in
-// the reverse order of the additions returns the forward's state to within the
-// pair's precision.  Bound by the tile totals' traffic through L2.
+// One thread per (chain, V consecutive state elements): the totals are loaded KB at
+// a time so that their latencies overlap, then folded in order into the value/error
+// pair (TwoSum), so that rolling back by subtraction (eq. 17) in the reverse
+// order of the additions returns the forward's state to within the pair's
+// precision.  Bound by the totals' traffic, and with few chains by the loads in
+// flight: one element per thread there (V = 1), four where the threads fill the chip.
+// The totals come one per frame (PAIR false) or as pairs.
 namespace {
-constexpr int KB = 16;
-__device__ __forceinline__ void pair_add4(float4& h, float4& l, const float4& x) {
-  pair_add(h.x, l.x, x.x);
-  pair_add(h.y, l.y, x.y);
-  pair_add(h.z, l.z, x.z);
-  pair_add(h.w, l.w, x.w);
+template <int V> struct Vec;
+template <> struct Vec<1> { typedef float T; };
+template <> struct Vec<4> { typedef float4 T; };
+
+__device__ __forceinline__ void pair_add2(float& hi, float& lo, float xh, float xl) {
+  float s, e;
+  two_sum(hi, xh, s, e);
+  two_sum(s, __fadd_rn(__fadd_rn(lo, xl), e), hi, lo);
 }
-__device__ __forceinline__ float4 pair_val4(const float4& h, const float4& l) {
-  return make_float4(h.x + l.x, h.y + l.y, h.z + l.z, h.w + l.w);
-}
-__device__ __forceinline__ float4 neg4(const float4& x) { return make_float4(-x.x, -x.y, -x.z, -x.w); }
 }  // namespace
 
-__global__ void k_carry(float4* buf, float4* hi_p, float4* lo_p, int chains, int nt, int per, int M,
-                        int d, int mode, int first, StateInit init, StateOut out) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int S4 = M * d / 4, E4 = S4 + M / 4;
+template <int V, int KB, bool PAIR>
+__global__ void __launch_bounds__(256) k_carry(const __grid_constant__ CarryArgs A) {
+  typedef typename Vec<V>::T T;
+  union Reg {
+    T v;
+    float f[V];
+  };
+  pdl_wait();
+  pdl_launch();
+  const int SV = A.M * A.d / V, EV = SV + A.M / V, mode = A.mode;
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= (long long)chains * E4) return;
-  const int c = (int)(idx / E4), e = (int)(idx % E4);
+  if (idx >= (long long)A.chains * EV) return;
+  const int c = (int)(idx / EV), e = (int)(idx % EV);
   // this element's place in a caller's (S, z) pair of arrays
-  const bool in_s = e < S4;
-  const size_t so = in_s ? (size_t)c * S4 + e : (size_t)c * (M / 4) + (e - S4);
-  float4 hi = make_float4(0.f, 0.f, 0.f, 0.f), lo = hi;
-  if (!first) {
-    hi = hi_p[idx];
-    lo = lo_p[idx];
-  } else if (init.S) {
-    hi = reinterpret_cast<const float4*>(in_s ? init.S : init.z)[so];
-    const float* il = in_s ? init.S_lo : init.z_lo;
-    if (il) lo = reinterpret_cast<const float4*>(il)[so];
+  const bool in_s = e < SV;
+  const size_t so = in_s ? (size_t)c * SV + e : (size_t)c * (A.M / V) + (e - SV);
+  T* hi_p = reinterpret_cast<T*>(A.hi);
+  T* lo_p = reinterpret_cast<T*>(A.lo);
+  Reg hi{}, lo{};
+  if (!A.first) {
+    hi.v = hi_p[idx];
+    lo.v = lo_p[idx];
+  } else if (A.init.S) {
+    hi.v = reinterpret_cast<const T*>(in_s ? A.init.S : A.init.z)[so];
+    const float* il = in_s ? A.init.S_lo : A.init.z_lo;
+    if (il) lo.v = reinterpret_cast<const T*>(il)[so];
   }
-  float4* col = buf + (size_t)c * nt * E4 + e;
-  if (mode == CARRY_GREV || mode == CARRY_ROLLBACK) {
-    for (int t0 = nt - 1; t0 >= 0; t0 -= KB) {
-      float4 x[KB];
+  const bool rev = mode == CARRY_GREV || mode == CARRY_ROLLBACK;
+  // frame i's place in buf
+  const size_t fs = (size_t)(PAIR ? 2 : 1) * EV;
+  T* col = reinterpret_cast<T*>(A.buf) + (size_t)c * A.nf * fs + e;
+  const int n = A.nf;
+  // passes over the totals: backwards for G and the rollback, forwards for P
+  for (int pass = rev ? 0 : 1; pass < (mode == CARRY_GREV ? 1 : 2); ++pass) {
+    const bool neg = pass == 0 && mode == CARRY_ROLLBACK;
+    for (int i0 = 0; i0 < n; i0 += KB) {
+      Reg x[KB], y[PAIR ? KB : 1];
 #pragma unroll
       for (int k = 0; k < KB; ++k)
-        if (t0 - k >= 0) x[k] = col[(size_t)(t0 - k) * E4];
+        if (i0 + k < n) {
+          const int i = pass == 0 ? n - 1 - i0 - k : i0 + k;
+          x[k].v = col[(size_t)i * fs];
+          if (PAIR) y[k].v = col[(size_t)i * fs + EV];
+        }
 #pragma unroll
       for (int k = 0; k < KB; ++k)
-        if (t0 - k >= 0) {
-          if (mode == CARRY_GREV) col[(size_t)(t0 - k) * E4] = pair_val4(hi, lo);
-          pair_add4(hi, lo, mode == CARRY_GREV ? x[k] : neg4(x[k]));
+        if (i0 + k < n) {
+          const int i = pass == 0 ? n - 1 - i0 - k : i0 + k;
+          if (mode != CARRY_SUM && (pass == 1 || mode == CARRY_GREV)) {
+            T* dst = col + (size_t)i * fs;
+            if (PAIR && mode == CARRY_FWD) {  // the frame's kernel moves on from the pair
+              dst[0] = hi.v;
+              dst[EV] = lo.v;
+            } else {
+              Reg p;
+#pragma unroll
+              for (int j = 0; j < V; ++j) p.f[j] = hi.f[j] + lo.f[j];
+              dst[0] = p.v;
+            }
+          }
+#pragma unroll
+          for (int j = 0; j < V; ++j) {
+            const float xh = neg ? -x[k].f[j] : x[k].f[j];
+            if (PAIR)
+              pair_add2(hi.f[j], lo.f[j], xh, neg ? -y[k].f[j] : y[k].f[j]);
+            else
+              pair_add(hi.f[j], lo.f[j], xh);
+          }
         }
     }
-    hi_p[idx] = hi;
-    lo_p[idx] = lo;
-  }
-  if (mode != CARRY_GREV) {
-    for (int t0 = 0; t0 < nt; t0 += KB) {
-      float4 x[KB];
-#pragma unroll
-      for (int k = 0; k < KB; ++k)
-        if (t0 + k < nt) x[k] = col[(size_t)(t0 + k) * E4];
-#pragma unroll
-      for (int k = 0; k < KB; ++k)
-        if (t0 + k < nt) {
-          if (mode == CARRY_FWD || (mode == CARRY_ROLLBACK && (t0 + k) % per == 0))
-            col[(size_t)(t0 + k) * E4] = pair_val4(hi, lo);
-          pair_add4(hi, lo, x[k]);
-        }
+    // the state to carry on: after the sums, or rolled back
+    if (pass == 0 || mode != CARRY_ROLLBACK) {
+      hi_p[idx] = hi.v;
+      lo_p[idx] = lo.v;
     }
   }
-  if (mode == CARRY_FWD || mode == CARRY_SUM) {
-    hi_p[idx] = hi;
-    lo_p[idx] = lo;
-  }
-  if (out.S) {
-    reinterpret_cast<float4*>(in_s ? out.S : out.z)[so] = hi;
-    float* ol = in_s ? out.S_lo : out.z_lo;
-    if (ol) reinterpret_cast<float4*>(ol)[so] = lo;
+  if (A.out.S) {
+    reinterpret_cast<T*>(in_s ? A.out.S : A.out.z)[so] = hi.v;
+    float* ol = in_s ? A.out.S_lo : A.out.z_lo;
+    if (ol) reinterpret_cast<T*>(ol)[so] = lo.v;
   }
 }
 
-cudaError_t launch_carry(cudaStream_t s, float* buf, float* hi, float* lo, int chains, int nt,
-                         int per, int M, int d, CarryMode mode, bool first, const StateInit& init,
-                         const StateOut& out) {
-  const long long n = (long long)chains * (M * (d + 1) / 4);
-  prof::Scope ps(prof::K_SCAN, s, 0.0, (double)n * 16.0 * (2.0 * nt + 4.0));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((n + 255) / 256));
-  cfg.blockDim = dim3(256);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_carry, reinterpret_cast<float4*>(buf),
-                            reinterpret_cast<float4*>(hi), reinterpret_cast<float4*>(lo), chains, nt,
-                            per, M, d, (int)mode, first ? 1 : 0, init, out);
+cudaError_t launch_carry(cudaStream_t s, const CarryArgs& a) {
+  const long long n = (long long)a.chains * a.M * (a.d + 1);
+  prof::Scope ps(prof::K_SCAN, s, 0.0, (double)n * 4.0 * (2.0 * a.nf + 4.0));
+  const bool few = n / 4 < kSms * 64;  // too few threads for the chip with four elements each
+  const unsigned grid = (unsigned)((few ? n + 255 : n / 4 + 255) / 256);
+  if (a.pairs)
+    return few ? launch_pdl(k_carry<1, 16, true>, grid, 256, 0, s, a)
+               : launch_pdl(k_carry<4, 8, true>, grid, 256, 0, s, a);
+  return few ? launch_pdl(k_carry<1, 16, false>, grid, 256, 0, s, a)
+             : launch_pdl(k_carry<4, 8, false>, grid, 256, 0, s, a);
 }
 
 // 16 float4 columns per CTA, 16 runs of partials each summed by one thread
 // (independent loads in flight: the partials come from L2), the runs then in
 // order.
 __global__ void __launch_bounds__(256) k_domega(const float4* slots, int n, float* domega, int M, int d) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_wait();
+  pdl_launch();
   __shared__ float4 sh[2][16][16];
   const int col = threadIdx.x % 16, run = threadIdx.x / 16, n4 = M * d / 4;
   const int e = blockIdx.x * 16 + col;  // M d / 4 is a multiple of 64
@@ -197,16 +209,8 @@ __global__ void __launch_bounds__(256) k_domega(const float4* slots, int n, floa
 
 cudaError_t launch_domega(cudaStream_t s, const float* slots, int n, float* domega, int M, int d) {
   prof::Scope ps(prof::K_REDUCE, s, 0.0, (double)n * M * d * 4.0);
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(M * d / 64));
-  cfg.blockDim = dim3(256);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_domega, reinterpret_cast<const float4*>(slots), n, domega, M, d);
+  return launch_pdl(k_domega, (unsigned)(M * d / 64), 256, 0, s, reinterpret_cast<const float4*>(slots), n,
+                    domega, M, d);
 }
 
 }  // namespace simt

@@ -88,10 +88,8 @@ Seq sequence(const Problem& p, int chains, bool small) {
   const long long fill = kSeqFrames / chains;  // frames per chain
   long long rows = Cs;
   if (Cs < kTile) {
-    // half as many: a frame of short tiles brings several states
-    const long long frame = (long long)q.per * q.pitch, half = kSeqFrames / 2 / chains;
-    const long long least = (kShortRows + frame - 1) / frame;
-    rows = frame * (small ? 1 : (half > least ? half : least));
+    const long long frame = (long long)q.per * q.pitch, least = (kShortRows + frame - 1) / frame;
+    rows = frame * (small ? 1 : (fill > least ? fill : least));
   } else if (!small) {
     const long long slices = fill / ((Cs + kTile - 1) / kTile);
     if (slices > 1) rows = slices * Cs;
@@ -109,7 +107,7 @@ Seq sequence(const Problem& p, int chains, bool small) {
 
 struct SeqWs {
   int* err;
-  float *st_hi, *st_lo, *delta, *om_t, *om_norm;
+  float *st_hi, *st_lo, *delta, *zdelta, *om_t, *om_norm;
   __nv_bfloat16 *om_row, *phi_k;
   float *g_hi, *g_lo, *gdelta, *slots;
   __nv_bfloat16 *phi_q, *sA, *sdA, *sW;
@@ -124,7 +122,8 @@ SeqWs carve_seq(Carver& cv, const Seq& q, bool bwd) {
   w.om_t = cv.take<float>((size_t)(q.M + 63) / 64 * 64 * q.d);
   w.om_row = cv.take<__nv_bfloat16>((size_t)3 * q.M * q.d);
   w.om_norm = cv.take<float>(q.M);
-  w.delta = cv.take<float>(C * q.nt * q.E);
+  w.delta = cv.take<float>(frames * (q.per > 1 ? 2 : 1) * q.E);
+  if (q.per > 1) w.zdelta = cv.take<float>(C * q.nt * q.M);
   w.phi_k = cv.take<__nv_bfloat16>(frames * q.ns * q.M * kTile);
   if (bwd) {
     w.g_hi = cv.take<float>(C * q.E);
@@ -150,6 +149,7 @@ TileArgs seq_args(const Problem& p, const Seq& q, const SeqWs& w, const void* qp
   A.om_row = w.om_row;
   A.om_norm = w.om_norm;
   A.delta = w.delta;
+  A.zdelta = w.zdelta;
   A.phi_k = w.phi_k;
   A.gdelta = w.gdelta;
   A.phi_q = w.phi_q;
@@ -190,11 +190,20 @@ void seq_rows(TileArgs& A, const Problem& p, const Seq& q, int n) {
   A.nt = tiles_of(A.b, q.slice, q.pitch);
   A.nf = (A.nt + A.per - 1) / A.per;
   A.P = A.delta;
-  A.p_chain = (long long)A.nt * q.E;
-  A.p_tile = q.E;
+  A.p_frame = (q.per > 1 ? 2LL : 1LL) * q.E;
+  A.p_chain = A.nf * A.p_frame;
+  A.p_lo = q.E;
   A.G = A.gdelta;
   A.g_chain = (long long)A.nf * q.E;
-  A.g_tile = q.E;
+  A.g_frame = q.E;
+}
+
+// the carry of the state (over `delta`) or of its gradient (over `gdelta`)
+CarryArgs carry(const Seq& q, const SeqWs& w, const TileArgs& A, CarryMode mode, bool first,
+                const StateInit& init, const StateOut& out) {
+  const bool grad = mode == CARRY_GREV;
+  return CarryArgs{grad ? w.gdelta : w.delta, !grad && q.per > 1, grad ? w.g_hi : w.st_hi,
+                   grad ? w.g_lo : w.st_lo, q.chains, A.nf, q.M, q.d, mode, first ? 1 : 0, init, out};
 }
 
 const float* used_omega(const Problem& p, const float* omega) {
@@ -228,8 +237,7 @@ slim_status fwd_chains(const Problem& p, int c0, const Seq& sq, const void* q, c
   for (int n = 0; n < sq.N; ++n) {
     seq_rows(A, p, sq, n);
     SLIM_TRY(tk.delta(A, s));
-    SLIM_TRY(launch_carry(s, w.delta, w.st_hi, w.st_lo, sq.chains, A.nt, 1, sq.M, sq.d, CARRY_FWD,
-                          n == 0, init, n + 1 == sq.N ? st : StateOut{}));
+    SLIM_TRY(launch_carry(s, carry(sq, w, A, CARRY_FWD, n == 0, init, n + 1 == sq.N ? st : StateOut{})));
     SLIM_TRY(tk.out(A, s));
   }
   return SLIM_OK;
@@ -271,11 +279,9 @@ slim_status bwd_impl(const Problem& p, const void* q, const void* k, const void*
     const bool first = n + 1 == sq.N;
     seq_rows(A, p, sq, n);
     SLIM_TRY(tk.delta(A, s));
-    SLIM_TRY(launch_carry(s, w.delta, w.st_hi, w.st_lo, sq.chains, A.nt, A.per, sq.M, sq.d, CARRY_ROLLBACK,
-                          first, b_in, StateOut{}));
+    SLIM_TRY(launch_carry(s, carry(sq, w, A, CARRY_ROLLBACK, first, b_in, StateOut{})));
     SLIM_TRY(tk.bwd_q(A, s));
-    SLIM_TRY(launch_carry(s, w.gdelta, w.g_hi, w.g_lo, sq.chains, A.nf, 1, sq.M, sq.d, CARRY_GREV,
-                          first, g_in, n == 0 ? g_out : StateOut{}));
+    SLIM_TRY(launch_carry(s, carry(sq, w, A, CARRY_GREV, first, g_in, n == 0 ? g_out : StateOut{})));
     SLIM_TRY(tk.bwd_k(A, s));
     if (om) SLIM_TRY(launch_domega(s, w.slots, used_slots(sq, A), domega, sq.M, sq.d));
   }
@@ -303,15 +309,15 @@ slim_status fwd_bidir_impl(const Problem& p, const void* q, const void* k, const
   for (int n = 0; n < sq.N; ++n) {
     seq_rows(A, p, sq, n);
     SLIM_TRY(tk.delta(A, s));
-    SLIM_TRY(launch_carry(s, w.delta, w.st_hi, w.st_lo, sq.chains, A.nt, 1, sq.M, sq.d, CARRY_SUM,
-                          n == 0, StateInit{}, n + 1 == sq.N ? st : StateOut{}));
+    SLIM_TRY(launch_carry(s, carry(sq, w, A, CARRY_SUM, n == 0, StateInit{}, n + 1 == sq.N ? st : StateOut{})));
   }
   // sweep 2: [num | den] = g(Q) B, out = num / den
   for (int n = 0; n < sq.N; ++n) {
     seq_rows(A, p, sq, n);
     A.P = w.st_hi;
     A.p_chain = sq.E;
-    A.p_tile = 0;
+    A.p_frame = 0;
+    A.p_lo = w.st_lo - w.st_hi;  // the pair, as the forward leaves it per frame
     SLIM_TRY(tk.out(A, s));
   }
   return SLIM_OK;
@@ -334,17 +340,18 @@ slim_status bwd_bidir_impl(const Problem& p, const void* q, const void* k, const
   A.dk = dk;
   A.dv = dv;
   // the global state as the kernels read it: a carry over no tiles
-  SLIM_TRY(launch_carry(s, w.delta, w.st_hi, w.st_lo, sq.chains, 0, 1, sq.M, sq.d, CARRY_SUM, true,
-                        StateInit{st.S, st.z, st.S_lo, st.z_lo}, StateOut{}));
+  SLIM_TRY(launch_carry(s, carry(sq, w, A, CARRY_SUM, true, StateInit{st.S, st.z, st.S_lo, st.z_lo},
+                                 StateOut{})));
   // sweep 1, query side: dphiQ = W B^T, G += g(Q)^T W
   for (int n = 0; n < sq.N; ++n) {
     seq_rows(A, p, sq, n);
     A.P = w.st_hi;
     A.p_chain = sq.E;
-    A.p_tile = 0;
+    A.p_frame = 0;
     SLIM_TRY(tk.bwd_q(A, s));
-    SLIM_TRY(launch_carry(s, w.gdelta, w.g_hi, w.g_lo, sq.chains, A.nf, 1, sq.M, sq.d, CARRY_SUM, n == 0,
-                          StateInit{}, StateOut{}));
+    CarryArgs g = carry(sq, w, A, CARRY_GREV, n == 0, StateInit{}, StateOut{});
+    g.mode = CARRY_SUM;
+    SLIM_TRY(launch_carry(s, g));
     if (om) SLIM_TRY(launch_domega(s, w.slots, used_slots(sq, A), domega, sq.M, sq.d));
   }
   // sweep 2, key/value side: dphiK = [V | 1] G^T, dV = g(K) G_S
@@ -353,7 +360,7 @@ slim_status bwd_bidir_impl(const Problem& p, const void* q, const void* k, const
     seq_rows(A, p, sq, n);
     A.G = w.g_hi;
     A.g_chain = sq.E;
-    A.g_tile = 0;
+    A.g_frame = 0;
     SLIM_TRY(tk.bwd_k(A, s));
     if (om) SLIM_TRY(launch_domega(s, w.slots, used_slots(sq, A), domega, sq.M, sq.d));
   }

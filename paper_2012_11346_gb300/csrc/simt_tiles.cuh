@@ -42,14 +42,18 @@ __device__ __noinline__ float dot2(const IO* x, const float* om, int d) {
 // recheck bound covers the accumulation of the 6 (3) piece products over d / 16
 // MMA steps, each step's truncation taken as 2^-23 of |omega| |x|, with a
 // factor of 2 to spare.
+// rowc: row_const of the row.
 template <typename IO>
-__device__ __forceinline__ float feature_value(const TileArgs& A, float dot, float half_norm, int f,
+__device__ __forceinline__ float feature_value(const TileArgs& A, float dot, float rowc, int f,
                                                const IO* x, int d) {
-  if (A.feature == SLIM_FEAT_EXP) return expf(dot - half_norm) * A.inv_sqrt_m;
-  const float gamma = 4.f * (float)(d + 2) * 5.9604645e-08f;
-  if (fabsf(dot) <= gamma * A.om_norm[f] * sqrtf(2.f * half_norm))
-    dot = dot2<IO>(x, A.omega + (size_t)f * d, d);
+  if (A.feature == SLIM_FEAT_EXP) return expf(dot - rowc) * A.inv_sqrt_m;
+  if (fabsf(dot) <= A.om_norm[f] * rowc) dot = dot2<IO>(x, A.omega + (size_t)f * d, d);
   return dot > 0.f ? dot * A.inv_sqrt_m : 0.f;
+}
+// 0.5 |x|^2 for the exponential map; for ReLU the row's factor of the recheck bound
+__device__ __forceinline__ float row_const(const TileArgs& A, float half_norm, int d) {
+  return A.feature == SLIM_FEAT_RELU ? 4.f * (float)(d + 2) * 5.9604645e-08f * sqrtf(2.f * half_norm)
+                                     : half_norm;
 }
 
 // A frame is the 64 rows a CTA works on: one tile of 48 or 64 rows, two of 32
@@ -76,24 +80,24 @@ __device__ __forceinline__ int frame_row(const TileArgs& A, const Frame& f, int 
 }
 
 // The frame's rows of one caller tensor (src: its first row; padding rows are
-// zero) as pieces [NX][64][D + 8]; half_norm (when given): 0.5 |x|^2 per row.
+// zero) as pieces [NX][64][D + 8]; row_c (when given): row_const per row.
 // D / 8 neighbouring lanes share a row.
 template <typename IO, int D>
 __device__ __forceinline__ void load_rows(const TileArgs& A, const Frame& f, const IO* src, bf16* dst,
-                                          float* half_norm) {
+                                          float* row_c) {
   constexpr int NX = Pieces<IO>::NX, PD = D + 8, G = D / 8;
   for (int e = threadIdx.x; e < kTile * G; e += kThreads) {
     const int r = e / G, c8 = (e % G) * 8, x = frame_row(A, f, r);
     float v[8] = {};
     if (x >= 0) load8(src + (size_t)x * D + c8, v);
     store_pieces8<NX>(dst + r * PD + c8, kTile * PD, v);
-    if (half_norm) {
+    if (row_c) {
       float s = 0.f;
 #pragma unroll
       for (int i = 0; i < 8; ++i) s = fmaf(v[i], v[i], s);
 #pragma unroll
       for (int o = 1; o < G; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (c8 == 0) half_norm[r] = 0.5f * s;
+      if (c8 == 0) row_c[r] = row_const(A, 0.5f * s, D);
     }
   }
 }
@@ -241,7 +245,10 @@ __device__ __forceinline__ void features_to_pieces(const TileArgs& A, const Fram
 // then the tile products from there.  g(K)'s pieces are kept for the kernels that
 // read the frame's keys.  The z column (sum of g(K) over the tile's rows) is a
 // running fp32 sum in row order for d >= 64 and a column of ones in the MMAs
-// otherwise.
+// otherwise.  The tiles of a frame of short ones are added up here, in order, as a
+// value/error pair: a state is 132 KB for d = 128, M = 256, and one per 16 rows through
+// global memory (written, scanned, read back) was most of the C = 16 step.  k_out_short
+// forms the states inside the frame again.
 // Forward and backward call this kernel on the same tiles, so the backward's
 // rollback subtracts exactly what the forward added.
 template <typename IO, int D>
@@ -249,7 +256,7 @@ struct DeltaSmem {
   static constexpr int NX = Pieces<IO>::NX, NS = Pieces<IO>::NS, PD = D + 8;
   static constexpr int xs = kTile * fp_pitch<D>() * 4, om = D * 64 * 4, v = NX * kTile * PD * 2,
                        ph = NS * 64 * kPF * 2;
-  static constexpr int bytes = xs + om + v + ph + kTile * 4;
+  static constexpr int bytes = xs + om + v + ph + kTile * 4 + 4 * 64 * 4;
   static_assert(bytes <= kSmemMax, "shared memory");
 };
 
@@ -264,6 +271,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_delta(const __grid_constant__ T
   bf16* Vs = reinterpret_cast<bf16*>(om + S::om / 4);
   bf16* Ph = Vs + S::v / 2;
   float* norm2 = reinterpret_cast<float*>(Ph + S::ph / 2);
+  float* zt = norm2 + kTile;  // [tile][64]
   pdl_wait();
   pdl_launch();
   const int frame = blockIdx.x;
@@ -283,7 +291,9 @@ __global__ void __launch_bounds__(kThreads, 2) k_delta(const __grid_constant__ T
   const int ksteps = A.rows / 16;          // k16 steps per tile
   // two reduction groups (even and odd steps) for few features
   const bool two = A.rows == 64 && (A.M == 32 || (A.M == 16 && NS == 3));
-  float* dl = A.delta + ((size_t)f.c * A.nt + f.t0) * A.E;
+  // a tile's total, or (several tiles) the frame's pair: values, then errors
+  float* dl = A.delta + (A.per == 1 ? (size_t)frame : 2 * (size_t)frame) * A.E;
+  float* zd = A.per == 1 ? dl + A.M * D : A.zdelta + ((size_t)f.c * A.nt + f.t0) * A.M;
   bf16* pk = A.phi_k ? A.phi_k + (size_t)frame * NS * 64 * A.M : nullptr;
   const int ntl = min(A.per, A.nt - f.t0);  // tiles of this frame
   for (int c0 = 0; c0 < A.M; c0 += 64) {
@@ -306,7 +316,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_delta(const __grid_constant__ T
       }
     if (16 * fb < nf) {
       const int f0 = c0 + 16 * fb + g;
-      float a0[NB][4] = {}, a1[NB][4] = {}, z0[4] = {}, z1[4] = {};
+      float a0[NB][4] = {}, a1[NB][4] = {}, lo[NB][4] = {}, z0[4] = {}, z1[4] = {}, zlo[4] = {};
 #pragma unroll
       for (int ks = 0; ks < 4; ++ks) {
         const int i = 16 * ks >> A.shift, last = ks == ksteps * (i + 1) - 1;
@@ -333,18 +343,28 @@ __global__ void __launch_bounds__(kThreads, 2) k_delta(const __grid_constant__ T
             mma_n8<NS>(z0, a, one, one);
         }
         if (last) {
-          float* dt = dl + (size_t)i * A.E;
           if (D >= 32 || h == 0) {
 #pragma unroll
             for (int nb = 0; nb < NB; ++nb) {
-              if (two)
+              float* dst = dl + (size_t)f0 * D + (D >= 32 ? CW * h : 0) + 8 * nb + 2 * t;
+              if (A.per > 1) {  // a1: the pair's value, lo its error
 #pragma unroll
-                for (int c = 0; c < 4; ++c) a0[nb][c] += a1[nb][c];
-              float* dst = dt + (size_t)f0 * D + (D >= 32 ? CW * h : 0) + 8 * nb + 2 * t;
-              *reinterpret_cast<float2*>(dst) = make_float2(a0[nb][0], a0[nb][1]);
-              *reinterpret_cast<float2*>(dst + 8 * D) = make_float2(a0[nb][2], a0[nb][3]);
+                for (int c = 0; c < 4; ++c) {
+                  pair_add(a1[nb][c], lo[nb][c], a0[nb][c]);
+                  a0[nb][c] = 0.f;
+                }
+                if (i + 1 < ntl) continue;
+                *reinterpret_cast<float2*>(dst) = make_float2(a1[nb][0], a1[nb][1]);
+                *reinterpret_cast<float2*>(dst + 8 * D) = make_float2(a1[nb][2], a1[nb][3]);
+                *reinterpret_cast<float2*>(dst + A.E) = make_float2(lo[nb][0], lo[nb][1]);
+                *reinterpret_cast<float2*>(dst + A.E + 8 * D) = make_float2(lo[nb][2], lo[nb][3]);
+              } else {
+                if (two)
 #pragma unroll
-              for (int c = 0; c < 4; ++c) a0[nb][c] = 0.f;
+                  for (int c = 0; c < 4; ++c) a0[nb][c] += a1[nb][c];
+                *reinterpret_cast<float2*>(dst) = make_float2(a0[nb][0], a0[nb][1]);
+                *reinterpret_cast<float2*>(dst + 8 * D) = make_float2(a0[nb][2], a0[nb][3]);
+              }
             }
           }
           if (D < 64 && h == 1) {
@@ -352,8 +372,19 @@ __global__ void __launch_bounds__(kThreads, 2) k_delta(const __grid_constant__ T
 #pragma unroll
               for (int c = 0; c < 4; ++c) z0[c] += z1[c];
             if (t == 0) {
-              dt[A.M * D + f0] = z0[0];
-              dt[A.M * D + f0 + 8] = z0[2];
+              zd[(size_t)i * A.M + f0] = z0[0];
+              zd[(size_t)i * A.M + f0 + 8] = z0[2];
+            }
+            if (A.per > 1) {
+#pragma unroll
+              for (int c = 0; c < 4; c += 2) pair_add(z1[c], zlo[c], z0[c]);
+              if (i + 1 == ntl && t == 0) {
+                float* dz = dl + A.M * D + f0;
+                dz[0] = z1[0];
+                dz[8] = z1[2];
+                dz[A.E] = zlo[0];
+                dz[A.E + 8] = zlo[2];
+              }
             }
 #pragma unroll
             for (int c = 0; c < 4; ++c) z0[c] = 0.f;
@@ -393,7 +424,17 @@ __global__ void __launch_bounds__(kThreads, 2) k_delta(const __grid_constant__ T
           s[0][0] += s[1][0];
           s[0][1] += s[1][1];
         }
-        *reinterpret_cast<float2*>(dl + (size_t)i * A.E + A.M * D + c0 + 2 * lane) = make_float2(s[0][0], s[0][1]);
+        *reinterpret_cast<float2*>(zd + (size_t)i * A.M + c0 + 2 * lane) = make_float2(s[0][0], s[0][1]);
+        if (A.per > 1) *reinterpret_cast<float2*>(zt + i * 64 + 2 * lane) = make_float2(s[0][0], s[0][1]);
+      }
+      if (A.per > 1) {  // the frame's pair
+        __syncthreads();
+        if (tid < nf) {
+          float zh = 0.f, zl = 0.f;
+          for (int i = 0; i < ntl; ++i) pair_add(zh, zl, zt[i * 64 + tid]);
+          dl[A.M * D + c0 + tid] = zh;
+          dl[A.E + A.M * D + c0 + tid] = zl;
+        }
       }
     }
   }
@@ -439,32 +480,26 @@ __device__ __forceinline__ void stage_rows(bf16* dst, int ss, int sp, const bf16
 
 // ------------------------------------------------------------------ readout
 // One CTA per frame: g(Q), A = tril(g(Q) g(K)^T) inside each tile, out = (g(Q) S +
-// A V) / (g(Q) z + A 1).  Warp (r, h) has rows 16 r .. 16 r + 15 and the h-th half
-// of every product's columns.  MODE 0: one tile of 48 or 64 rows, its state staged
-// in shared memory.  MODE 1 (two tiles of 32) and 2 (four of 16): every row group
-// has its own tile's state, read straight into MMA fragments; their products
-// sum the k16 steps in A.ks_* interleaved groups, added in order at the end.
-// The next chunk's Omega and state travel while this one's products run, its g(K)
-// while it is projected; FMA and tensor pipe overlap across the two CTAs of an SM.
-template <typename IO, int D, int MODE>
+// A V) / (g(Q) z + A 1).  k_out: one tile of 48 or 64 rows.  Warp (r, h) has rows 16 r ..
+// 16 r + 15 and the h-th half of every product's columns.  The next chunk's Omega and
+// state travel while this one's products run, its g(K) while it is projected; FMA and
+// tensor pipe overlap across the two CTAs of an SM.
+template <typename IO, int D>
 struct OutSmem {
   static constexpr int NX = Pieces<IO>::NX, NS = Pieces<IO>::NS, PD = D + 8;
   static constexpr int xs = kTile * fp_pitch<D>() * 4, om = D * 64 * 4, ph = NS * 64 * kPF * 2,
-                       ps = MODE == 0 ? NS * 64 * PD * 2 : 0, zs = 4 * 64 * 4;
+                       ps = NS * 64 * PD * 2, zs = 64 * 4;
   static constexpr int bytes = xs + om + 2 * ph + ps + zs + 2 * kTile * 4;
   static_assert(NX * kTile * PD * 2 <= xs + om, "V in the projections' buffers");
   static_assert(bytes <= kSmemMax, "shared memory");
 };
 
-template <typename IO, int D, int MODE>
+template <typename IO, int D>
 __global__ void __launch_bounds__(kThreads, D <= 64 ? 2 : 1)
     k_out(const __grid_constant__ TileArgs A) {
-  using S = OutSmem<IO, D, MODE>;
+  using S = OutSmem<IO, D>;
   constexpr int NX = S::NX, NS = S::NS, PD = S::PD;
   constexpr int CW = D >= 32 ? D / 2 : 16, NB = CW / 8;       // columns of a warp
-  constexpr int GN = MODE == 0 ? 1 : MODE == 1 ? 2 : NS == 2 ? 4 : 2;  // most groups: readout
-  constexpr int GA = MODE == 0 ? 1 : MODE == 1 ? 2 : NS == 2 ? 8 : 4;  // scores
-  constexpr int KB = MODE == 0 ? 4 : MODE == 1 ? 2 : 1;       // n8 blocks of a warp's scores
   constexpr bool ZM = D < 64;                                 // den as an MMA column
   extern __shared__ uint4 smem_raw[];
   float* xs = reinterpret_cast<float*>(smem_raw);
@@ -472,8 +507,8 @@ __global__ void __launch_bounds__(kThreads, D <= 64 ? 2 : 1)
   bf16* Ph = reinterpret_cast<bf16*>(om + S::om / 4);
   bf16* Kp = Ph + S::ph / 2;
   bf16* Ps = Kp + S::ph / 2;
-  float* zs = reinterpret_cast<float*>(Ps + S::ps / 2);  // [tile][64]: z rounded to the pieces
-  float* norm2 = zs + 4 * 64;
+  float* zs = reinterpret_cast<float*>(Ps + S::ps / 2);  // z rounded to the pieces
+  float* norm2 = zs + 64;
   float* den_s = norm2 + kTile;
   bf16* Vs = reinterpret_cast<bf16*>(xs);
   pdl_wait();
@@ -482,17 +517,13 @@ __global__ void __launch_bounds__(kThreads, D <= 64 ? 2 : 1)
   const Frame f = frame_pos(A, frame);
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32, g = lane >> 2, t = lane & 3;
   const int h = warp >> 2, r = warp & 3, r0 = 16 * r;
-  const int ti = MODE == 0 ? 0 : MODE == 1 ? r >> 1 : r;  // this warp's tile of the frame
-  const int ntl = min(A.per, A.nt - f.t0);
   const size_t MD = (size_t)A.M * D;
-  const float* P0 = A.P + f.c * A.p_chain + f.t0 * A.p_tile;
-  const float* Pt = P0 + min(ti, ntl - 1) * A.p_tile;
+  const float* Pt = A.P + f.c * A.p_chain + f.t0 * A.p_frame;
   const bf16* pk = A.phi_k + (size_t)frame * NS * 64 * A.M;
   const bool square = A.feature == SLIM_FEAT_SQUARE;
   const int cb = D >= 32 ? CW * h : 0;                    // first column
   const bool cols = D >= 32 || h == 0;
-  // first key of this warp's scores, and whether any of them is unmasked
-  const int k0 = MODE == 0 ? 32 * h : MODE == 1 ? 32 * ti + 16 * h : r0;
+  const int k0 = 32 * h;                                  // first key of this warp's scores
 
   StateChunk<D, 64> pc;
   auto stage_keys = [&](int c0) {
@@ -506,72 +537,323 @@ __global__ void __launch_bounds__(kThreads, D <= 64 ? 2 : 1)
   };
   stage_om(0);
   stage_keys(0);
-  if (MODE == 0) pc.load(P0, min(64, A.M));
+  pc.load(Pt, min(64, A.M));
   load_rows_fp<IO, D>(A, f, static_cast<const IO*>(A.q) + f.row0 * D, xs);
   __syncthreads();
   row_norms<D>(xs, norm2);
-  if (MODE == 0) pc.template store<NS>(Ps, min(64, A.M));
+  pc.template store<NS>(Ps, min(64, A.M));
 
-  float num[GN][NB][4] = {}, sc[GA][KB][4] = {}, dz[GN][4] = {}, de[GN] = {};
+  float num[NB][4] = {}, sc[4][4] = {}, dz[4] = {}, de = 0.f;
   // the warps with the fewest scores sum den for d >= 64, a row per lane
   const int dr = warp == 4 ? lane : warp == 5 ? 32 + lane : -1;
-  const float* zrow = zs + (dr < 0 ? 0 : (MODE == 0 ? 0 : MODE == 1 ? dr / 32 : dr / 16) * 64);
   for (int c0 = 0; c0 < A.M; c0 += 64) {
     const int nf = min(64, A.M - c0);
     cp_wait<1>();
     __syncthreads();
     features_to_pieces<D, NS>(A, f, xs, norm2, om, c0, Ph);
-    if (!ZM)
-      for (int e = tid; e < 64 * ntl; e += kThreads)
-        if (e % 64 < nf) zs[e] = round_pieces<NS>(P0[(e / 64) * A.p_tile + MD + c0 + e % 64]);
+    if (!ZM && tid < nf) zs[tid] = round_pieces<NS>(Pt[MD + c0 + tid]);
     cp_wait<0>();
     __syncthreads();
     const bool more = c0 + 64 < A.M;
     if (more) stage_om(c0 + 64);
-    if (MODE == 0 && more) pc.load(P0 + (size_t)(c0 + 64) * D, min(64, A.M - c0 - 64));
+    if (more) pc.load(Pt + (size_t)(c0 + 64) * D, min(64, A.M - c0 - 64));
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       if (16 * i >= nf) break;
-      const int step = c0 / 16 + i;
-      const int gn = GN == 1 ? 0 : step & (A.ks_n - 1), ga = GA == 1 ? 0 : step & (A.ks_a - 1);
       uint32_t a[NS][4];
       ld_a<NS>(a, Ph, 64 * kPF, kPF, r0, 16 * i);
-      const int m0 = c0 + 16 * i;
       if (cols) {
 #pragma unroll
         for (int nb = 0; nb < NB / 2; ++nb) {
           uint32_t b[NS][4];
-          if (MODE == 0) {
-            ld_bt<NS>(b, Ps, 64 * PD, PD, cb + 16 * nb, 16 * i);
-          } else {
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-              const float* p = Pt + (size_t)(m0 + 2 * t) * D + cb + 16 * nb + 8 * q + g;
-              uint32_t w0[NS], w1[NS];
-              split_pair<NS>(p[0], p[D], w0);
-              split_pair<NS>(p[8 * D], p[9 * D], w1);
-#pragma unroll
-              for (int u = 0; u < NS; ++u) {
-                b[u][2 * q] = w0[u];
-                b[u][2 * q + 1] = w1[u];
-              }
-            }
-          }
-#pragma unroll
-          for (int q = 0; q < GN; ++q)
-            if (GN == 1 || q == gn) mma_pieces<NS, NS>(num[q][2 * nb], num[q][2 * nb + 1], a, b);
+          ld_bt<NS>(b, Ps, 64 * PD, PD, cb + 16 * nb, 16 * i);
+          mma_pieces<NS, NS>(num[2 * nb], num[2 * nb + 1], a, b);
         }
       }
       if (ZM && h == 1) {  // the z column
         uint32_t w0[NS] = {}, w1[NS] = {};
         if (g == 0) {
-          const float* z = Pt + MD + m0 + 2 * t;
+          const float* z = Pt + MD + c0 + 16 * i + 2 * t;
           split_pair<NS>(z[0], z[1], w0);
           split_pair<NS>(z[8], z[9], w1);
         }
 #pragma unroll
-        for (int q = 0; q < GN; ++q)
-          if (GN == 1 || q == gn) {
+        for (int o = NS - 1; o >= 0; --o)
+#pragma unroll
+          for (int x = 0; x <= o; ++x) mma16816(dz, a[x], w0[o - x], w1[o - x]);
+      }
+      if (A.causal) {
+#pragma unroll
+        for (int kb = 0; kb < 2; ++kb)
+          if (k0 + 16 * kb <= r0) {  // later keys are masked
+            uint32_t b[NS][4];
+            ld_b<NS>(b, Kp, 64 * kPF, kPF, k0 + 16 * kb, 16 * i);
+            mma_pieces<NS, NS>(sc[2 * kb], sc[2 * kb + 1], a, b);
+          }
+      }
+      if (!ZM && dr >= 0) {  // den += g(q) z, feature after feature
+#pragma unroll
+        for (int k = 0; k < 16; k += 8) {
+          float x[8];
+          add_pieces8<NS>(Ph + dr * kPF + 16 * i + k, 64 * kPF, x);
+#pragma unroll
+          for (int u = 0; u < 8; ++u) de = fmaf(x[u], zs[16 * i + k + u], de);
+        }
+      }
+    }
+    __syncthreads();
+    if (more) {
+      stage_keys(c0 + 64);
+      pc.template store<NS>(Ps, min(64, A.M - c0 - 64));
+    }
+  }
+  if (A.causal) {
+    // masked scores as pieces (in g(Q)'s place), then A [V | 1]
+#pragma unroll
+    for (int kb = 0; kb < 4; ++kb)
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        const int row = r0 + g + 8 * hf, key = k0 + 8 * kb + 2 * t;
+        uint32_t w[NS];
+        split_pair<NS>(key <= row ? sc[kb][2 * hf] : 0.f, key + 1 <= row ? sc[kb][2 * hf + 1] : 0.f, w);
+#pragma unroll
+        for (int p = 0; p < NS; ++p)
+          *reinterpret_cast<uint32_t*>(Ph + (p * 64 + row) * kPF + key) = w[p];
+      }
+    load_rows<IO, D>(A, f, static_cast<const IO*>(A.v) + f.row0 * D, Vs, nullptr);
+    __syncthreads();
+    float av[NB][4] = {}, az[4] = {};
+#pragma unroll
+    for (int kb = 0; kb < 4; ++kb)
+      if (kb <= r) {
+        uint32_t a[NS][4];
+        ld_a<NS>(a, Ph, 64 * kPF, kPF, r0, 16 * kb);
+        if (cols) {
+#pragma unroll
+          for (int nb = 0; nb < NB / 2; ++nb) {
+            uint32_t b[NX][4];
+            ld_bt<NX>(b, Vs, kTile * PD, PD, cb + 16 * nb, 16 * kb);
+            mma_pieces<NS, NX>(av[2 * nb], av[2 * nb + 1], a, b);
+          }
+        }
+        if (ZM && h == 1) {
+          const uint32_t one = g == 0 ? kOnes : 0u;
+          mma_n8<NS>(az, a, one, one);
+        }
+      }
+#pragma unroll
+    for (int nb = 0; nb < NB; ++nb)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) num[nb][c] = av[nb][c] + num[nb][c];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) dz[c] = az[c] + dz[c];
+    if (!ZM && dr >= 0) {
+      float e = 0.f;
+      for (int k = 0; k <= dr; k += 8) {
+        float x[8];
+        add_pieces8<NS>(Ph + dr * kPF + k, 64 * kPF, x);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          if (k + u <= dr) e += x[u];
+      }
+      de = e + de;
+    }
+  }
+  if (ZM) {
+    if (h == 1 && t == 0) {
+      den_s[r0 + g] = dz[0];
+      den_s[r0 + g + 8] = dz[2];
+    }
+  } else if (dr >= 0) {
+    den_s[dr] = de;
+  }
+  __syncthreads();
+  if (!cols) return;
+  IO* og = static_cast<IO*>(A.o) + f.row0 * D;
+#pragma unroll
+  for (int hf = 0; hf < 2; ++hf) {
+    const int row = r0 + g + 8 * hf, x = frame_row(A, f, row);
+    const float den = den_s[row];
+    if (x >= 0) {
+#pragma unroll
+      for (int nb = 0; nb < NB; ++nb)
+        store2(og + (size_t)x * D + cb + 8 * nb + 2 * t, den != 0.f ? num[nb][2 * hf] / den : 0.f,
+               den != 0.f ? num[nb][2 * hf + 1] / den : 0.f);
+    }
+  }
+}
+
+// k_out for frames of several short tiles (two of 32 rows, four of 16).  The state
+// moves on from tile to tile inside the frame: a warp owns 16 columns of a chunk's
+// state, as a value/error pair in registers from the chunk's start (k_carry's
+// pair), and after each tile's readout adds the tile's Delta^T = V^T g(K) from an MMA, in
+// the layout of the readout's B fragments.  Products over the features sum their k16
+// steps in A.ks_n (readout) and A.ks_a (scores) interleaved groups, added in order
+// at the end.  Where the columns leave half of the warps free (d = 64 and less) two
+// warps share a column block, each with every other k16 step.  Scores, den and masks as
+// in k_out, warp (r, h) with rows 16 r .. 16 r + 15 and half of the tile's keys.
+template <typename IO, int D>
+struct ShortSmemOut {
+  static constexpr int NX = Pieces<IO>::NX, NS = Pieces<IO>::NS, PD = D + 8;
+  static constexpr int xs = kTile * fp_pitch<D>() * 4, om = D * 64 * 4, ph = NS * 64 * kPF * 2,
+                       v = NX * kTile * PD * 2, zs = 4 * 64 * 4;
+  static constexpr int bytes = xs + om + 2 * ph + v + zs + 2 * kTile * 4;
+  static constexpr int NCB = D / 16, NH = D == 128 ? 1 : 2;
+  static_assert(NH == 1 || NCB * 32 * 64 * 4 <= xs + om, "the second halves' sums");
+  static_assert(bytes <= kSmemMax, "shared memory");
+};
+
+template <typename IO, int D, int MODE>
+__global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant__ TileArgs A) {
+  using S = ShortSmemOut<IO, D>;
+  constexpr int NX = S::NX, NS = S::NS, PD = S::PD, NCB = S::NCB, NH = S::NH;
+  constexpr int GN = NH == 1 && MODE == 2 && NS == 2 ? 4 : 2;          // readout groups of a warp, at most
+  constexpr int GA = MODE == 1 ? 2 : NS == 2 ? 8 : 4;                  // score groups, at most
+  constexpr int KB = MODE == 1 ? 2 : 1;                                // n8 blocks of a warp's scores
+  constexpr int NTI = MODE == 1 ? 2 : 4, RB = 4 / NTI;                 // tiles, 16-row groups of a tile
+  constexpr bool ZM = D < 64;                                          // den as an MMA column
+  extern __shared__ uint4 smem_raw[];
+  float* xs = reinterpret_cast<float*>(smem_raw);
+  float* om = xs + S::xs / 4;
+  bf16* Ph = reinterpret_cast<bf16*>(om + S::om / 4);
+  bf16* Kp = Ph + S::ph / 2;
+  bf16* Vs = Kp + S::ph / 2;
+  float* zs = reinterpret_cast<float*>(Vs + S::v / 2);  // [tile][64]: z (d >= 64: rounded to the pieces)
+  float* norm2 = zs + 4 * 64;
+  float* den_s = norm2 + kTile;
+  pdl_wait();
+  pdl_launch();
+  const int frame = blockIdx.x;
+  const Frame f = frame_pos(A, frame);
+  const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32, g = lane >> 2, t = lane & 3;
+  const int h = warp >> 2, r = warp & 3, r0 = 16 * r;
+  const int ti = r / RB;                                  // this warp's tile in the scores
+  const int cb = 16 * (warp % NCB), hh = warp / NCB;      // its columns and half in the readout
+  const bool halves = NH == 2 && A.ks_n > 1;
+  const int ntl = min(A.per, A.nt - f.t0);
+  const size_t MD = (size_t)A.M * D;
+  const float* Pt = A.P + f.c * A.p_chain + f.t0 / A.per * A.p_frame;
+  const long long plo = A.p_lo;                           // from the pair's values to its errors
+  const float* zd = A.zdelta + ((size_t)f.c * A.nt + f.t0) * A.M;
+  const bf16* pk = A.phi_k + (size_t)frame * NS * 64 * A.M;
+  const bool square = A.feature == SLIM_FEAT_SQUARE;
+  const int k0 = MODE == 1 ? 32 * ti + 16 * h : r0;       // first key of this warp's scores
+
+  auto stage_keys = [&](int c0) {
+    if (A.causal)
+      stage_rows<NS>(Kp, 64 * kPF, kPF, pk + c0, (size_t)64 * A.M, A.M, 64, min(64, A.M - c0));
+    cp_commit();
+  };
+  auto stage_om = [&](int c0) {
+    if (!square) stage_omega<D, 64>(om, A.om_t, c0);
+    cp_commit();
+  };
+  stage_om(0);
+  stage_keys(0);
+  load_rows_fp<IO, D>(A, f, static_cast<const IO*>(A.q) + f.row0 * D, xs);
+  load_rows<IO, D>(A, f, static_cast<const IO*>(A.v) + f.row0 * D, Vs, nullptr);
+  __syncthreads();
+  row_norms<D>(xs, norm2);
+
+  float num[GN][4][2][4] = {}, sc[GA][KB][4] = {}, dz[4][4] = {}, de[4] = {};
+  const int dr = warp == 4 ? lane : warp == 5 ? 32 + lane : -1;  // den's rows (d >= 64)
+  const float* zrow = zs + (dr < 0 ? 0 : dr / (16 * RB) * 64);
+  auto own = [&](int i) { return halves ? hh < 2 && (i & 1) == hh : hh == 0; };
+  for (int c0 = 0; c0 < A.M; c0 += 64) {
+    const int nf = min(64, A.M - c0);
+    // the chunk's state at the frame's start: element i of step s is column cb + g + 8
+    // ((i >> 1) & 1), feature c0 + 16 s + 2 t + (i & 1) + 8 (i >> 2)
+    float hi[4][8], lo[4][8];
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        hi[s][i] = lo[s][i] = 0.f;
+        if (own(s) && 16 * s < nf) {
+          const float* p = Pt + (size_t)(c0 + 16 * s + 2 * t + (i & 1) + 8 * (i >> 2)) * D + cb + g + 8 * ((i >> 1) & 1);
+          hi[s][i] = p[0];
+          lo[s][i] = p[plo];
+        }
+      }
+    cp_wait<1>();
+    __syncthreads();
+    features_to_pieces<D, NS>(A, f, xs, norm2, om, c0, Ph);
+    if (tid < nf) {  // z at every tile of the frame
+      const float* p = Pt + MD + c0 + tid;
+      float zh = p[0], zl = p[plo];
+#pragma unroll
+      for (int j = 0; j < NTI; ++j)
+        if (j < ntl) {
+          const float z = zh + zl;
+          zs[j * 64 + tid] = ZM ? z : round_pieces<NS>(z);
+          if (A.causal) pair_add(zh, zl, zd[(size_t)j * A.M + c0 + tid]);
+        }
+    }
+    cp_wait<0>();
+    __syncthreads();
+    const bool more = c0 + 64 < A.M;
+    if (more) stage_om(c0 + 64);
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      if (16 * s >= nf) break;
+      if (own(s)) {
+        const int gn = halves ? (A.ks_n == 4 ? s >> 1 : 0) : s & (A.ks_n - 1);
+#pragma unroll
+        for (int j = 0; j < NTI; ++j) {
+          uint32_t b[NS][4];
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            uint32_t w0[NS], w1[NS];
+            split_pair<NS>(hi[s][2 * q] + lo[s][2 * q], hi[s][2 * q + 1] + lo[s][2 * q + 1], w0);
+            split_pair<NS>(hi[s][4 + 2 * q] + lo[s][4 + 2 * q], hi[s][5 + 2 * q] + lo[s][5 + 2 * q], w1);
+#pragma unroll
+            for (int p = 0; p < NS; ++p) {
+              b[p][2 * q] = w0[p];
+              b[p][2 * q + 1] = w1[p];
+            }
+          }
+          float d[2][4] = {};
+#pragma unroll
+          for (int y = 0; y < RB; ++y) {
+            const int rb = j * RB + y;
+            uint32_t a[NS][4];
+            ld_a<NS>(a, Ph, 64 * kPF, kPF, 16 * rb, 16 * s);
+#pragma unroll
+            for (int q = 0; q < GN; ++q)
+              if (q == gn) mma_pieces<NS, NS>(num[q][rb][0], num[q][rb][1], a, b);
+            if (A.causal && j + 1 < NTI) {  // Delta^T, the pieces' products in Delta's order
+              uint32_t v[NX][4], k[NS][4];
+              ld_at<NX>(v, Vs, kTile * PD, PD, cb, 16 * rb);
+              ld_bt<NS>(k, Kp, 64 * kPF, kPF, 16 * s, 16 * rb);
+#pragma unroll
+              for (int o = NS - 1; o >= 0; --o)
+#pragma unroll
+                for (int i = 0; i <= o; ++i)
+                  if (o - i < NX) {
+                    mma16816(d[0], v[o - i], k[i][0], k[i][1]);
+                    mma16816(d[1], v[o - i], k[i][2], k[i][3]);
+                  }
+            }
+          }
+          if (A.causal && j + 1 < NTI) {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) pair_add(hi[s][i], lo[s][i], d[i >> 2][i & 3]);
+          }
+        }
+      }
+      uint32_t a[NS][4];
+      ld_a<NS>(a, Ph, 64 * kPF, kPF, r0, 16 * s);
+      const int step = c0 / 16 + s, gz = s & (A.ks_n - 1), ga = step & (A.ks_a - 1);
+      if (ZM && h == 1) {  // the z column
+        uint32_t w0[NS] = {}, w1[NS] = {};
+        if (g == 0) {
+          const float* z = zs + min(ti, ntl - 1) * 64 + 16 * s + 2 * t;
+          split_pair<NS>(z[0], z[1], w0);
+          split_pair<NS>(z[8], z[9], w1);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (q == gz) {
 #pragma unroll
             for (int o = NS - 1; o >= 0; --o)
 #pragma unroll
@@ -579,9 +861,9 @@ __global__ void __launch_bounds__(kThreads, D <= 64 ? 2 : 1)
           }
       }
       if (A.causal) {
+        uint32_t b[NS][4];
         if (MODE == 2) {
-          uint32_t b[NS][4];
-          ld_b<NS>(b, Kp, 64 * kPF, kPF, r0, 16 * i);
+          ld_b<NS>(b, Kp, 64 * kPF, kPF, r0, 16 * s);
 #pragma unroll
           for (int q = 0; q < GA; ++q)
             if (q == ga) {
@@ -591,55 +873,50 @@ __global__ void __launch_bounds__(kThreads, D <= 64 ? 2 : 1)
                 for (int x = 0; x <= o; ++x)
                   mma16816(sc[q][0], a[x], h ? b[o - x][2] : b[o - x][0], h ? b[o - x][3] : b[o - x][1]);
             }
-        } else {
+        } else if (k0 <= r0) {  // later keys are masked
+          ld_b<NS>(b, Kp, 64 * kPF, kPF, k0, 16 * s);
 #pragma unroll
-          for (int kb = 0; kb < KB / 2; ++kb)
-            if (k0 + 16 * kb <= r0) {  // later keys are masked
-              uint32_t b[NS][4];
-              ld_b<NS>(b, Kp, 64 * kPF, kPF, k0 + 16 * kb, 16 * i);
-#pragma unroll
-              for (int q = 0; q < GA; ++q)
-                if (GA == 1 || q == ga) mma_pieces<NS, NS>(sc[q][2 * kb], sc[q][(2 * kb + 1) % KB], a, b);
-            }
+          for (int q = 0; q < GA; ++q)
+            if (q == ga) mma_pieces<NS, NS>(sc[q][0], sc[q][KB - 1], a, b);
         }
       }
       if (!ZM && dr >= 0) {  // den += g(q) z, feature after feature
         float e = 0.f;
 #pragma unroll
-        for (int q = 0; q < GN; ++q)
-          if (q == gn) e = de[q];
+        for (int q = 0; q < 4; ++q)
+          if (q == gz) e = de[q];
 #pragma unroll
         for (int k = 0; k < 16; k += 8) {
           float x[8];
-          add_pieces8<NS>(Ph + dr * kPF + 16 * i + k, 64 * kPF, x);
+          add_pieces8<NS>(Ph + dr * kPF + 16 * s + k, 64 * kPF, x);
 #pragma unroll
-          for (int u = 0; u < 8; ++u) e = fmaf(x[u], zrow[16 * i + k + u], e);
+          for (int u = 0; u < 8; ++u) e = fmaf(x[u], zrow[16 * s + k + u], e);
         }
 #pragma unroll
-        for (int q = 0; q < GN; ++q)
-          if (q == gn) de[q] = e;
+        for (int q = 0; q < 4; ++q)
+          if (q == gz) de[q] = e;
       }
     }
     __syncthreads();
-    if (more) {
-      stage_keys(c0 + 64);
-      if (MODE == 0) pc.template store<NS>(Ps, min(64, A.M - c0 - 64));
-    }
+    if (more) stage_keys(c0 + 64);
   }
   // the groups' sums, in order
 #pragma unroll
-  for (int q = 1; q < GN; ++q)
+  for (int q = 1; q < 4; ++q)
     if (q < A.ks_n) {
-#pragma unroll
-      for (int nb = 0; nb < NB; ++nb)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) num[0][nb][c] += num[q][nb][c];
 #pragma unroll
       for (int c = 0; c < 4; ++c) dz[0][c] += dz[q][c];
       de[0] += de[q];
     }
+  float* red = xs + (warp % NCB) * 32 * 64 + lane;  // [group][32 values] of the second half's warps
+  if (halves && hh == 1) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+#pragma unroll
+      for (int i = 0; i < 32; ++i) red[(q * 32 + i) * 32] = num[q][i >> 3][(i >> 2) & 1][i & 3];
+  }
   if (A.causal) {
-    // masked scores as pieces (in g(Q)'s place), then A [V | 1]
+    // masked scores as pieces, in g(Q)'s place
 #pragma unroll
     for (int q = 1; q < GA; ++q)
       if (q < A.ks_a) {
@@ -659,37 +936,25 @@ __global__ void __launch_bounds__(kThreads, D <= 64 ? 2 : 1)
         for (int p = 0; p < NS; ++p)
           *reinterpret_cast<uint32_t*>(Ph + (p * 64 + row) * kPF + key) = w[p];
       }
-    load_rows<IO, D>(A, f, static_cast<const IO*>(A.v) + f.row0 * D, Vs, nullptr);
-    __syncthreads();
-    float av[NB][4] = {}, az[4] = {};
+  }
+  __syncthreads();
+  if (A.causal) {
+    if (ZM && h == 1) {
+      float az[4] = {};
 #pragma unroll
-    for (int kb = 0; kb < 4; ++kb)
-      if (kb <= r && (MODE == 0 || kb == r || (MODE == 1 && kb == r - 1 && (r & 1)))) {
-        uint32_t a[NS][4];
-        ld_a<NS>(a, Ph, 64 * kPF, kPF, r0, 16 * kb);
-        if (cols) {
-#pragma unroll
-          for (int nb = 0; nb < NB / 2; ++nb) {
-            uint32_t b[NX][4];
-            ld_bt<NX>(b, Vs, kTile * PD, PD, cb + 16 * nb, 16 * kb);
-            mma_pieces<NS, NX>(av[2 * nb], av[2 * nb + 1], a, b);
-          }
-        }
-        if (ZM && h == 1) {
+      for (int kb = 0; kb < 4; ++kb)
+        if (kb <= r && kb / RB == ti) {
+          uint32_t a[NS][4];
+          ld_a<NS>(a, Ph, 64 * kPF, kPF, r0, 16 * kb);
           const uint32_t one = g == 0 ? kOnes : 0u;
           mma_n8<NS>(az, a, one, one);
         }
-      }
 #pragma unroll
-    for (int nb = 0; nb < NB; ++nb)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) num[0][nb][c] = av[nb][c] + num[0][nb][c];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) dz[0][c] = az[c] + dz[0][c];
+      for (int c = 0; c < 4; ++c) dz[0][c] = az[c] + dz[0][c];
+    }
     if (!ZM && dr >= 0) {
       float e = 0.f;
-      const int kf = MODE == 0 ? 0 : dr >> A.shift << A.shift;  // the tile's first key
-      for (int k = kf; k <= dr; k += 8) {
+      for (int k = dr / (16 * RB) * (16 * RB); k <= dr; k += 8) {
         float x[8];
         add_pieces8<NS>(Ph + dr * kPF + k, 64 * kPF, x);
 #pragma unroll
@@ -708,17 +973,50 @@ __global__ void __launch_bounds__(kThreads, D <= 64 ? 2 : 1)
     den_s[dr] = de[0];
   }
   __syncthreads();
-  if (!cols) return;
+  if (hh > 0) return;
   IO* og = static_cast<IO*>(A.o) + f.row0 * D;
 #pragma unroll
-  for (int hf = 0; hf < 2; ++hf) {
-    const int row = r0 + g + 8 * hf, x = frame_row(A, f, row);
-    const float den = den_s[row];
-    if (x >= 0) {
+  for (int rb = 0; rb < 4; ++rb) {
+    float av[2][4] = {};
+    if (A.causal) {
 #pragma unroll
-      for (int nb = 0; nb < NB; ++nb)
-        store2(og + (size_t)x * D + cb + 8 * nb + 2 * t, den != 0.f ? num[0][nb][2 * hf] / den : 0.f,
-               den != 0.f ? num[0][nb][2 * hf + 1] / den : 0.f);
+      for (int kb = 0; kb < 4; ++kb)
+        if (kb <= rb && kb / RB == rb / RB) {
+          uint32_t a[NS][4], b[NX][4];
+          ld_a<NS>(a, Ph, 64 * kPF, kPF, 16 * rb, 16 * kb);
+          ld_bt<NX>(b, Vs, kTile * PD, PD, cb, 16 * kb);
+          mma_pieces<NS, NX>(av[0], av[1], a, b);
+        }
+    }
+#pragma unroll
+    for (int nb = 0; nb < 2; ++nb)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int i = rb * 8 + nb * 4 + c;
+        float v = num[0][rb][nb][c];
+        if (halves) {  // groups 0, 2 here and 1, 3 in the second half
+          v += red[i * 32];
+          if (A.ks_n == 4) {
+            v += num[1][rb][nb][c];
+            v += red[(32 + i) * 32];
+          }
+        } else {
+#pragma unroll
+          for (int q = 1; q < GN; ++q)
+            if (q < A.ks_n) v += num[q][rb][nb][c];
+        }
+        av[nb][c] += v;
+      }
+#pragma unroll
+    for (int hf = 0; hf < 2; ++hf) {
+      const int row = 16 * rb + g + 8 * hf, x = frame_row(A, f, row);
+      const float den = den_s[row];
+      if (x >= 0) {
+#pragma unroll
+        for (int nb = 0; nb < 2; ++nb)
+          store2(og + (size_t)x * D + cb + 8 * nb + 2 * t, den != 0.f ? av[nb][2 * hf] / den : 0.f,
+                 den != 0.f ? av[nb][2 * hf + 1] / den : 0.f);
+      }
     }
   }
 }
@@ -968,7 +1266,7 @@ __global__ void __launch_bounds__(kThreads, (bwd_occupancy<IO, D>()))
     const IO* vg = static_cast<const IO*>(A.v) + tp.row0 * D;
     const IO* dog = static_cast<const IO*>(A.dout) + tp.row0 * D;
     const IO* og = static_cast<const IO*>(A.out) + tp.row0 * D;
-    const float* Pt = A.P + tp.c * A.p_chain + tp.t0 * A.p_tile;
+    const float* Pt = A.P + tp.c * A.p_chain + tp.t0 / A.per * A.p_frame;
     const bf16* kt = A.phi_k + (size_t)tile * NS * A.M * kTile;
     bf16* pq = A.phi_q + (size_t)tile * NS * A.M * kTile;
     bf16* sA = A.sA + (size_t)tile * NS * kTile * kTile;
@@ -1339,7 +1637,7 @@ __global__ void __launch_bounds__(kThreads, (bwd_occupancy<IO, D>()))
     const Frame tp = frame_pos(A, tile);
     const int x0 = frame_row(A, tp, r0 + g), x1 = frame_row(A, tp, r0 + g + 8);
     const IO* kg = static_cast<const IO*>(A.k) + tp.row0 * D;
-    const float* Gt = A.G + tp.c * A.g_chain + tp.t0 / A.per * A.g_tile;
+    const float* Gt = A.G + tp.c * A.g_chain + tp.t0 / A.per * A.g_frame;
     const bf16* pq = A.phi_q + (size_t)tile * NS * A.M * kTile;
     const bf16* sA = A.sA + (size_t)tile * NS * kTile * kTile;
     const bf16* sdA = A.sdA + (size_t)tile * NS * kTile * kTile;
@@ -1547,11 +1845,11 @@ cudaError_t run_delta(const TileArgs& A, cudaStream_t s) {
   return launch_pdl(k_delta<IO, D>, (unsigned)(A.chains * A.nf), kThreads, smem, s, A);
 }
 template <typename IO, int D, int MODE>
-cudaError_t run_out_mode(const TileArgs& A, cudaStream_t s) {
-  constexpr int smem = OutSmem<IO, D, MODE>::bytes;
-  cudaError_t e = smem_limit<IO, D, 4 + MODE>((const void*)k_out<IO, D, MODE>, smem);
+cudaError_t run_out_short(const TileArgs& A, cudaStream_t s) {
+  constexpr int smem = ShortSmemOut<IO, D>::bytes;
+  cudaError_t e = smem_limit<IO, D, 4 + MODE>((const void*)k_out_short<IO, D, MODE>, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_out<IO, D, MODE>, (unsigned)(A.chains * A.nf), kThreads, smem, s, A);
+  return launch_pdl(k_out_short<IO, D, MODE>, (unsigned)(A.chains * A.nf), kThreads, smem, s, A);
 }
 template <typename IO, int D>
 cudaError_t run_out(const TileArgs& A, cudaStream_t s) {
@@ -1559,9 +1857,12 @@ cudaError_t run_out(const TileArgs& A, cudaStream_t s) {
   const double proj = A.feature == SLIM_FEAT_SQUARE ? 0.0 : 2.0;
   prof::Scope ps(prof::K_TILE_OUT, s, (2.0 + proj) * rows * D * A.M,
                  (A.causal ? 3.0 : 2.0) * rows * D * sizeof(IO));
-  return A.rows == 16   ? run_out_mode<IO, D, 2>(A, s)
-         : A.rows == 32 ? run_out_mode<IO, D, 1>(A, s)
-                        : run_out_mode<IO, D, 0>(A, s);
+  if (A.rows == 16) return run_out_short<IO, D, 2>(A, s);
+  if (A.rows == 32) return run_out_short<IO, D, 1>(A, s);
+  constexpr int smem = OutSmem<IO, D>::bytes;
+  cudaError_t e = smem_limit<IO, D, 1>((const void*)k_out<IO, D>, smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_out<IO, D>, (unsigned)(A.chains * A.nf), kThreads, smem, s, A);
 }
 template <typename IO, int D>
 constexpr int slot_count() {

@@ -18,12 +18,14 @@ struct TileArgs {
   const float* om_t;           // transposed in blocks of 64 features: [M / 64][d][64], zero past M
   const __nv_bfloat16* om_row; // its pieces [3][M][d]
   const float* om_norm;        // |omega_m|
-  float* delta;                // [tiles][E]: a tile's sum of T_l
-  const float* P;              // state of tile t at P + chain * p_chain + t * p_tile
-  long long p_chain, p_tile;
+  float* delta;                // [frames][E]: a tile's sum of T_l; with several tiles per frame
+                               // [frames][2][E], the frame's sum as a value/error pair
+  float* zdelta;               // [tiles][M]: the z part of every tile (several tiles per frame)
+  const float* P;              // state of frame i at P + chain * p_chain + i * p_frame; its errors
+  long long p_chain, p_frame, p_lo;  // p_lo further (the forward, several tiles per frame)
   float* gdelta;               // [frames][E]: a frame's share of the state gradient
   const float* G;              // state gradient of frame i, as for P
-  long long g_chain, g_tile;
+  long long g_chain, g_frame;
   __nv_bfloat16* phi_k;        // [frames][pieces][64][M]: g(K)
   // what the query side of the backward leaves for the key side, in pieces
   __nv_bfloat16 *phi_q;        // [frames][pieces][64][M]: g(Q)
@@ -57,18 +59,22 @@ cudaError_t launch_setup(cudaStream_t s, const float* omega, int M, int d, float
                          __nv_bfloat16* om_row, float* om_norm, float* domega, int* err);
 
 enum CarryMode {
-  CARRY_FWD = 0,       // P_t = B + sum_{t'<t} D_t' (in place), then B += sum_t D_t
-  CARRY_SUM = 1,       // B += sum_t D_t only
-  CARRY_ROLLBACK = 2,  // B -= sum_t D_t (eq. 17), then P_t as CARRY_FWD, B left rolled back
-  CARRY_GREV = 3       // G_t = G + sum_{t'>t} D_t' (in place), then G += sum_t D_t
+  CARRY_FWD = 0,       // P_i = B + sum_{i'<i} D_i' (in place), then B += sum_i D_i
+  CARRY_SUM = 1,       // B += sum_i D_i only
+  CARRY_ROLLBACK = 2,  // B -= sum_i D_i (eq. 17), then P_i as CARRY_FWD, B left rolled back
+  CARRY_GREV = 3       // G_i = G + sum_{i'>i} D_i' (in place), then G += sum_i D_i
 };
-// The carried state over the nt tile totals of `buf`, as a value/error pair
-// (hi, lo) [chains][E].  first: the pair starts from `init` (zero when init.S
-// is null) instead of hi / lo.  out.S non-null: the pair is also written there.
-// per: CARRY_ROLLBACK writes only every per-th tile's P_t (a frame's first).
-cudaError_t launch_carry(cudaStream_t s, float* buf, float* hi, float* lo, int chains, int nt,
-                         int per, int M, int d, CarryMode mode, bool first, const StateInit& init,
-                         const StateOut& out);
+struct CarryArgs {
+  float* buf;           // frame totals [chains][nf][E], or pairs [chains][nf][2][E]
+  int pairs;
+  float *hi, *lo;       // the carried state, a value/error pair [chains][E]
+  int chains, nf, M, d;
+  CarryMode mode;
+  int first;            // the pair starts from `init` (zero when init.S is null) instead of hi / lo
+  StateInit init;
+  StateOut out;         // out.S non-null: the pair is also written there
+};
+cudaError_t launch_carry(cudaStream_t s, const CarryArgs& a);
 
 // dOmega += the `n` partials, in a fixed order, compensated (TwoSum).
 cudaError_t launch_domega(cudaStream_t s, const float* slots, int n, float* domega, int M, int d);
