@@ -230,7 +230,10 @@ slim_status fwd_chains(const Problem& p, int c0, const Seq& sq, const void* q, c
   st = StateOut{off(st.S, so), off(st.z, zo), off(st.S_lo, so), off(st.z_lo, zo)};
   init = StateInit{off(init.S, so), off(init.z, zo), off(init.S_lo, so), off(init.z_lo, zo)};
   TileArgs A = seq_args(p, sq, w, rows_from(p, q, c0), rows_from(p, k, c0), rows_from(p, v, c0), omega);
-  A.o = const_cast<void*>(rows_from(p, out, c0));
+  if (out)
+    A.o = const_cast<void*>(rows_from(p, out, c0));
+  else
+    A.phi_k = nullptr;  // the state alone
   A.causal = 1;
   SLIM_TRY(launch_setup(s, used_omega(p, omega), sq.M, sq.d, w.om_t, w.om_row, w.om_norm, nullptr,
                         w.err));
@@ -238,7 +241,7 @@ slim_status fwd_chains(const Problem& p, int c0, const Seq& sq, const void* q, c
     seq_rows(A, p, sq, n);
     SLIM_TRY(tk.delta(A, s));
     SLIM_TRY(launch_carry(s, carry(sq, w, A, CARRY_FWD, n == 0, init, n + 1 == sq.N ? st : StateOut{})));
-    SLIM_TRY(tk.out(A, s));
+    if (out) SLIM_TRY(tk.out(A, s));
   }
   return SLIM_OK;
 }
@@ -382,7 +385,7 @@ slim_status fwd(const Problem& p, const void* q_ptr, const void* k, const void* 
                 const float* omega, void* out, const StateOut& st, const StateInit& init,
                 void* workspace, size_t bytes, cudaStream_t s) {
   int batch = p.chains();
-  if (p.L <= kShortMax && p.C >= p.L) {
+  if (out && p.L <= kShortMax && p.C >= p.L) {
     // a few rows on a running state: one launch (a frame of the general kernels
     // holds 64 rows; measured 70 us for one row of 64 chains there, 13 us here)
     const Seq q = sequence(p, 1, true);

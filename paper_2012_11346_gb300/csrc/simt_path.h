@@ -9,6 +9,7 @@ namespace simt {
 // on, and sweeps fewer rows and chains at a time below the full size)
 size_t workspace_bytes(const Problem& p, bool bwd, bool small = false);
 
+// out null: the state alone
 slim_status fwd(const Problem& p, const void* q, const void* k, const void* v,
                 const float* omega, void* out, const StateOut& st, const StateInit& init,
                 void* workspace, size_t bytes, cudaStream_t s);

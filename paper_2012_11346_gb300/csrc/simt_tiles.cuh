@@ -257,11 +257,14 @@ struct DeltaSmem {
   static constexpr int xs = kTile * fp_pitch<D>() * 4, om = D * 64 * 4, v = NX * kTile * PD * 2,
                        ph = NS * 64 * kPF * 2;
   static constexpr int bytes = xs + om + v + ph + kTile * 4 + 4 * 64 * 4;
+  // three CTAs on an SM for bf16 where their shared memory fits (228 KB, 1 KB of it per
+  // CTA): 482 -> 465 us of the non-causal step; fp32 spills (ragged step 378 -> 388 us)
+  static constexpr int ctas = NX == 1 && 3 * (bytes + 1024) <= 233472 ? 3 : 2;
   static_assert(bytes <= kSmemMax, "shared memory");
 };
 
 template <typename IO, int D>
-__global__ void __launch_bounds__(kThreads, 2) k_delta(const __grid_constant__ TileArgs A) {
+__global__ void __launch_bounds__(kThreads, (DeltaSmem<IO, D>::ctas)) k_delta(const __grid_constant__ TileArgs A) {
   using S = DeltaSmem<IO, D>;
   constexpr int NX = S::NX, NS = S::NS, PD = S::PD;
   constexpr int CW = D >= 32 ? D / 2 : 16, NB = CW / 8;  // columns of a warp

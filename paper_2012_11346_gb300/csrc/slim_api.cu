@@ -80,13 +80,15 @@ cudaError_t copy_or_zero(float* dst, const float* src, size_t n, cudaStream_t s)
 // report: the non-blocking timeout report of report.cu (off for the
 // allocation-free entry point).  small: a workspace below the size
 // slim_fwd_workspace_size gives is taken too, down to the least the sweep runs
-// in (the allocation-free entry point's fixed scratch).
+// in (the allocation-free entry point's fixed scratch).  state_only: out is null and
+// only the state is computed.
 slim_status forward(const void* q, const void* k, const void* v, const float* omega, int B,
                     int H, int L, int d, int M, int C, slim_dtype dtype, slim_feature feature,
                     const float* S_init, const float* z_init, const float* S_init_lo,
                     const float* z_init_lo, void* out, float* S_state, float* z_state,
                     float* S_state_lo, float* z_state_lo, void* workspace,
-                    size_t workspace_bytes, cudaStream_t s, bool report, bool small) {
+                    size_t workspace_bytes, cudaStream_t s, bool report, bool small,
+                    bool state_only = false) {
   Problem p;
   slim_status st = check_problem(B, H, L, d, M, C, dtype, feature, &p);
   if (st != SLIM_OK) return st;
@@ -95,7 +97,7 @@ slim_status forward(const void* q, const void* k, const void* v, const float* om
   const void* seq[] = {q, k, v, out};
   const void* fixed[] = {S_state, z_state};
   const void* opt[] = {S_state_lo, z_state_lo, S_init, z_init, S_init_lo, z_init_lo, omega};
-  if (!pointers_ok(seq, 4, L == 0) || !pointers_ok(fixed, 2, false) || !pointers_ok(opt, 7, true))
+  if (!pointers_ok(seq, state_only ? 3 : 4, L == 0) || !pointers_ok(fixed, 2, false) || !pointers_ok(opt, 7, true))
     return SLIM_ERR_INVALID_ARG;
   if (omega == nullptr && feature != SLIM_FEAT_SQUARE) return SLIM_ERR_INVALID_ARG;
   if (!pair_ok(S_init, z_init) || (S_init == nullptr && (S_init_lo || z_init_lo)))
@@ -179,6 +181,16 @@ slim_status fwd_least_workspace(int B, int H, int L, int d, int M, int C, slim_d
   if (st != SLIM_OK) return st;
   *bytes = ws_bytes(p, false, true);
   return SLIM_OK;
+}
+
+// slim_fwd's state alone (the same bits), without out, from the zero state.
+slim_status fwd_state(const void* q, const void* k, const void* v, const float* omega, int B, int H,
+                      int L, int d, int M, int C, slim_dtype dtype, slim_feature feature,
+                      float* S_state, float* z_state, float* S_state_lo, float* z_state_lo,
+                      void* workspace, size_t workspace_bytes, cudaStream_t stream) {
+  return forward(q, k, v, omega, B, H, L, d, M, C, dtype, feature, nullptr, nullptr, nullptr, nullptr,
+                 nullptr, S_state, z_state, S_state_lo, z_state_lo, workspace, workspace_bytes, stream,
+                 true, false, true);
 }
 
 // slim_fwd without the timeout report (for the allocation-free entry point,

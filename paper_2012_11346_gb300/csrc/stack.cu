@@ -22,18 +22,43 @@
 #include "stack.h"
 
 namespace slim {
+slim_status fwd_state(const void* q, const void* k, const void* v, const float* omega, int B, int H,
+                      int L, int d, int M, int C, slim_dtype dtype, slim_feature feature,
+                      float* S_state, float* z_state, float* S_state_lo, float* z_state_lo,
+                      void* workspace, size_t workspace_bytes, cudaStream_t stream);  // slim_api.cu
+
 namespace stack {
 namespace {
 
-// (hi, lo) -= (dhi, dlo): the rollback of eq. 17 on an fp32 value/error pair
-__global__ void k_pair_sub(float* hi, float* lo, const float* dhi, const float* dlo, long long n) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float h = hi[i], l = lo[i];
-  pair_add(h, l, -dhi[i]);
-  pair_add(h, l, -dlo[i]);
-  hi[i] = h;
-  lo[i] = l;
+// The rollback of eq. 17 on fp32 value/error pairs, S and z in one launch:
+// (hi2, lo2) = (hi, lo) - (dhi, dlo), 4 elements per thread (bound by its traffic; the
+// state's element counts are multiples of 4); dlo null: zero.
+struct PairSub {
+  const float *hi, *lo, *dhi, *dlo;
+  float *hi2, *lo2;
+  long long n4;
+};
+__global__ void k_pair_sub(PairSub S, PairSub z) {
+  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool in_s = i < S.n4;
+  if (!in_s) i -= S.n4;
+  const PairSub& p = in_s ? S : z;
+  if (i >= p.n4) return;
+  float4 h = reinterpret_cast<const float4*>(p.hi)[i], l = reinterpret_cast<const float4*>(p.lo)[i];
+  const float4 dh = reinterpret_cast<const float4*>(p.dhi)[i];
+  pair_add(h.x, l.x, -dh.x);
+  pair_add(h.y, l.y, -dh.y);
+  pair_add(h.z, l.z, -dh.z);
+  pair_add(h.w, l.w, -dh.w);
+  if (p.dlo) {
+    const float4 dl = reinterpret_cast<const float4*>(p.dlo)[i];
+    pair_add(h.x, l.x, -dl.x);
+    pair_add(h.y, l.y, -dl.y);
+    pair_add(h.z, l.z, -dl.z);
+    pair_add(h.w, l.w, -dl.w);
+  }
+  reinterpret_cast<float4*>(p.hi2)[i] = h;
+  reinterpret_cast<float4*>(p.lo2)[i] = l;
 }
 constexpr float kNormEps = 1e-6f;
 constexpr int kRowThreads = 256;  // threads per block of the row kernels
@@ -223,12 +248,12 @@ cudaError_t scatter(const void* src, void* dst, const Geo& g, int L, int d, int 
 struct Ws {
   uint8_t** xin;  // backward: [s] each layer's slice input; forward: two, ping-pong
   uint8_t** yout; // [s] layer outputs on the slice
-  float *Sb, *zb, *Slb, *zlb;   // [s] running states (backward), value/error pairs
-  float *Se, *ze, *Sle, *zle;   // [s] states at the slice's end (backward)
+  float *Se, *ze, *Sle, *zle;   // [s] states at the slice's end (backward), value/error pairs
+  float *Sb, *zb, *Slb, *zlb;   // [s] the same rolled back to its start
   float *dS, *dz, *dSl, *dzl;   // one slice's own contribution (rollback)
   float *G, *gz, *G2, *gz2;     // [s] state gradients, double-buffered
   float *dx;                    // fp32 dX of the slice
-  uint8_t *dout, *dq, *dk, *dv, *scratch_y;
+  uint8_t *dout, *dq, *dk, *dv;
   uint8_t* u;                   // the normalised rows of one layer's slice input
   float* dom;                   // one call's dOmega
   float *Ssc, *zsc;             // a recompute's end state, not needed
@@ -268,7 +293,6 @@ Ws carve(Carver& cv, const Problem& p, const Geo& g, bool bwd, uint8_t** xin_ptr
     w.dq = cv.take<uint8_t>(sb);
     w.dk = cv.take<uint8_t>(sb);
     w.dv = cv.take<uint8_t>(sb);
-    w.scratch_y = cv.take<uint8_t>(sb);
     w.dom = cv.take<float>((size_t)p.M * p.d);
     w.Ssc = cv.take<float>(g.st);
     w.zsc = cv.take<float>(g.zt);
@@ -357,16 +381,17 @@ slim_status bwd_impl(const Problem& p, int layers, const T* x, const float* omeg
   Carver cv(workspace);
   uint8_t* xin[65];
   uint8_t* yo[64];
-  const Ws w = carve(cv, p, g, true, xin, yo);
+  Ws w = carve(cv, p, g, true, xin, yo);
   const int d = p.d, M = p.M;
   const size_t S = (size_t)layers * g.st, Z = (size_t)layers * g.zt;
-  // running states start at the final states B^(N) (value/error pairs)
-  ST_TRY(cudaMemcpyAsync(w.Sb, S_state, S * 4, cudaMemcpyDeviceToDevice, s));
-  ST_TRY(cudaMemcpyAsync(w.zb, z_state, Z * 4, cudaMemcpyDeviceToDevice, s));
-  if (S_lo) ST_TRY(cudaMemcpyAsync(w.Slb, S_lo, S * 4, cudaMemcpyDeviceToDevice, s));
-  else ST_TRY(cudaMemsetAsync(w.Slb, 0, S * 4, s));
-  if (z_lo) ST_TRY(cudaMemcpyAsync(w.zlb, z_lo, Z * 4, cudaMemcpyDeviceToDevice, s));
-  else ST_TRY(cudaMemsetAsync(w.zlb, 0, Z * 4, s));
+  // running states start at the final states B^(N) (value/error pairs): in Se, the state
+  // at a slice's end; rolled back into Sb, which is the next slice's Se
+  ST_TRY(cudaMemcpyAsync(w.Se, S_state, S * 4, cudaMemcpyDeviceToDevice, s));
+  ST_TRY(cudaMemcpyAsync(w.ze, z_state, Z * 4, cudaMemcpyDeviceToDevice, s));
+  if (S_lo) ST_TRY(cudaMemcpyAsync(w.Sle, S_lo, S * 4, cudaMemcpyDeviceToDevice, s));
+  else ST_TRY(cudaMemsetAsync(w.Sle, 0, S * 4, s));
+  if (z_lo) ST_TRY(cudaMemcpyAsync(w.zle, z_lo, Z * 4, cudaMemcpyDeviceToDevice, s));
+  else ST_TRY(cudaMemsetAsync(w.zle, 0, Z * 4, s));
   if (domegas) ST_TRY(cudaMemsetAsync(domegas, 0, (size_t)layers * M * d * 4, s));
   float *G = w.G, *gz = w.gz, *G2 = w.G2, *gz2 = w.gz2;
   const float scale = powf((float)d, -0.25f);
@@ -375,6 +400,8 @@ slim_status bwd_impl(const Problem& p, int layers, const T* x, const float* omeg
     const int a = n * g.Cs, b = (p.L - a < g.Cs) ? p.L - a : g.Cs;
     const long long rows = (long long)g.chains * b;
     const double sb = (double)rows * d * g.esz;
+    int path = 0;  // the slice's kernels (a short last slice can differ)
+    ST_CALL(slim_path_for(p.B, p.H, b, d, M, b, p.dtype, p.feature, &path));
     ST_TRY(gather(x, w.xin[0], g, p.L, d, a, b, s));
     STACK_LAUNCH(2 * sb, k_rownorm<T><<<nrb(rows, d), kRowThreads, 0, s>>>(
                              reinterpret_cast<const T*>(w.xin[0]), U, d, scale, rows));
@@ -383,21 +410,17 @@ slim_status bwd_impl(const Problem& p, int layers, const T* x, const float* omeg
     for (int r = 0; r < layers; ++r) {
       const T* X = reinterpret_cast<const T*>(w.xin[r]);
       const float* om = omegas ? omegas + (size_t)r * M * d : nullptr;
-      float* Sb = w.Sb + r * g.st;
-      float* zb = w.zb + r * g.zt;
-      float* Slb = w.Slb + r * g.st;
-      float* zlb = w.zlb + r * g.zt;
-      // the state at the slice's end, for the layer's backward
-      ST_TRY(cudaMemcpyAsync(w.Se + r * g.st, Sb, g.st * 4, cudaMemcpyDeviceToDevice, s));
-      ST_TRY(cudaMemcpyAsync(w.ze + r * g.zt, zb, g.zt * 4, cudaMemcpyDeviceToDevice, s));
-      ST_TRY(cudaMemcpyAsync(w.Sle + r * g.st, Slb, g.st * 4, cudaMemcpyDeviceToDevice, s));
-      ST_TRY(cudaMemcpyAsync(w.zle + r * g.zt, zlb, g.zt * 4, cudaMemcpyDeviceToDevice, s));
-      // eq. 17: B_r -= the slice's sum of T_l (its own contribution, from zero)
-      ST_CALL(slim_fwd_from(U, U, U, om, p.B, p.H, b, d, M, b, p.dtype, p.feature, nullptr,
-                            nullptr, nullptr, nullptr, w.scratch_y, w.dS, w.dz, w.dSl, w.dzl,
-                            w.inner, g.inner, s));
-      STACK_LAUNCH(24.0 * g.st, k_pair_sub<<<nb(g.st), 256, 0, s>>>(Sb, Slb, w.dS, w.dSl, (long long)g.st));
-      STACK_LAUNCH(24.0 * g.zt, k_pair_sub<<<nb(g.zt), 256, 0, s>>>(zb, zlb, w.dz, w.dzl, (long long)g.zt));
+      // eq. 17: B_r -= the slice's sum of T_l (its own contribution, from zero).  The
+      // state at the slice's end stays where it is, for the layer's backward; the
+      // tensor-core kernels' residuals are zero and not formed
+      float *Se = w.Se + r * g.st, *ze = w.ze + r * g.zt, *Sle = w.Sle + r * g.st, *zle = w.zle + r * g.zt;
+      float *Sb = w.Sb + r * g.st, *zb = w.zb + r * g.zt, *Slb = w.Slb + r * g.st, *zlb = w.zlb + r * g.zt;
+      ST_CALL(fwd_state(U, U, U, om, p.B, p.H, b, d, M, b, p.dtype, p.feature, w.dS, w.dz,
+                        path ? nullptr : w.dSl, path ? nullptr : w.dzl, w.inner, g.inner, s));
+      STACK_LAUNCH((path ? 20.0 : 24.0) * (g.st + g.zt),
+                   k_pair_sub<<<nb((long long)(g.st + g.zt) / 4), 256, 0, s>>>(
+                       PairSub{Se, Sle, w.dS, path ? nullptr : w.dSl, Sb, Slb, (long long)g.st / 4},
+                       PairSub{ze, zle, w.dz, path ? nullptr : w.dzl, zb, zlb, (long long)g.zt / 4}));
       ST_TRY(cudaGetLastError());
       // the layer's output on the slice from the rolled-back state
       T* Y = reinterpret_cast<T*>(w.yout[r]);
@@ -440,8 +463,17 @@ slim_status bwd_impl(const Problem& p, int layers, const T* x, const float* omeg
     }
     // dout now holds dX^(0) of the slice, rounded to the dtype
     ST_TRY(scatter(w.dout, dx, g, p.L, d, a, b, s));
-    float* t = G; G = G2; G2 = t;
-    t = gz; gz = gz2; gz2 = t;
+    auto swap = [](float*& x, float*& y) {
+      float* t = x;
+      x = y;
+      y = t;
+    };
+    swap(G, G2);
+    swap(gz, gz2);
+    swap(w.Sb, w.Se);
+    swap(w.zb, w.ze);
+    swap(w.Slb, w.Sle);
+    swap(w.zlb, w.zle);
   }
   return SLIM_OK;
 }

@@ -469,6 +469,7 @@ __device__ __forceinline__ void role_fwd(const FwdJob& J, int pos, int c, uint8_
   float* own = J.slot + ((size_t)c * J.nt + t) * C::E;
   int* oflag = J.flag + ((size_t)c * J.nt + t) * FLAG_STRIDE;
   const bool last = pos == J.P - 1;
+  const bool state_only = J.out == nullptr;  // the chain alone: no g(Q), scores or readout
   const int tid = threadIdx.x, warp = tid >> 5;
   const int row = 32 * (warp & 3) + (tid & 31);
   const int cg = warp >> 2;
@@ -485,8 +486,8 @@ __device__ __forceinline__ void role_fwd(const FwdJob& J, int pos, int c, uint8_
   if (tid == 0) {
     // the three row tiles by TMA (rows past the chain's end read as zero)
     const uint32_t bar = smem_u32(&mb[MB_TILES]);
-    mbar_expect_tx(bar, 3 * ROWT);
-    tma_load_3d(smem_u32(sQ), &J.tq, row0, c, bar);
+    mbar_expect_tx(bar, (state_only ? 2 : 3) * ROWT);
+    if (!state_only) tma_load_3d(smem_u32(sQ), &J.tq, row0, c, bar);
     tma_load_3d(smem_u32(sK), &J.tk, row0, c, bar);
     tma_load_3d(smem_u32(sV), &J.tv, row0, c, bar);
   }
@@ -507,10 +508,10 @@ __device__ __forceinline__ void role_fwd(const FwdJob& J, int pos, int c, uint8_
   {
     const bool rv = row < valid;
     float* redN = reinterpret_cast<float*>(sPhiQ);  // 4 KB scratch below Omega lo
-    redN[cg * T + row] = row_norm2_part(sQ, row, cg);
+    if (!state_only) redN[cg * T + row] = row_norm2_part(sQ, row, cg);
     redN[(NG + cg) * T + row] = row_norm2_part(sK, row, cg);
     publish();
-    const float q2 = group_total(redN, row), k2 = group_total(redN + NG * T, row);
+    const float q2 = state_only ? 0.f : group_total(redN, row), k2 = group_total(redN + NG * T, row);
     const uint32_t tmem = tmem_base;
     const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
     if (tid == 0) {
@@ -522,11 +523,13 @@ __device__ __forceinline__ void role_fwd(const FwdJob& J, int pos, int c, uint8_
         mma(tmem + 256, kmaj(aK, T, k0), kmaj(aOl, MF, k0), idesc_bf16(T, MF, 0, 0), 1);
       }
       mma_commit(smem_u32(&mb[0]));
-      for (int k0 = 0; k0 < D; k0 += 16) {
-        mma(tmem, kmaj(aQ, T, k0), kmaj(aOm, MF, k0), idesc_bf16(T, MF, 0, 0), k0 > 0);
-        mma(tmem, kmaj(aQ, T, k0), kmaj(aOl, MF, k0), idesc_bf16(T, MF, 0, 0), 1);
+      if (!state_only) {
+        for (int k0 = 0; k0 < D; k0 += 16) {
+          mma(tmem, kmaj(aQ, T, k0), kmaj(aOm, MF, k0), idesc_bf16(T, MF, 0, 0), k0 > 0);
+          mma(tmem, kmaj(aQ, T, k0), kmaj(aOl, MF, k0), idesc_bf16(T, MF, 0, 0), 1);
+        }
+        mma_commit(smem_u32(&mb[1]));
       }
-      mma_commit(smem_u32(&mb[1]));
     }
     if (!mbar_wait(smem_u32(&mb[0]), 0, J.err)) abort_ = 1;
     tc_fence_after();
@@ -548,6 +551,7 @@ __device__ __forceinline__ void role_fwd(const FwdJob& J, int pos, int c, uint8_
     }
     if (warp < 8) {
       // ---- compute group: g(Q), A = tril(g(Q) g(K)^T), A's bf16 tile and row sums
+      if (state_only) goto join;
       if (!mbar_wait(smem_u32(&mb[1]), 0, J.err)) gfail[0] = 1;
       tc_fence_after();
       group_bar(1);
@@ -678,7 +682,7 @@ __device__ __forceinline__ void role_fwd(const FwdJob& J, int pos, int c, uint8_
     }
   join:
     __syncthreads();
-    if (gfail[0] | gfail[1]) goto teardown;
+    if ((gfail[0] | gfail[1]) || state_only) goto teardown;
     publish();
     // three issuing threads: the narrow products are issue-bound
     if (tid == 0) {
@@ -2095,8 +2099,9 @@ Slice slice_of(const Problem& p, const Geo& g, int n) {
 
 cudaError_t prepare(const Ws& w, const Geo& g, const float* omega, unsigned* rep,
                     cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(w.err, 0, sizeof(int), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(w.flags, 0, (size_t)w.nflags * sizeof(int), s);
+  // the error word and, right behind it, every flag and counter: one memset
+  const cudaError_t e = cudaMemsetAsync(
+      w.err, 0, (size_t)(reinterpret_cast<char*>(w.flags + w.nflags) - reinterpret_cast<char*>(w.err)), s);
   if (e != cudaSuccess) return e;
   prof::Scope ps(prof::K_TC_PREP, s);
   k_omega_bf16<<<nblk(g.MF * D), 256, 0, s>>>(omega, w.om16, g.MF * D, w.err, rep);  // hi and lo

@@ -15,6 +15,7 @@ int bwd_schedule(const Problem& p, int* items, int cap, int* ring);
 
 // report: the device address of the call's timeout-report counter, or null
 // (see report.h); the first kernel of the call stores it in the workspace.
+// out null: the state alone.
 slim_status fwd(const Problem& p, const void* q, const void* k, const void* v,
                 const float* omega, void* out, const StateOut& st, const StateInit& init,
                 unsigned* report, void* workspace, cudaStream_t s);
