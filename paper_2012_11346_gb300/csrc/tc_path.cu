@@ -373,7 +373,9 @@ __device__ __forceinline__ void group_publish(int id) {
   tc_fence_after();
 }
 // Bounded poll of a flag by one thread: returns once *flag == want (then an
-// acquire fence).  It gives up after kWaitLimitNs (or kWaitMaxPolls polls), or
+// acquire fence).  The first polls come back to back (each is an L2 round trip
+// anyway): a sleep between them is added to every hop of a chain (bench step
+// 739 -> 732 us without it).  It gives up after kWaitLimitNs (or kWaitMaxPolls polls), or
 // early once another CTA has reported an error (checked every 64 polls, so
 // that waiting CTAs do not all hammer the error word); a wait that gives up
 // records itself through give_up(err).
@@ -389,7 +391,7 @@ __device__ __forceinline__ bool flag_poll(const int* flag, int want, int* err) {
       if (i == 63) t0 = globaltimer_ns();
       else if (globaltimer_ns() - t0 > kWaitLimitNs) break;
     }
-    __nanosleep(i < 16 ? 32 : 256);
+    if (i >= 64) __nanosleep(64);
   }
   give_up(err);
   return false;
@@ -410,7 +412,7 @@ __device__ __forceinline__ bool flag_poll2(const int* f1, int w1, const int* f2,
       if (i == 63) t0 = globaltimer_ns();
       else if (globaltimer_ns() - t0 > kWaitLimitNs) break;
     }
-    __nanosleep(i < 16 ? 32 : 256);
+    if (i >= 64) __nanosleep(64);
   }
   give_up(err);
   return false;
@@ -432,7 +434,7 @@ __device__ __forceinline__ bool counter_poll(const int* ctr, int want, int* err)
       if (i == 63) t0 = globaltimer_ns();
       else if (globaltimer_ns() - t0 > kWaitLimitNs) break;
     }
-    __nanosleep(i < 16 ? 32 : 256);
+    if (i >= 64) __nanosleep(64);
   }
   give_up(err);
   return false;
@@ -631,6 +633,7 @@ __device__ __forceinline__ void role_fwd(const FwdJob& J, int pos, int c, uint8_
             pz[h] = __ldcg(J.init.z + e) + (J.init.z_lo ? __ldcg(J.init.z_lo + e) : 0.f);
         }
       }
+      // this tile's slot first: the next tile of the chain waits for it
 #pragma unroll
       for (int h = 0; h < C::MH; ++h) {
         const int m = 128 * h + row;
@@ -641,7 +644,6 @@ __device__ __forceinline__ void role_fwd(const FwdJob& J, int pos, int c, uint8_
 #pragma unroll
           for (int i = 0; i < 16; ++i) inc[i] += pv[h][j][i];
           st_lm16(own, h, cq + j, row, inc);
-          st_tile16(sS, MF, m, 16 * (cq + j), pv[h][j]);
           if (last) {
             st_f32x16(J.st.S + ((size_t)c * MF + m) * 64 + 16 * (cq + j), inc);
             if (J.st.S_lo) {
@@ -652,8 +654,6 @@ __device__ __forceinline__ void role_fwd(const FwdJob& J, int pos, int c, uint8_
           }
         }
       }
-      // z_t as the first two rows (hi, lo in bf16) of a K-major [16][MF]
-      // operand, so that g(Q) z_t is a tensor-core product with ~16-bit z
       if (cq == 0) {
 #pragma unroll
         for (int h = 0; h < C::MH; ++h) {
@@ -661,24 +661,36 @@ __device__ __forceinline__ void role_fwd(const FwdJob& J, int pos, int c, uint8_
           float dz;
           tmem_ld1(trow + 384 + 16 * h, dz);
           __stcg(own + MF * 64 + m, pz[h] + dz);
-          const __nv_bfloat16 zh = __float2bfloat16_rn(pz[h]);
-          *reinterpret_cast<__nv_bfloat16*>(sZt + tile_off(16, 0, m)) = zh;
-          *reinterpret_cast<__nv_bfloat16*>(sZt + tile_off(16, 1, m)) =
-              __float2bfloat16_rn(pz[h] - __bfloat162float(zh));
           if (last) {
             J.st.z[(size_t)c * MF + m] = pz[h] + dz;
             if (J.st.z_lo) J.st.z_lo[(size_t)c * MF + m] = 0.f;
           }
         }
+      }
+      group_bar(2);  // every slot write of the group is issued
+      if (gl == 0) st_release_gpu(oflag, n + 1);
+      // then S_t as the readout's operand, and z_t as the first two rows (hi, lo in
+      // bf16) of a K-major [16][MF] operand, so that g(Q) z_t is a tensor-core
+      // product with ~16-bit z (rows 2..15 are zero; the ones tile was there)
+#pragma unroll
+      for (int h = 0; h < C::MH; ++h)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) st_tile16(sS, MF, 128 * h + row, 16 * (cq + j), pv[h][j]);
+      if (cq == 0) {
+#pragma unroll
+        for (int h = 0; h < C::MH; ++h) {
+          const int m = 128 * h + row;
+          const __nv_bfloat16 zh = __float2bfloat16_rn(pz[h]);
+          *reinterpret_cast<__nv_bfloat16*>(sZt + tile_off(16, 0, m)) = zh;
+          *reinterpret_cast<__nv_bfloat16*>(sZt + tile_off(16, 1, m)) =
+              __float2bfloat16_rn(pz[h] - __bfloat162float(zh));
+        }
       } else {
-        // rows 2..15 of the z operand are zero (the ones tile was there)
         for (int e = gl - 128; e < 14 * MF / 8; e += 128) {
           const int r16 = 2 + e / (MF / 8), k = (e % (MF / 8)) * 8;
           st_chunk(sZt, 16, r16, k, make_uint4(0u, 0u, 0u, 0u));
         }
       }
-      group_bar(2);  // every slot write of the group is issued
-      if (gl == 0) st_release_gpu(oflag, n + 1);
     }
   join:
     __syncthreads();
@@ -1030,7 +1042,6 @@ __device__ __forceinline__ void role_bwd_q(const BwdQJob& J, int b, uint8_t* sme
       if (gfail[1]) goto join1;
 #pragma unroll
       for (int h = 0; h < C::MH; ++h) {
-        const int m = 128 * h + row;
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           float d[16];
@@ -1038,7 +1049,6 @@ __device__ __forceinline__ void role_bwd_q(const BwdQJob& J, int b, uint8_t* sme
 #pragma unroll
           for (int i = 0; i < 16; ++i) sv[h][j][i] -= d[i];
           st_lm16(own1, h, cq + j, row, sv[h][j]);
-          st_tile16(sS, MF, m, 16 * (cq + j), sv[h][j]);
         }
       }
       if (cq == 0) {
@@ -1058,6 +1068,11 @@ __device__ __forceinline__ void role_bwd_q(const BwdQJob& J, int b, uint8_t* sme
       if (linked && snext != t) discard_l2(s1.S, (size_t)C::E * 4, gl, GRP);
       group_bar(2);  // every slot write of the group is issued
       if (gl == 0) st_release_gpu(of1, n + 1);
+      // the slot released, this tile's own copy of the state
+#pragma unroll
+      for (int h = 0; h < C::MH; ++h)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) st_tile16(sS, MF, 128 * h + row, 16 * (cq + j), sv[h][j]);
     }
   join1:
     __syncthreads();
@@ -1244,14 +1259,13 @@ __device__ __forceinline__ void role_bwd_q(const BwdQJob& J, int b, uint8_t* sme
       for (int h = 0; h < C::MH; ++h) {
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-          st_lm16_bf16(J.gS + tf * MF * 64, h, cq + j, row, gs[h][j]);  // G_t(S), dk/dv side
           float gd[16];
           tmem_ld16(trow + 64 * h + 16 * (cq + j), gd);
 #pragma unroll
-          for (int i = 0; i < 16; ++i) gs[h][j][i] += gd[i];
-          st_lm16(own2, h, cq + j, row, gs[h][j]);
+          for (int i = 0; i < 16; ++i) gd[i] += gs[h][j][i];
+          st_lm16(own2, h, cq + j, row, gd);
           if (seq_first)
-            st_f32x16(J.gio.S_out + ((size_t)c * MF + 128 * h + row) * 64 + 16 * (cq + j), gs[h][j]);
+            st_f32x16(J.gio.S_out + ((size_t)c * MF + 128 * h + row) * 64 + 16 * (cq + j), gd);
         }
       }
       if (cq == 0) {
@@ -1260,7 +1274,6 @@ __device__ __forceinline__ void role_bwd_q(const BwdQJob& J, int b, uint8_t* sme
           const int m = 128 * h + row;
           float gdz;
           tmem_ld1(trow + 128 + 16 * h, gdz);
-          J.gz[tf * MF + m] = gzs[h];
           __stcg(own2 + MF * 64 + m, gzs[h] + gdz);
           if (seq_first) J.gio.z_out[(size_t)c * MF + m] = gzs[h] + gdz;
         }
@@ -1268,6 +1281,13 @@ __device__ __forceinline__ void role_bwd_q(const BwdQJob& J, int b, uint8_t* sme
       if (linked && snext != t) discard_l2(s2.S, (size_t)C::E * 4, gl, GRP);
       group_bar(2);  // every slot write of the group is issued
       if (gl == 0) st_release_gpu(of2, n + 1);
+      // the slot released, G_t for the dk/dv part
+#pragma unroll
+      for (int h = 0; h < C::MH; ++h) {
+#pragma unroll
+        for (int j = 0; j < 2; ++j) st_lm16_bf16(J.gS + tf * MF * 64, h, cq + j, row, gs[h][j]);
+        if (cq == 0) J.gz[tf * MF + 128 * h + row] = gzs[h];
+      }
     }
   join2:
     __syncthreads();
