@@ -78,8 +78,6 @@ __global__ void __launch_bounds__(256) k_carry(const __grid_constant__ CarryArgs
     T v;
     float f[V];
   };
-  pdl_wait();
-  pdl_launch();
   const int SV = A.M * A.d / V, EV = SV + A.M / V, mode = A.mode;
   const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= (long long)A.chains * EV) return;
@@ -91,13 +89,15 @@ __global__ void __launch_bounds__(256) k_carry(const __grid_constant__ CarryArgs
   T* lo_p = reinterpret_cast<T*>(A.lo);
   Reg hi{}, lo{};
   if (!A.first) {
-    hi.v = hi_p[idx];
-    lo.v = lo_p[idx];
+    hi.v = __ldcg(hi_p + idx);
+    lo.v = __ldcg(lo_p + idx);
   } else if (A.init.S) {
     hi.v = reinterpret_cast<const T*>(in_s ? A.init.S : A.init.z)[so];
     const float* il = in_s ? A.init.S_lo : A.init.z_lo;
     if (il) lo.v = reinterpret_cast<const T*>(il)[so];
   }
+  pdl_wait();  // the totals; the carried state is older
+  pdl_launch();
   const bool rev = mode == CARRY_GREV || mode == CARRY_ROLLBACK;
   // frame i's place in buf
   const size_t fs = (size_t)(PAIR ? 2 : 1) * EV;

@@ -275,19 +275,20 @@ __global__ void __launch_bounds__(kThreads, (DeltaSmem<IO, D>::ctas)) k_delta(co
   bf16* Ph = Vs + S::v / 2;
   float* norm2 = reinterpret_cast<float*>(Ph + S::ph / 2);
   float* zt = norm2 + kTile;  // [tile][64]
-  pdl_wait();
-  pdl_launch();
   const int frame = blockIdx.x;
   const Frame f = frame_pos(A, frame);
   const bool square = A.feature == SLIM_FEAT_SQUARE;
-  if (!square) {
-    stage_omega<D, 64>(om, A.om_t, 0);
-    cp_commit();
-  }
+  // the caller's rows before the kernel ahead is waited for (see launch_pdl)
   load_rows_fp<IO, D>(A, f, static_cast<const IO*>(A.k) + f.row0 * D, xs);
   load_rows<IO, D>(A, f, static_cast<const IO*>(A.v) + f.row0 * D, Vs, nullptr);
   __syncthreads();
   row_norms<D>(xs, norm2);
+  pdl_wait();
+  pdl_launch();
+  if (!square) {
+    stage_omega<D, 64>(om, A.om_t, 0);
+    cp_commit();
+  }
 
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32, g = lane >> 2, t = lane & 3;
   const int fb = warp & 3, h = warp >> 2;  // 16 features of the chunk, half of the columns
@@ -514,8 +515,6 @@ __global__ void __launch_bounds__(kThreads, D <= 64 ? 2 : 1)
   float* norm2 = zs + 64;
   float* den_s = norm2 + kTile;
   bf16* Vs = reinterpret_cast<bf16*>(xs);
-  pdl_wait();
-  pdl_launch();
   const int frame = blockIdx.x;
   const Frame f = frame_pos(A, frame);
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32, g = lane >> 2, t = lane & 3;
@@ -538,12 +537,15 @@ __global__ void __launch_bounds__(kThreads, D <= 64 ? 2 : 1)
     if (!square) stage_omega<D, 64>(om, A.om_t, c0);
     cp_commit();
   };
+  // all but the state comes from the caller or from kernels before the one ahead
   stage_om(0);
   stage_keys(0);
-  pc.load(Pt, min(64, A.M));
   load_rows_fp<IO, D>(A, f, static_cast<const IO*>(A.q) + f.row0 * D, xs);
   __syncthreads();
   row_norms<D>(xs, norm2);
+  pdl_wait();
+  pdl_launch();
+  pc.load(Pt, min(64, A.M));
   pc.template store<NS>(Ps, min(64, A.M));
 
   float num[NB][4] = {}, sc[4][4] = {}, dz[4] = {}, de = 0.f;
@@ -724,8 +726,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
   float* zs = reinterpret_cast<float*>(Vs + S::v / 2);  // [tile][64]: z (d >= 64: rounded to the pieces)
   float* norm2 = zs + 4 * 64;
   float* den_s = norm2 + kTile;
-  pdl_wait();
-  pdl_launch();
   const int frame = blockIdx.x;
   const Frame f = frame_pos(A, frame);
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32, g = lane >> 2, t = lane & 3;
@@ -757,6 +757,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
   load_rows<IO, D>(A, f, static_cast<const IO*>(A.v) + f.row0 * D, Vs, nullptr);
   __syncthreads();
   row_norms<D>(xs, norm2);
+  pdl_wait();  // the state; the rest is older
+  pdl_launch();
 
   float num[GN][4][2][4] = {}, sc[GA][KB][4] = {}, dz[4][4] = {}, de[4] = {};
   const int dr = warp == 4 ? lane : warp == 5 ? 32 + lane : -1;  // den's rows (d >= 64)
@@ -1258,8 +1260,6 @@ __global__ void __launch_bounds__(kThreads, (bwd_occupancy<IO, D>()))
   const bool square = A.feature == SLIM_FEAT_SQUARE;
   const size_t MD = (size_t)A.M * D;
   float* slot = A.slots + (size_t)blockIdx.x * MD;
-  pdl_wait();
-  pdl_launch();
 
   for (int tile = blockIdx.x; tile < A.chains * A.nf; tile += gridDim.x) {
     const Frame tp = frame_pos(A, tile);
@@ -1322,6 +1322,8 @@ __global__ void __launch_bounds__(kThreads, (bwd_occupancy<IO, D>()))
       row_norms<D>(xf, dn + kTile);
       __syncthreads();
     }
+    pdl_wait();  // the state; all staged so far is older (a no-op after the first frame)
+    pdl_launch();
 
     // pass 1: g(Q), A, den
     float den0 = 0.f, den1 = 0.f;
@@ -1633,8 +1635,6 @@ __global__ void __launch_bounds__(kThreads, (bwd_occupancy<IO, D>()))
   const bool square = A.feature == SLIM_FEAT_SQUARE;
   const size_t MD = (size_t)A.M * D;
   float* slot = A.slots + (size_t)blockIdx.x * MD;
-  pdl_wait();
-  pdl_launch();
 
   for (int tile = blockIdx.x; tile < A.chains * A.nf; tile += gridDim.x) {
     const Frame tp = frame_pos(A, tile);
@@ -1655,13 +1655,15 @@ __global__ void __launch_bounds__(kThreads, (bwd_occupancy<IO, D>()))
         stage_rows<NS>(Qs, kTile * kPT, kPT, pq + c0, (size_t)kTile * A.M, A.M, kTile, nf);
       if (F::FP && !square) stage_omega<D, kChunk>(omf, A.om_t, c0);
       cp_commit();
-      gc.load(Gt + (size_t)c0 * D, nf);
     };
     if (A.causal) stage_rows<NS>(dAs, kTile * PK, PK, sdA, kTile * kTile, kTile, kTile, kTile);
     stage(0);
     load_rows<IO, D>(A, tp, kg, Ks, hx);
     if (F::FP) load_rows_fp<IO, D>(A, tp, kg, xf);
     load_rows<IO, D>(A, tp, static_cast<const IO*>(A.v) + tp.row0 * D, Vs, nullptr);
+    pdl_wait();  // the state gradient; all staged so far is older
+    pdl_launch();
+    gc.load(Gt, min(kChunk, A.M));
     gc.template store<NS>(Gs, min(kChunk, A.M));
     cp_wait<0>();
     __syncthreads();
@@ -1733,7 +1735,10 @@ __global__ void __launch_bounds__(kThreads, (bwd_occupancy<IO, D>()))
       }
       __syncthreads();
       const bool more = c0 + kChunk < A.M;
-      if (more) stage(c0 + kChunk);
+      if (more) {
+        stage(c0 + kChunk);
+        gc.load(Gt + (size_t)(c0 + kChunk) * D, min(kChunk, A.M - c0 - kChunk));
+      }
       if (!square) {
         for (int u = warp; u < 2 * KD; u += kThreads / 32) {  // 16 features x 16 columns
           const int mb = u & 1, n16 = u >> 1;

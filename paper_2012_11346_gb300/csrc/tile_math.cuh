@@ -132,7 +132,12 @@ __device__ __forceinline__ void store2(float* p, float x, float y) {
   *reinterpret_cast<float2*>(p) = make_float2(x, y);
 }
 
-// A launch as a programmatic dependent of the kernel before it in the stream.
+// A launch as a programmatic dependent of the kernel before it in the stream: its
+// CTAs may start once every CTA of that kernel has called pdl_launch.  Every kernel
+// of a launch sequence calls pdl_wait before pdl_launch, so when a kernel starts, all
+// but the one directly ahead of it have completed: before its own pdl_wait it reads
+// the caller's tensors and what older kernels left (never the kernel ahead's output),
+// and writes shared memory only.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem,
                        cudaStream_t s, Args... args) {
