@@ -409,9 +409,14 @@ slim_status slim_diag_wait_timeout(void* workspace, void* stream);
  *     reserves the array: the first libslim call that reaches a device does
  *     it.  Make a first call on each device at start-up, outside any context
  *     that must not allocate (and before any stream capture on the device).
- *   - Returns SLIM_ERR_WORKSPACE when the problem needs more scratch than
- *     SLIM_NOALLOC_SCRATCH_BYTES (compare slim_fwd_workspace_size); use
- *     slim_fwd with a caller workspace, or a smaller C or B*H, then.
+ *   - Returns SLIM_ERR_WORKSPACE for problems beyond SLIM_NOALLOC_SCRATCH_BYTES:
+ *     those whose slim_fwd_workspace_size exceeds it on the tensor-core kernels;
+ *     on the fp32-compute kernels those with
+ *       4*B*H*((T + 2)*M*(d + 1) + R*(4*d + 2*M + 2 + R/T)) bytes
+ *     above it (R rows of a slice in T tiles of 64; of up to 1024 rows in tiles
+ *     of C when C is 16, 32 or 48).  slim_fwd_workspace_size may be larger there:
+ *     the sweep then takes fewer rows and chains at a time, with the same results.
+ *     Use slim_fwd with a caller workspace, or a smaller C or B*H, beyond it.
  *   - The first call on a device looks up the array's device address
  *     (cudaGetSymbolAddress) with that device current.
  *   - All calls share the one array and it keeps the last call's contents;

@@ -21,8 +21,8 @@ slim_status fwd_unreported(const void* q, const void* k, const void* v, const fl
                            slim_feature feature, void* out, float* S_state, float* z_state,
                            float* S_state_lo, float* z_state_lo, void* workspace,
                            size_t workspace_bytes, cudaStream_t stream);
-slim_status fwd_least_workspace(int B, int H, int L, int d, int M, int C, slim_dtype dtype,
-                                slim_feature feature, size_t* bytes);
+slim_status fwd_noalloc_bytes(int B, int H, int L, int d, int M, int C, slim_dtype dtype,
+                              slim_feature feature, size_t* bytes);
 }
 
 namespace {
@@ -65,7 +65,7 @@ extern "C" slim_status slim_fwd_noalloc(const void* q, const void* k, const void
   if (feature != SLIM_FEAT_EXP && feature != SLIM_FEAT_RELU && feature != SLIM_FEAT_SQUARE)
     return SLIM_ERR_INVALID_ARG;
   size_t need = 0;
-  slim_status st = slim::fwd_least_workspace(B, H, L, d, M, C, dtype, feature, &need);
+  slim_status st = slim::fwd_noalloc_bytes(B, H, L, d, M, C, dtype, feature, &need);
   if (st != SLIM_OK) return st;
   if (need > (size_t)SLIM_NOALLOC_SCRATCH_BYTES) return SLIM_ERR_WORKSPACE;  // too large here
   void* scratch = nullptr;

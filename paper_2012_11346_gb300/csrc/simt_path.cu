@@ -379,6 +379,25 @@ size_t workspace_bytes(const Problem& p, bool bwd, bool small) {
   return cv.bytes();
 }
 
+size_t noalloc_bytes(const Problem& p) {
+  const size_t n = p.chains(), M = p.M, d = p.d, dp = p.d + 1;
+  const int Cs = p.slice_len();
+  long long rows = Cs;
+  int tile = Cs >= 64 ? 64 : Cs > 0 ? (Cs + 15) / 16 * 16 : 16;
+  if (Cs < 64 && Cs % 16 == 0 && p.L > Cs) {
+    tile = Cs;
+    const long long whole = ((long long)p.L + tile - 1) / tile * tile, most = 1024 / tile * tile;
+    rows = most < whole ? most : whole;
+  }
+  const size_t nt = (size_t)((rows + tile - 1) / tile), R = n * nt * tile;
+  Carver cv(nullptr);
+  cv.take<int>(64);
+  for (size_t count : {n * M * dp, n * M * dp, R * d, R * d, R * dp, R * M, R * M, n * nt * M * dp,
+                       R * tile, R * dp, (M + 127) / 128 * 128 * d, M})
+    cv.take<float>(count);
+  return cv.bytes();
+}
+
 // With less workspace than workspace_bytes asks for, the fewest rows per
 // sequence, and as many chains at a time as fit.
 slim_status fwd(const Problem& p, const void* q_ptr, const void* k, const void* v,

@@ -9,6 +9,13 @@ namespace simt {
 // on, and sweeps fewer rows and chains at a time below the full size)
 size_t workspace_bytes(const Problem& p, bool bwd, bool small = false);
 
+// What slim_fwd_noalloc's limit counts: a call's state and the rows of one slice
+// (of 1024 rows of shorter slices) with their features and tile totals in fp32.
+// This is the size of the problem, not of the scratch: the limit stays where it is
+// when the layout of the scratch changes.  fwd runs in less for every problem
+// within SLIM_NOALLOC_SCRATCH_BYTES.
+size_t noalloc_bytes(const Problem& p);
+
 // out null: the state alone
 slim_status fwd(const Problem& p, const void* q, const void* k, const void* v,
                 const float* omega, void* out, const StateOut& st, const StateInit& init,

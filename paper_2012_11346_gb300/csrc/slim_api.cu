@@ -172,14 +172,16 @@ slim_status backward(const void* q, const void* k, const void* v, const float* o
 }  // namespace
 
 namespace slim {
-// The least workspace the forward runs in (slim_fwd_workspace_size, or less
-// where that asks for more rows per launch sequence than it must).
-slim_status fwd_least_workspace(int B, int H, int L, int d, int M, int C, slim_dtype dtype,
-                                slim_feature feature, size_t* bytes) {
+// The bytes that slim_fwd_noalloc holds against its scratch: the tensor-core path's
+// workspace, or the fp32-compute path's limit (its forward sweeps fewer rows and
+// chains at a time in a scratch below slim_fwd_workspace_size).
+slim_status fwd_noalloc_bytes(int B, int H, int L, int d, int M, int C, slim_dtype dtype,
+                              slim_feature feature, size_t* bytes) {
   Problem p;
   slim_status st = check_problem(B, H, L, d, M, C, dtype, feature, &p);
   if (st != SLIM_OK) return st;
-  *bytes = ws_bytes(p, false, true);
+  const size_t least = ws_bytes(p, false, true), limit = use_tc(p) ? 0 : slim::simt::noalloc_bytes(p);
+  *bytes = least > limit ? least : limit;
   return SLIM_OK;
 }
 

@@ -43,7 +43,8 @@ def test_tile_edges(cuda_device, B, L, d, M, C, dtype, feature):
 
 def test_noalloc_sweeps_chains_in_batches(cuda_device):
     """A forward whose full workspace exceeds slim_fwd_noalloc's scratch runs on
-    fewer rows and chains at a time: the same bits as slim_fwd."""
+    fewer rows and chains at a time: the same bits as slim_fwd.  The problem size
+    that it refuses does not follow the scratch's layout."""
     w = W.Workload("batches", 60, 1, 200, 64, 256, 7, "f32", "exp", "normal", "iid", seed=32)
     x = W.make_inputs(w, device=cuda_device)
     assert slim.workspace_size(60, 1, 200, 64, 256, 7, torch.float32, "exp", False) > 16 << 20
@@ -57,6 +58,14 @@ def test_noalloc_sweeps_chains_in_batches(cuda_device):
     torch.cuda.synchronize()
     for a, b in zip(got, ref):
         assert torch.equal(a, b)
+    # 4 B ((1 + 2) 256 65 + 16 (4 64 + 2 256 + 2 + 16)) bytes: 16.4 MiB at B = 69
+    z = [torch.zeros(69, 1, 200, 64, device=cuda_device) for _ in range(4)]
+    S, zs = torch.zeros(69, 1, 256, 64, device=cuda_device), torch.zeros(69, 1, 256, device=cuda_device)
+    st = slim.library().slim_fwd_noalloc(
+        z[0].data_ptr(), z[1].data_ptr(), z[2].data_ptr(), x["omega"].data_ptr(), 69, 1, w.L, w.d, w.M,
+        w.C, slim.DTYPES[torch.float32], slim.FEATURES[w.feature], z[3].data_ptr(), S.data_ptr(),
+        zs.data_ptr(), None, None, ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert st == 3  # SLIM_ERR_WORKSPACE
 
 
 SHORT = [
