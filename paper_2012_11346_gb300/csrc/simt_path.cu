@@ -35,6 +35,8 @@
 // this file cuts the rows into sequences and carves the workspace.
 #include <math.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "simt_path.h"
 #include "simt_short.h"
@@ -53,8 +55,16 @@ namespace {
 // A launch sequence covers `rows` rows of every chain in tiles of 64, or of the
 // whole slice when it is shorter: the state is formed at every slice boundary
 // (eq. 16), and a tile's rows are padded to a multiple of 16.  A sequence is a
-// slice, or several where one leaves the chip idle.
-constexpr int kSeqFrames = 304;  // frames that fill the chip: two CTAs on each of 152 SMs
+// slice, or several: as many as fill the chip (kSeqFrames), and beyond that up to
+// kSeqSlices within kMostFrames, because a launch of few waves (1 to 3 CTAs on an SM)
+// loses much of its last one.  Train steps at 304 / 1216 / 2432 frames: [4,12,8192]
+// fp32 relu, C = 512 (384 frames a slice) 6.43 / 5.46 / 5.36 ms; non-causal [8,8,4096]
+// bf16, C = 1024 (1024 frames) 2.52 / 2.52 / 2.28 ms; L = 65536, C = 16 9.17 / 8.95 /
+// 9.08 ms: short slices gain nothing from more, and the scratch stays in proportion to
+// C where C is small (200 KB to 600 KB a frame).
+constexpr int kSeqFrames = 2 * kSms;  // two CTAs on each SM
+constexpr int kMostFrames = 16 * kSms;
+constexpr int kSeqSlices = 8;
 constexpr int kShortRows = 1024; // rows per chain of a sequence of slices below 64 rows, about
 
 struct Seq {
@@ -85,14 +95,18 @@ Seq sequence(const Problem& p, int chains, bool small) {
   q.pitch = Cs < kTile ? (Cs > 0 ? Cs : 1) : kTile;
   q.tile = (q.pitch + 15) / 16 * 16;
   q.per = q.tile <= 32 ? kTile / q.tile : 1;
-  const long long fill = kSeqFrames / chains;  // frames per chain
+  const long long fill = kSeqFrames / chains, most = kMostFrames / chains;  // frames per chain
   long long rows = Cs;
   if (Cs < kTile) {
     const long long frame = (long long)q.per * q.pitch, least = (kShortRows + frame - 1) / frame;
     rows = frame * (small ? 1 : (fill > least ? fill : least));
   } else if (!small) {
-    const long long slices = fill / ((Cs + kTile - 1) / kTile);
-    if (slices > 1) rows = slices * Cs;
+    const long long per_slice = (Cs + kTile - 1) / kTile, more = most / per_slice;
+    const long long slices = std::max(fill / per_slice, std::min<long long>(more, kSeqSlices));
+    if (slices > 1) {  // evenly: the same number of sequences, without a small last one
+      const long long all = ((long long)p.L + Cs - 1) / Cs, seqs = (all + slices - 1) / slices;
+      rows = (all + seqs - 1) / seqs * Cs;
+    }
   }
   q.rows = (int)(rows < p.L ? rows : p.L);
   q.slice = Cs < kTile ? q.pitch : Cs;
@@ -100,8 +114,8 @@ Seq sequence(const Problem& p, int chains, bool small) {
   q.nf = (q.nt + q.per - 1) / q.per;
   q.N = p.L == 0 ? 0 : (p.L + q.rows - 1) / q.rows;
   const long long frames = (long long)q.chains * q.nf;
-  const int most = tile_kernels(p.dtype, p.d).slots;
-  q.slots = (int)(frames < most ? frames : most);
+  const int ctas = tile_kernels(p.dtype, p.d).slots;
+  q.slots = (int)(frames < ctas ? frames : ctas);
   return q;
 }
 
