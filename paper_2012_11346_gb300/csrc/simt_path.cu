@@ -3,7 +3,7 @@
 // problems) or 3 (fp32 problems) bf16 pieces of fp32 values where they are
 // operands of a product; products run as warp MMAs over the pieces.
 //
-// Rows are cut into tiles of 64 and every step is a batch over (chain, tile) --
+// Rows are cut into tiles of up to 64 and every step is a batch over (chain, tile) --
 // App. B's "block" evaluation with the block's prefix sums written as masked
 // matrix products:
 //

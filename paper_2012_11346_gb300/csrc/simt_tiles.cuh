@@ -1,6 +1,7 @@
 // Tile kernels of the fp32-compute path.
 //
-// A tile is 64 rows of one chain.  Operands are split once into bf16 pieces
+// A frame is 64 rows of one chain: one tile of 64 or 48 rows, or two or four tiles
+// of short slices.  Operands are split once into bf16 pieces
 // (NX for a caller's rows: 1 for bf16, 3 for fp32; NS for everything computed:
 // 2 for bf16 problems, 3 for fp32 ones) when they enter shared memory or become
 // an MMA fragment, and every product of a tile stays in the CTA: nothing but
@@ -10,7 +11,13 @@
 // an accumulator that already sits in registers becomes the next product's
 // operand without a trip through shared memory.  m16n8k16 bf16 measured 600
 // TFLOP/s on a GB300 (1.86 PFLOP/s for tcgen05), with 3 (bf16) or 6 (fp32)
-// piece products per product: that rate bounds these kernels.
+// piece products per product.
+//
+// Measured, train steps on a GB300, one batched contraction per launch (33 launches
+// per slice, every intermediate through memory) against these kernels: [4,12,8192]
+// fp32 relu, d = 64, M = 128, C = 512 10.17 -> 5.40 ms; non-causal [8,8,4096] bf16, d = 64,
+// M = 256 5.97 -> 2.28 ms; [1,4,65536] bf16, d = 128, M = 256, C = 16 30.05 -> 9.18 ms;
+// [1,1,256] fp32, d = 16, M = 32 843 -> 50 us.
 #pragma once
 #include "simt_tiles.h"
 #include "tile_math.cuh"
