@@ -465,16 +465,29 @@ struct StateChunk {
       if (e < rows * (D / 8)) load8(S + (size_t)e * 8, v[i]);
     }
   }
-  template <int NP>
+  // SWZ: rows of D elements without padding, their 16-byte chunks swizzled by the row
+  template <int NP, bool SWZ = false>
   __device__ __forceinline__ void store(bf16* dst, int rows) const {
+    constexpr int P = SWZ ? D : D + 8;
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      const int e = threadIdx.x + i * kThreads;
-      if (e < rows * (D / 8))
-        store_pieces8<NP>(dst + (e / (D / 8)) * (D + 8) + (e % (D / 8)) * 8, R * (D + 8), v[i]);
+      const int e = threadIdx.x + i * kThreads, r = e / (D / 8), c = e % (D / 8);
+      if (e < rows * (D / 8)) store_pieces8<NP>(dst + r * P + (SWZ ? c ^ (r & 7) : c) * 8, R * P, v[i]);
     }
   }
 };
+// ld_bt of 64 rows that StateChunk stored
+template <int NP, int D, bool SWZ>
+__device__ __forceinline__ void ld_state(uint32_t (&b)[NP][4], const bf16* p, int n0, int k0) {
+  if (!SWZ) {
+    ld_bt<NP>(b, p, 64 * (D + 8), D + 8, n0, k0);
+    return;
+  }
+  const int l = threadIdx.x & 31, r = k0 + (l & 15), c = n0 / 8 + (l >> 4);
+  p += r * D + (c ^ (r & 7)) * 8;
+#pragma unroll
+  for (int i = 0; i < NP; ++i) ldsm4t(b[i], p + i * 64 * D);
+}
 
 // `rows` rows of W bf16 (W % 8 == 0) in NP pieces, global row pitch gp and piece
 // stride gs, to shared memory (pitch sp, piece stride ss), asynchronously.
@@ -498,9 +511,12 @@ __device__ __forceinline__ void stage_rows(bf16* dst, int ss, int sp, const bf16
 template <typename IO, int D>
 struct OutSmem {
   static constexpr int NX = Pieces<IO>::NX, NS = Pieces<IO>::NS, PD = D + 8;
+  // d = 64 in fp32: a padded state chunk would leave room for one CTA on an SM
+  static constexpr bool SWZ = D == 64 && NX == 3;
   static constexpr int xs = kTile * fp_pitch<D>() * 4, om = D * 64 * 4, ph = NS * 64 * kPF * 2,
-                       ps = NS * 64 * PD * 2, zs = 64 * 4;
+                       ps = NS * 64 * (SWZ ? D : PD) * 2, zs = 64 * 4;
   static constexpr int bytes = xs + om + 2 * ph + ps + zs + 2 * kTile * 4;
+  static_assert(D > 64 || 2 * (bytes + 1024) <= 233472, "two CTAs on an SM");
   static_assert(NX * kTile * PD * 2 <= xs + om, "V in the projections' buffers");
   static_assert(bytes <= kSmemMax, "shared memory");
 };
@@ -553,7 +569,7 @@ __global__ void __launch_bounds__(kThreads, D <= 64 ? 2 : 1)
   pdl_wait();
   pdl_launch();
   pc.load(Pt, min(64, A.M));
-  pc.template store<NS>(Ps, min(64, A.M));
+  pc.template store<NS, S::SWZ>(Ps, min(64, A.M));
 
   float num[NB][4] = {}, sc[4][4] = {}, dz[4] = {}, de = 0.f;
   // the warps with the fewest scores sum den for d >= 64, a row per lane
@@ -578,7 +594,7 @@ __global__ void __launch_bounds__(kThreads, D <= 64 ? 2 : 1)
 #pragma unroll
         for (int nb = 0; nb < NB / 2; ++nb) {
           uint32_t b[NS][4];
-          ld_bt<NS>(b, Ps, 64 * PD, PD, cb + 16 * nb, 16 * i);
+          ld_state<NS, D, S::SWZ>(b, Ps, cb + 16 * nb, 16 * i);
           mma_pieces<NS, NS>(num[2 * nb], num[2 * nb + 1], a, b);
         }
       }
@@ -616,7 +632,7 @@ __global__ void __launch_bounds__(kThreads, D <= 64 ? 2 : 1)
     __syncthreads();
     if (more) {
       stage_keys(c0 + 64);
-      pc.template store<NS>(Ps, min(64, A.M - c0 - 64));
+      pc.template store<NS, S::SWZ>(Ps, min(64, A.M - c0 - 64));
     }
   }
   if (A.causal) {
