@@ -250,7 +250,7 @@ __device__ __forceinline__ void discard_l2(const void* p, size_t bytes, int i, i
 }
 
 // Flags sit 128 bytes apart, so the CTAs polling different flags do not
-// share a cache line.
+// share a cache line (a chain's eight warp flags of a tile share one).
 constexpr int FLAG_STRIDE = 32;
 
 // Buffers exchanged between tile CTAs (prefix slots, dOmega partials, G_t)
@@ -288,6 +288,21 @@ __device__ __forceinline__ void red_lm16(float* base, int h, int cg, int row, co
   for (int i = 0; i < 4; ++i)
     asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(d + lm4(h, cg, i, row)),
                  "f"(v[4 * i]), "f"(v[4 * i + 1]), "f"(v[4 * i + 2]), "f"(v[4 * i + 3])
+                 : "memory");
+}
+// Drops the L2 lines of a prefix that this warp of the chain group read (MH blocks of
+// 128 rows; rows 32 rq .., column groups cq and cq + 1, and z's rows when cq == 0): all
+// its lanes have their values, and no other warp reads these lines.
+__device__ __forceinline__ void discard_prefix(const float* base, int MH, int cq, int rq) {
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+  for (int h = 0; h < MH; ++h) {
+    const float4* p = reinterpret_cast<const float4*>(base) +
+                      lm4(h, cq + (lane >> 4), (lane >> 2) & 3, 32 * rq + 8 * (lane & 3));
+    asm volatile("discard.global.L2 [%0], 128;" ::"l"(p) : "memory");
+  }
+  if (cq == 0 && lane < MH)
+    asm volatile("discard.global.L2 [%0], 128;" ::"l"(base + MH * 128 * 64 + 128 * lane + 32 * rq)
                  : "memory");
 }
 // Row-major [M][64] (the caller's state tensors): 16 floats at p.
@@ -396,6 +411,40 @@ __device__ __forceinline__ bool flag_poll(const int* flag, int want, int* err) {
   give_up(err);
   return false;
 }
+// A chain hop of the chain group (warps 8-15).  by_warp: a prefix is lane-major, so a
+// warp reads exactly what the same warp of the neighbour's CTA wrote; each warp has
+// its own flag (word `warp` of the tile's flag line) and waits, adds and releases
+// without a barrier of the group, so that one warp's flag and loads travel while
+// another's stores drain.  Otherwise one thread polls and releases the line's first
+// word for the group (see by_warp_hops).  ok: false when the caller's own wait failed.
+template <bool by_warp>
+__device__ __forceinline__ bool chain_wait(const int* flag, bool seen, int want, bool wait, bool ok,
+                                           int* fail, int* err) {
+  if (!ok) *fail = 1;
+  if (wait && ok && (threadIdx.x & (by_warp ? 31 : GRP - 1)) == 0) {
+    if (seen)
+      fence_acq_rel_gpu();
+    else if (!flag_poll(flag, want, err)) {
+      *fail = 1;
+      ok = false;
+    }
+  }
+  if (!by_warp) {
+    group_bar(2);
+    return *fail == 0;
+  }
+  ok = __all_sync(0xffffffffu, ok);
+  __syncwarp();
+  return ok;
+}
+template <bool by_warp>
+__device__ __forceinline__ void chain_release(int* flag, int v) {
+  if (by_warp)
+    __syncwarp();
+  else
+    group_bar(2);  // every slot write of the group is issued
+  if ((threadIdx.x & (by_warp ? 31 : GRP - 1)) == 0) st_release_gpu(flag, v);
+}
 // Bounded wait by one thread for up to two flags at once (a null flag is not
 // waited on): both are read in every round, so a satisfied pair costs one trip.
 __device__ __forceinline__ bool flag_poll2(const int* f1, int w1, const int* f2, int w2, int* err) {
@@ -440,7 +489,7 @@ __device__ __forceinline__ bool counter_poll(const int* ctr, int want, int* err)
   return false;
 }
 
-template <int MF, int FEAT>
+template <int MF, int FEAT, bool BYW>
 __device__ __forceinline__ void role_fwd(const FwdJob& J, int pos, int c, uint8_t* smem_raw,
                                          uint64_t* mb, uint32_t& tmem_base, int& abort_) {
   using C = Cfg<MF>;
@@ -594,13 +643,13 @@ __device__ __forceinline__ void role_fwd(const FwdJob& J, int pos, int c, uint8_
       // ---- chain group: S_t, z_t = the predecessor's inclusive prefix (zero
       // for the first tile); S_t + Delta_t goes to this tile's slot.  Thread
       // (row, cg) handles column groups 2(cg-2) and 2(cg-2)+1.
-      const int gl = tid - GRP;  // 0..255
-      if (!mbar_wait(smem_u32(&mb[2]), 0, J.err)) gfail[1] = 1;
-      if (C::MH > 1 && !mbar_wait(smem_u32(&mb[5]), 0, J.err)) gfail[1] = 1;
+      const int gl = tid - GRP, cw = BYW ? gl >> 5 : 0;  // 0..255, and the flag
+      bool ok = mbar_wait(smem_u32(&mb[2]), 0, J.err);
+      if (C::MH > 1) ok = mbar_wait(smem_u32(&mb[5]), 0, J.err) && ok;
+      if (BYW) ok = __all_sync(0xffffffffu, ok);
       tc_fence_after();
-      if (pred && gl == 0 && !gfail[1] && !flag_poll(pflag, pwant, J.err)) gfail[1] = 1;
-      group_bar(2);
-      if (gfail[1]) goto join;
+      if (!chain_wait<BYW>(pflag + cw, false, pwant, pred != nullptr, ok, gfail + 1, J.err))
+        goto join;
       const int cq = 2 * (cg - 2);
       float pv[C::MH][2][16], pz[C::MH];
 #pragma unroll
@@ -667,8 +716,7 @@ __device__ __forceinline__ void role_fwd(const FwdJob& J, int pos, int c, uint8_
           }
         }
       }
-      group_bar(2);  // every slot write of the group is issued
-      if (gl == 0) st_release_gpu(oflag, n + 1);
+      chain_release<BYW>(oflag + cw, n + 1);
       // then S_t as the readout's operand, and z_t as the first two rows (hi, lo in
       // bf16) of a K-major [16][MF] operand, so that g(Q) z_t is a tensor-core
       // product with ~16-bit z (rows 2..15 are zero; the ones tile was there)
@@ -771,7 +819,7 @@ struct BwdQJob {
 // rollback chain (which needs only Delta_t); after dphiQ, warps 0-7 compute u
 // and issue dq while warps 8-15 run the state-gradient chain.  The TMEM
 // columns (all 512) are allocated by the caller for both parts of the tile.
-template <int MF, int FEAT>
+template <int MF, int FEAT, bool BYW>
 __device__ __forceinline__ void role_bwd_q(const BwdQJob& J, int b, uint8_t* smem_raw,
                                            uint64_t* mb, uint32_t& tmem_base, int& abort_,
                                            int& done_) {
@@ -831,17 +879,20 @@ __device__ __forceinline__ void role_bwd_q(const BwdQJob& J, int b, uint8_t* sme
   // the first tile of the sequence hands on G^(0), the gradient with respect
   // to the state the sequence started from
   const bool seq_first = n == 0 && t == 0 && J.gio.S_out != nullptr;
-  const int* f1 = J.flag1 + ((size_t)c * J.nt + snext) * FLAG_STRIDE;
-  const int* f2 = J.flag2 + ((size_t)c * J.nt + snext) * FLAG_STRIDE;
   float* own1 = J.slot1 + ((size_t)c * J.nt + t) * C::E;
   float* own2 = J.slot2 + ((size_t)c * J.nt + t) * C::E;
-  int* of1 = J.flag1 + ((size_t)c * J.nt + t) * FLAG_STRIDE;
-  int* of2 = J.flag2 + ((size_t)c * J.nt + t) * FLAG_STRIDE;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int row = 32 * (warp & 3) + (tid & 31);
   const int cg = warp >> 2;
   const int gl = tid - GRP;     // index inside the chain group (warps 8-15)
   const int cq = 2 * (cg - 2);  // chain group: column groups cq, cq + 1
+  // this warp's (or the group's) flags: the tile after this one, and this tile's
+  const int cw = BYW ? (gl >> 5) & 7 : 0;
+  const bool reads_flag = tid >= GRP && (gl & (BYW ? 31 : GRP - 1)) == 0 && linked;
+  const int* f1 = J.flag1 + ((size_t)c * J.nt + snext) * FLAG_STRIDE + cw;
+  const int* f2 = J.flag2 + ((size_t)c * J.nt + snext) * FLAG_STRIDE + cw;
+  int* of1 = J.flag1 + ((size_t)c * J.nt + t) * FLAG_STRIDE + cw;
+  int* of2 = J.flag2 + ((size_t)c * J.nt + t) * FLAG_STRIDE + cw;
   if (tid == 0) {
     abort_ = 0;
     for (int i = 0; i < NBAR; ++i) mbar_init(smem_u32(&mb[i]), 1);
@@ -867,7 +918,7 @@ __device__ __forceinline__ void role_bwd_q(const BwdQJob& J, int b, uint8_t* sme
   // now, so that its round trip overlaps the loads (an acquire fence follows
   // when it is used); the chain polls only if it was not set yet.
   int early1 = 0, early2 = 0;
-  if (tid == GRP && linked) early1 = ld_relaxed_gpu(f1);
+  if (reads_flag) early1 = ld_relaxed_gpu(f1);
   // this thread's 16 columns of its out row, fetched while the tiles stream in
   uint4 orow[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
   if (row < valid) {
@@ -998,14 +1049,11 @@ __device__ __forceinline__ void role_bwd_q(const BwdQJob& J, int b, uint8_t* sme
       // ---- chain group, rollback (eq. 17 per tile): the state before this
       // tile is the state after it minus Delta_t.  The prefix after this tile
       // is acquired and loaded while the Delta_t products run.
-      if (linked && gl == 0 && !gfail[1]) {
-        if (early1 == wnext)
-          fence_acq_rel_gpu();
-        else if (!flag_poll(f1, wnext, J.err))
-          gfail[1] = 1;
-      }
-      group_bar(2);
-      if (gfail[1]) goto join1;
+      // (gfail: the hand-off ring's wait, before the barrier above)
+      bool ok = gfail[1] == 0;
+      if (BYW) ok = __all_sync(0xffffffffu, ok);
+      if (!chain_wait<BYW>(f1, early1 == wnext, wnext, linked, ok, gfail + 1, J.err))
+        goto join1;
       // every load of the prefix after this tile before any store: one L2 trip
       float sv[C::MH][2][16], sz[C::MH];
 #pragma unroll
@@ -1035,11 +1083,16 @@ __device__ __forceinline__ void role_bwd_q(const BwdQJob& J, int b, uint8_t* sme
 #pragma unroll
         for (int h = 0; h < C::MH; ++h) sz[h] += __ldcg(s1.z_lo + 128 * h + row);
       }
-      if (!mbar_wait(smem_u32(&mb[2]), 0, J.err)) gfail[1] = 1;
-      if (C::MH > 1 && !mbar_wait(smem_u32(&mb[6]), 0, J.err)) gfail[1] = 1;
+      ok = mbar_wait(smem_u32(&mb[2]), 0, J.err);
+      if (C::MH > 1) ok = mbar_wait(smem_u32(&mb[6]), 0, J.err) && ok;
+      if (BYW) ok = __all_sync(0xffffffffu, ok);
       tc_fence_after();
-      group_bar(2);
-      if (gfail[1]) goto join1;
+      if (!ok) gfail[1] = 1;
+      if (!BYW) {
+        group_bar(2);
+        ok = gfail[1] == 0;
+      }
+      if (!ok) goto join1;
 #pragma unroll
       for (int h = 0; h < C::MH; ++h) {
 #pragma unroll
@@ -1065,9 +1118,13 @@ __device__ __forceinline__ void role_bwd_q(const BwdQJob& J, int b, uint8_t* sme
       // the prefix after this tile is read only here: drop it from L2 (before
       // the release, so that it comes before the slot's next writer), unless it
       // sits in this tile's own slot (one-tile slices), just rewritten
-      if (linked && snext != t) discard_l2(s1.S, (size_t)C::E * 4, gl, GRP);
-      group_bar(2);  // every slot write of the group is issued
-      if (gl == 0) st_release_gpu(of1, n + 1);
+      if (linked && snext != t) {
+        if (BYW)
+          discard_prefix(s1.S, C::MH, cq, warp & 3);
+        else  // the group's loads were complete at its last barrier
+          discard_l2(s1.S, (size_t)C::E * 4, gl, GRP);
+      }
+      chain_release<BYW>(of1, n + 1);
       // the slot released, this tile's own copy of the state
 #pragma unroll
       for (int h = 0; h < C::MH; ++h)
@@ -1078,7 +1135,7 @@ __device__ __forceinline__ void role_bwd_q(const BwdQJob& J, int b, uint8_t* sme
     __syncthreads();
     if (gfail[0] | gfail[1]) goto teardown;
     // the state-gradient chain's flag, read ahead of its use (see early1)
-    if (tid == GRP && linked) early2 = ld_relaxed_gpu(f2);
+    if (reads_flag) early2 = ld_relaxed_gpu(f2);
     // phiK's tile image, while the MMAs of the next phases run (the tile is
     // overwritten by u once the copy has read it); Q, read again after them,
     // back into L2
@@ -1231,14 +1288,8 @@ __device__ __forceinline__ void role_bwd_q(const BwdQJob& J, int b, uint8_t* sme
     } else {
       // ---- chain group, state gradient (eq. 18): G_t = the prefix after this
       // tile (zero at the end of the sequence); G_t + Gd_t goes on to tile t-1
-      if (linked && gl == 0) {
-        if (early2 == wnext)
-          fence_acq_rel_gpu();
-        else if (!flag_poll(f2, wnext, J.err))
-          gfail[1] = 1;
-      }
-      group_bar(2);
-      if (gfail[1]) goto join2;
+      if (!chain_wait<BYW>(f2, early2 == wnext, wnext, linked, true, gfail + 1, J.err))
+        goto join2;
       float gs[C::MH][2][16], gzs[C::MH];
 #pragma unroll
       for (int h = 0; h < C::MH; ++h) {
@@ -1278,9 +1329,8 @@ __device__ __forceinline__ void role_bwd_q(const BwdQJob& J, int b, uint8_t* sme
           if (seq_first) J.gio.z_out[(size_t)c * MF + m] = gzs[h] + gdz;
         }
       }
-      if (linked && snext != t) discard_l2(s2.S, (size_t)C::E * 4, gl, GRP);
-      group_bar(2);  // every slot write of the group is issued
-      if (gl == 0) st_release_gpu(of2, n + 1);
+      if (linked && snext != t) discard_prefix(s2.S, C::MH, cq, warp & 3);
+      chain_release<BYW>(of2, n + 1);
       // the slot released, G_t for the dk/dv part
 #pragma unroll
       for (int h = 0; h < C::MH; ++h) {
@@ -1726,7 +1776,7 @@ __device__ __forceinline__ void reduce_stage2(const RedJob& J, int s, float4* re
 // blockIdx, so the tiles handed out so far always belong to CTAs that are
 // running and every awaited tile is in progress whatever order the CTAs are
 // dispatched in.  (The counter is zeroed by the call's memset.)
-template <int MF, int FEAT>
+template <int MF, int FEAT, bool BYW>
 __global__ void __launch_bounds__(NTHR, 1) k_tc_fwd(const __grid_constant__ FwdJob J) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t mbar[NBAR];
@@ -1735,7 +1785,7 @@ __global__ void __launch_bounds__(NTHR, 1) k_tc_fwd(const __grid_constant__ FwdJ
   __shared__ int ticket;
   if (threadIdx.x == 0) ticket = atomicAdd(J.ticket, 1);
   __syncthreads();
-  role_fwd<MF, FEAT>(J, ticket / J.chains, ticket % J.chains, smem_raw, mbar, tmem_base, abort_);
+  role_fwd<MF, FEAT, BYW>(J, ticket / J.chains, ticket % J.chains, smem_raw, mbar, tmem_base, abort_);
 }
 
 // ------------------------------------------------------------------ backward launch
@@ -1805,7 +1855,7 @@ struct BwdJob {
   int *sums_done, *r1done;  // slice-0 tiles done, final stage-1 CTAs done
 };
 
-template <int MF, int FEAT>
+template <int MF, int FEAT, bool BYW>
 __global__ void __launch_bounds__(NTHR, 1) k_tc_bwd(const __grid_constant__ BwdJob J) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t mbar[2 * NBAR];  // the dq part's, then the dk/dv part's
@@ -1862,7 +1912,7 @@ __global__ void __launch_bounds__(NTHR, 1) k_tc_bwd(const __grid_constant__ BwdJ
     // one TMEM allocation (all 512 columns) serves both parts of the tile
     if (threadIdx.x == 0) done_ = 0;
     if (threadIdx.x < 32) tmem_alloc(smem_u32(&tmem_base), 512);
-    role_bwd_q<MF, FEAT>(q, it.idx, smem_raw, mbar, tmem_base, abort_, done_);
+    role_bwd_q<MF, FEAT, BYW>(q, it.idx, smem_raw, mbar, tmem_base, abort_, done_);
     __syncthreads();
     // the dk/dv part runs only after a complete dq part (a wait that gave up
     // has left the error word set; the part would wait on what never comes)
@@ -1927,6 +1977,14 @@ Geo geometry(const Problem& p) {
   g.E = g.MF * 65;
   return g;
 }
+
+// With few chains their hops bound the launch; with many, the tiles do, and eight flags
+// and releases per hop cost more than one.  Warp by warp against by group, M = 256,
+// L = 8192, forward / train step in us: 8 chains, C = 512 172 / 430 against 216 / 551;
+// 40 chains 227 / 903 against 236 / 910; 48 chains 262 / 1065 against 258 / 1052; 64
+// chains 341 / 1388 against 334 / 1380; the same for C = 64 to 2048.  At M = 128 the two
+// meet at 40 chains too.  B2 H8 L32768, C = 64: 3.27 against 3.84 ms.
+bool by_warp_hops(int chains) { return chains <= 40; }
 
 // The chain slots hold one prefix per (chain, tile of a slice): a slice's
 // tiles overwrite the previous slice's only after reading them.  The buffers
@@ -2016,17 +2074,17 @@ static_assert(NSLOT * 128 * 64 * 4 <= smem_bwd<128>() - 1024 &&
                   NSLOT * 256 * 64 * 4 <= smem_bwd<256>() - 1024,
               "stage-1 slots fit");
 
-template <int MF, int FEAT>
+template <int MF, int FEAT, bool BYW>
 cudaError_t configure() {
   static bool configured[kMaxDevices] = {};
   bool* done = device_flag(configured);
   if (done == nullptr) return cudaErrorInvalidDevice;
   if (*done) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(k_tc_fwd<MF, FEAT>,
+  cudaError_t e = cudaFuncSetAttribute(k_tc_fwd<MF, FEAT, BYW>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem_fwd<MF>());
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_tc_bwd<MF, FEAT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(k_tc_bwd<MF, FEAT, BYW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem_bwd<MF>());
   if (e != cudaSuccess) return e;
   *done = true;
@@ -2133,7 +2191,8 @@ slim_status fwd_impl(const Problem& p, const __nv_bfloat16* q, const __nv_bfloat
                      const __nv_bfloat16* v, const float* omega, __nv_bfloat16* out,
                      const StateOut& st, const StateInit& init, unsigned* rep, void* workspace,
                      cudaStream_t s) {
-  TC_TRY((configure<MF, FEAT>()));
+  const bool by_warp = by_warp_hops(p.chains());
+  TC_TRY(by_warp ? (configure<MF, FEAT, true>()) : (configure<MF, FEAT, false>()));
   const Geo g = geometry(p);
   Carver cv(workspace);
   const Ws w = carve(cv, g, false);
@@ -2149,7 +2208,7 @@ slim_status fwd_impl(const Problem& p, const __nv_bfloat16* q, const __nv_bfloat
   TC_TRY(prepare(w, g, omega, rep, s));
   const double rows = (double)g.chains * p.L, MD = (double)MF * D;
   prof::Scope ps(prof::K_TC_FWD, s, rows * 8.0 * MD, rows * D * 2.0 * 4);
-  TC_TRY(launch_dep(k_tc_fwd<MF, FEAT>, dim3(P * g.chains), dim3(NTHR), smem_fwd<MF>(), s, J));
+  TC_TRY(launch_dep(by_warp ? k_tc_fwd<MF, FEAT, true> : k_tc_fwd<MF, FEAT, false>, dim3(P * g.chains), dim3(NTHR), smem_fwd<MF>(), s, J));
   return SLIM_OK;
 }
 
@@ -2169,7 +2228,8 @@ slim_status bwd_impl(const Problem& p, const __nv_bfloat16* q, const __nv_bfloat
                      const __nv_bfloat16* dout, const StateIn& st, const GradIO& gio,
                      __nv_bfloat16* dq, __nv_bfloat16* dk, __nv_bfloat16* dv, float* domega,
                      unsigned* rep, void* workspace, cudaStream_t s) {
-  TC_TRY((configure<MF, FEAT>()));
+  const bool by_warp = by_warp_hops(p.chains());
+  TC_TRY(by_warp ? (configure<MF, FEAT, true>()) : (configure<MF, FEAT, false>()));
   const Geo g = geometry(p);
   Carver cv(workspace);
   const Ws w = carve(cv, g, true);
@@ -2215,7 +2275,7 @@ slim_status bwd_impl(const Problem& p, const __nv_bfloat16* q, const __nv_bfloat
   const double rows = (double)g.chains * p.L, MD = (double)MF * D;
   const long long items = sched_items(J.s);
   prof::Scope ps(prof::K_TC_BWD, s, rows * 22.0 * MD, rows * D * 2.0 * 12);
-  TC_TRY(launch_dep(k_tc_bwd<MF, FEAT>, dim3((unsigned)items), dim3(NTHR), smem_bwd<MF>(), s, J));
+  TC_TRY(launch_dep(by_warp ? k_tc_bwd<MF, FEAT, true> : k_tc_bwd<MF, FEAT, false>, dim3((unsigned)items), dim3(NTHR), smem_bwd<MF>(), s, J));
   return SLIM_OK;
 }
 
