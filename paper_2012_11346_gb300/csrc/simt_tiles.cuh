@@ -15,7 +15,7 @@
 //
 // Measured, train steps on a GB300, one batched contraction per launch (33 launches
 // per slice, every intermediate through memory) against these kernels: [4,12,8192]
-// fp32 relu, d = 64, M = 128, C = 512 10.17 -> 5.40 ms; non-causal [8,8,4096] bf16, d = 64,
+// fp32 relu, d = 64, M = 128, C = 512 10.17 -> 5.02 ms; non-causal [8,8,4096] bf16, d = 64,
 // M = 256 5.97 -> 2.28 ms; [1,4,65536] bf16, d = 128, M = 256, C = 16 30.05 -> 9.18 ms;
 // [1,1,256] fp32, d = 16, M = 32 843 -> 50 us.
 #pragma once

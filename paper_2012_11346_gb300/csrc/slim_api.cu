@@ -8,6 +8,7 @@
 #include "report.h"
 #include "simt_path.h"
 #include "stack.h"
+#include "stack_tail.h"
 #include "tc_path.h"
 
 using slim::Problem;
@@ -134,7 +135,7 @@ slim_status backward(const void* q, const void* k, const void* v, const float* o
                      const float* G_S_in, const float* g_z_in, int B, int H, int L, int d,
                      int M, int C, slim_dtype dtype, slim_feature feature, void* dq, void* dk,
                      void* dv, float* domega, float* G_S_out, float* g_z_out, void* workspace,
-                     size_t workspace_bytes, cudaStream_t s) {
+                     size_t workspace_bytes, cudaStream_t s, bool in_stack = false) {
   Problem p;
   slim_status st = check_problem(B, H, L, d, M, C, dtype, feature, &p);
   if (st != SLIM_OK) return st;
@@ -166,6 +167,10 @@ slim_status backward(const void* q, const void* k, const void* v, const float* o
   if (tc)
     return slim::tc::bwd(p, q, k, v, omega, out, dout, si, gio, dq, dk, dv, domega, counter,
                          workspace, s);
+  if (in_stack && slim::tail::supports(p))
+    return workspace_bytes < slim::tail::workspace_bytes(p)
+               ? SLIM_ERR_WORKSPACE
+               : slim::tail::bwd(p, q, k, v, omega, out, dout, si, gio, dq, dk, dv, domega, workspace, s);
   return slim::simt::bwd(p, q, k, v, omega, out, dout, si, gio, dq, dk, dv, domega, workspace, s);
 }
 
@@ -193,6 +198,19 @@ slim_status fwd_state(const void* q, const void* k, const void* v, const float* 
   return forward(q, k, v, omega, B, H, L, d, M, C, dtype, feature, nullptr, nullptr, nullptr, nullptr,
                  nullptr, S_state, z_state, S_state_lo, z_state_lo, workspace, workspace_bytes, stream,
                  true, false, true);
+}
+
+// slim_bwd_from for a slice of the layer stack (see stack_tail.cu).
+slim_status bwd_in_stack(const void* q, const void* k, const void* v, const float* omega,
+                         const void* out, const void* dout, const float* S_state,
+                         const float* z_state, const float* S_state_lo, const float* z_state_lo,
+                         const float* G_S_in, const float* g_z_in, int B, int H, int L, int d, int M,
+                         int C, slim_dtype dtype, slim_feature feature, void* dq, void* dk, void* dv,
+                         float* domega, float* G_S_out, float* g_z_out, void* workspace,
+                         size_t workspace_bytes, cudaStream_t stream) {
+  return backward(q, k, v, omega, out, dout, S_state, z_state, S_state_lo, z_state_lo, G_S_in, g_z_in, B,
+                  H, L, d, M, C, dtype, feature, dq, dk, dv, domega, G_S_out, g_z_out, workspace,
+                  workspace_bytes, stream, true);
 }
 
 // slim_fwd without the timeout report (for the allocation-free entry point,

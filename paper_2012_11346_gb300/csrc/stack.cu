@@ -17,15 +17,25 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "profiler.h"
 #include "stack.h"
+#include "stack_tail.h"
 
 namespace slim {
 slim_status fwd_state(const void* q, const void* k, const void* v, const float* omega, int B, int H,
                       int L, int d, int M, int C, slim_dtype dtype, slim_feature feature,
                       float* S_state, float* z_state, float* S_state_lo, float* z_state_lo,
                       void* workspace, size_t workspace_bytes, cudaStream_t stream);  // slim_api.cu
+slim_status bwd_in_stack(const void* q, const void* k, const void* v, const float* omega,
+                         const void* out, const void* dout, const float* S_state,
+                         const float* z_state, const float* S_state_lo, const float* z_state_lo,
+                         const float* G_S_in, const float* g_z_in, int B, int H, int L, int d, int M,
+                         int C, slim_dtype dtype, slim_feature feature, void* dq, void* dk, void* dv,
+                         float* domega, float* G_S_out, float* g_z_out, void* workspace,
+                         size_t workspace_bytes, cudaStream_t stream);  // slim_api.cu
 
 namespace stack {
 namespace {
@@ -264,7 +274,13 @@ size_t inner_bytes(const Problem& p, int Cs) {
   size_t f = 0, b = 0;
   slim_fwd_workspace_size(p.B, p.H, Cs, p.d, p.M, Cs, p.dtype, p.feature, &f);
   slim_bwd_workspace_size(p.B, p.H, Cs, p.d, p.M, Cs, p.dtype, p.feature, &b);
-  return f > b ? f : b;
+  if (b > f) f = b;
+  // full slices and the last one, where the backward of short ones has its own kernel
+  for (int rows : {Cs, Cs > 0 ? p.L % Cs : 0}) {
+    const Problem t{p.B, p.H, rows, p.d, p.M, rows, p.dtype, p.feature};
+    if (tail::supports(t)) f = std::max(f, tail::workspace_bytes(t));
+  }
+  return f;
 }
 
 Ws carve(Carver& cv, const Problem& p, const Geo& g, bool bwd, uint8_t** xin_ptrs,
@@ -443,11 +459,11 @@ slim_status bwd_impl(const Problem& p, int layers, const T* x, const float* omeg
         STACK_LAUNCH(2 * sb, k_rownorm<T><<<nrb(rows, d), kRowThreads, 0, s>>>(X, U, d, scale, rows));
         ST_TRY(cudaGetLastError());
       }
-      ST_CALL(slim_bwd_from(U, U, U, om, w.yout[r], w.dout, w.Se + r * g.st, w.ze + r * g.zt,
-                            w.Sle + r * g.st, w.zle + r * g.zt, n + 1 < g.N ? G + r * g.st : nullptr,
-                            n + 1 < g.N ? gz + r * g.zt : nullptr, p.B, p.H, b, d, M, b, p.dtype,
-                            p.feature, w.dq, w.dk, w.dv, domegas ? w.dom : nullptr,
-                            G2 + r * g.st, gz2 + r * g.zt, w.inner, g.inner, s));
+      ST_CALL(bwd_in_stack(U, U, U, om, w.yout[r], w.dout, w.Se + r * g.st, w.ze + r * g.zt,
+                           w.Sle + r * g.st, w.zle + r * g.zt, n + 1 < g.N ? G + r * g.st : nullptr,
+                           n + 1 < g.N ? gz + r * g.zt : nullptr, p.B, p.H, b, d, M, b, p.dtype,
+                           p.feature, w.dq, w.dk, w.dv, domegas ? w.dom : nullptr,
+                           G2 + r * g.st, gz2 + r * g.zt, w.inner, g.inner, s));
       if (domegas) {
         STACK_LAUNCH(12.0 * M * d, k_add<<<nb((long long)M * d), 256, 0, s>>>(
                                        domegas + (size_t)r * M * d, w.dom, (long long)M * d));
