@@ -61,8 +61,7 @@ size_t ws_bytes(const Problem& p, bool bwd, bool small = false) {
   return use_tc(p) ? slim::tc::workspace_bytes(p, bwd) : slim::simt::workspace_bytes(p, bwd, small);
 }
 
-slim_status check_workspace(const Problem& p, bool bwd, void* ws, size_t bytes, bool small = false) {
-  const size_t need = ws_bytes(p, bwd, small);
+slim_status check_workspace(size_t need, void* ws, size_t bytes) {
   if (need == 0) return SLIM_OK;
   if (ws == nullptr || bytes < need) return SLIM_ERR_WORKSPACE;
   if ((reinterpret_cast<uintptr_t>(ws) & 255u) != 0) return SLIM_ERR_INVALID_ARG;
@@ -103,7 +102,7 @@ slim_status forward(const void* q, const void* k, const void* v, const float* om
   if (omega == nullptr && feature != SLIM_FEAT_SQUARE) return SLIM_ERR_INVALID_ARG;
   if (!pair_ok(S_init, z_init) || (S_init == nullptr && (S_init_lo || z_init_lo)))
     return SLIM_ERR_INVALID_ARG;
-  st = check_workspace(p, false, workspace, workspace_bytes, small);
+  st = check_workspace(ws_bytes(p, false, small), workspace, workspace_bytes);
   if (st != SLIM_OK) return st;
   cudaStream_t s_ = s;
   if (L == 0) {
@@ -147,7 +146,9 @@ slim_status backward(const void* q, const void* k, const void* v, const float* o
   if ((omega == nullptr || domega == nullptr) && feature != SLIM_FEAT_SQUARE)
     return SLIM_ERR_INVALID_ARG;
   if (!pair_ok(G_S_in, g_z_in) || !pair_ok(G_S_out, g_z_out)) return SLIM_ERR_INVALID_ARG;
-  st = check_workspace(p, true, workspace, workspace_bytes);
+  // the kernels that run decide what the workspace has to hold
+  const bool tail = in_stack && slim::tail::supports(p);
+  st = check_workspace(tail ? slim::tail::workspace_bytes(p) : ws_bytes(p, true), workspace, workspace_bytes);
   if (st != SLIM_OK) return st;
   if (L == 0) {
     if (domega && cudaMemsetAsync(domega, 0, (size_t)M * d * sizeof(float), s) != cudaSuccess)
@@ -167,10 +168,8 @@ slim_status backward(const void* q, const void* k, const void* v, const float* o
   if (tc)
     return slim::tc::bwd(p, q, k, v, omega, out, dout, si, gio, dq, dk, dv, domega, counter,
                          workspace, s);
-  if (in_stack && slim::tail::supports(p))
-    return workspace_bytes < slim::tail::workspace_bytes(p)
-               ? SLIM_ERR_WORKSPACE
-               : slim::tail::bwd(p, q, k, v, omega, out, dout, si, gio, dq, dk, dv, domega, workspace, s);
+  if (tail)
+    return slim::tail::bwd(p, q, k, v, omega, out, dout, si, gio, dq, dk, dv, domega, workspace, s);
   return slim::simt::bwd(p, q, k, v, omega, out, dout, si, gio, dq, dk, dv, domega, workspace, s);
 }
 
