@@ -270,17 +270,21 @@ struct Ws {
   void* inner;
 };
 
+// what the segment calls need: those on full slices, and those on the last one, which
+// can need more (short slices have kernels and a workspace layout of their own)
 size_t inner_bytes(const Problem& p, int Cs) {
-  size_t f = 0, b = 0;
-  slim_fwd_workspace_size(p.B, p.H, Cs, p.d, p.M, Cs, p.dtype, p.feature, &f);
-  slim_bwd_workspace_size(p.B, p.H, Cs, p.d, p.M, Cs, p.dtype, p.feature, &b);
-  if (b > f) f = b;
-  // full slices and the last one, where the backward of short ones has its own kernel
+  size_t most = 0;
   for (int rows : {Cs, Cs > 0 ? p.L % Cs : 0}) {
     const Problem t{p.B, p.H, rows, p.d, p.M, rows, p.dtype, p.feature};
-    if (tail::supports(t)) f = std::max(f, tail::workspace_bytes(t));
+    size_t f = 0, b = 0;
+    slim_fwd_workspace_size(p.B, p.H, rows, p.d, p.M, rows, p.dtype, p.feature, &f);
+    if (tail::supports(t))
+      b = tail::workspace_bytes(t);
+    else
+      slim_bwd_workspace_size(p.B, p.H, rows, p.d, p.M, rows, p.dtype, p.feature, &b);
+    most = std::max(most, std::max(f, b));
   }
-  return f;
+  return most;
 }
 
 Ws carve(Carver& cv, const Problem& p, const Geo& g, bool bwd, uint8_t** xin_ptrs,
