@@ -18,7 +18,8 @@
  * The backward pass walks the slices in reverse (Sec. 3.3): it recomputes
  * each slice, rolls the state back by subtraction (eq. 17) and carries the
  * state gradient G^(n) (eq. 18).  Memory beyond inputs and outputs is the
- * caller-provided workspace, whose size grows with C, not with L.
+ * caller-provided workspace, whose size follows from C, not from L (see
+ * slim_fwd_workspace_size).
  *
  * Feature maps g: R^d -> R_+^M (Omega is [M, d], shared by all chains):
  *     SLIM_FEAT_EXP    : g(x)_m = exp(omega_m.x - |x|^2/2) / sqrt(M)   (FAVOR+)
@@ -99,8 +100,17 @@ int slim_version(void);
 
 /*
  * Workspace bytes needed by slim_fwd / slim_bwd for this problem.  Pure host
- * computation (no CUDA call).  The size grows linearly with min(C, L) and with
- * B*H, and does not depend on L otherwise (Sec. 3.4: O(C) memory).
+ * computation (no CUDA call).  O(C) memory (Sec. 3.4): the size does not depend
+ * on L once L is many slices.
+ *   - Tensor-core kernels (slim_path_for): linear in min(C, L) and in B*H.
+ *   - fp32-compute kernels: in proportion to the frames of 64 rows that one
+ *     launch sequence covers (backward: 50 to 630 KB a frame, by d, M and dtype):
+ *     a slice of every chain, but as many slices as make 304 frames where that is
+ *     more, and up to eight within 2432 frames.  So C and B*H set the size above
+ *     a floor of 304 frames (backward, one chain, d = 64, M = 128, fp32: 78 MB up
+ *     to C = 2432, 127 MB at C = 4096, 494 MB at C = 16384).  It never falls as L
+ *     or B*H grows: a buffer for the longest sequence and the most chains serves
+ *     every smaller call with the same d, M, C, dtype and feature map.
  * Returns SLIM_ERR_INVALID_ARG / SLIM_ERR_UNSUPPORTED as the entry points
  * would; *bytes is written only on SLIM_OK.
  */

@@ -60,8 +60,8 @@ namespace {
 // loses much of its last one.  Train steps at 304 / 1216 / 2432 frames: [4,12,8192]
 // fp32 relu, C = 512 (384 frames a slice) 6.43 / 5.46 / 5.36 ms; non-causal [8,8,4096]
 // bf16, C = 1024 (1024 frames) 2.52 / 2.52 / 2.28 ms; L = 65536, C = 16 9.17 / 8.95 /
-// 9.08 ms: short slices gain nothing from more, and the scratch stays in proportion to
-// C where C is small (200 KB to 600 KB a frame).
+// 9.08 ms: short slices gain nothing from more than the first two (200 KB to 600 KB of
+// scratch a frame).
 constexpr int kSeqFrames = 2 * kSms;  // two CTAs on each SM
 constexpr int kMostFrames = 16 * kSms;
 constexpr int kSeqSlices = 8;
@@ -74,16 +74,21 @@ struct Seq {
   int rows, nt, nf, N;   // rows per sequence, tiles and frames per chain, sequences
   int ns;                // pieces per computed operand
   int slots;             // dOmega partials of a backward launch
+  size_t frames, tiles;  // of all chains, that the workspace holds
 };
 
 // tiles of the first `rows` rows of a sequence (tiles start anew in every slice)
 int tiles_of(int rows, int slice, int pitch) {
-  const int per = (slice + pitch - 1) / pitch;
-  return rows / slice * per + (rows % slice + pitch - 1) / pitch;
+  const int per = (int)(((long long)slice + pitch - 1) / pitch);
+  return rows / slice * per + (int)(((long long)(rows % slice) + pitch - 1) / pitch);
 }
 
-// chains: how many are swept together.  small: the fewest rows per sequence; the
-// tiles are the same either way.
+// The sweep of `chains` chains.  small: the fewest rows per sequence; the tiles are the
+// same either way.
+//
+// The workspace is sized by the most frames that a sequence may have, not by those
+// that the even cut below leaves: it then falls neither with a shorter sequence nor with
+// fewer chains, and a buffer for the largest of several problems serves them all.
 Seq sequence(const Problem& p, int chains, bool small) {
   Seq q;
   q.chains = chains;
@@ -95,27 +100,32 @@ Seq sequence(const Problem& p, int chains, bool small) {
   q.pitch = Cs < kTile ? (Cs > 0 ? Cs : 1) : kTile;
   q.tile = (q.pitch + 15) / 16 * 16;
   q.per = q.tile <= 32 ? kTile / q.tile : 1;
-  const long long fill = kSeqFrames / chains, most = kMostFrames / chains;  // frames per chain
+  q.slice = Cs < kTile ? q.pitch : Cs;
+  const long long frame = (long long)q.per * q.pitch;  // its rows
+  // frames of one slice, or the one frame that several short ones share, of all chains
+  const long long slice = Cs < kTile ? chains : (((long long)Cs + kTile - 1) / kTile) * chains;
+  long long most = slice;
+  if (!small && Cs < kTile)
+    most = std::max<long long>(kSeqFrames, (kShortRows + frame - 1) / frame * chains);
+  else if (!small)
+    most = std::max<long long>({slice, kSeqFrames, std::min<long long>(kSeqSlices * slice, kMostFrames)});
   long long rows = Cs;
   if (Cs < kTile) {
-    const long long frame = (long long)q.per * q.pitch, least = (kShortRows + frame - 1) / frame;
-    rows = frame * (small ? 1 : (fill > least ? fill : least));
-  } else if (!small) {
-    const long long per_slice = (Cs + kTile - 1) / kTile, more = most / per_slice;
-    const long long slices = std::max(fill / per_slice, std::min<long long>(more, kSeqSlices));
-    if (slices > 1) {  // evenly: the same number of sequences, without a small last one
-      const long long all = ((long long)p.L + Cs - 1) / Cs, seqs = (all + slices - 1) / slices;
-      rows = (all + seqs - 1) / seqs * Cs;
-    }
+    rows = frame * (most / chains);
+  } else if (most / slice > 1) {  // evenly: the same number of sequences, without a small last one
+    const long long slices = most / slice, all = ((long long)p.L + Cs - 1) / Cs,
+                    seqs = (all + slices - 1) / slices;
+    rows = (all + seqs - 1) / seqs * Cs;
   }
   q.rows = (int)(rows < p.L ? rows : p.L);
-  q.slice = Cs < kTile ? q.pitch : Cs;
   q.nt = tiles_of(q.rows, q.slice, q.pitch);
   q.nf = (q.nt + q.per - 1) / q.per;
-  q.N = p.L == 0 ? 0 : (p.L + q.rows - 1) / q.rows;
-  const long long frames = (long long)q.chains * q.nf;
-  const int ctas = tile_kernels(p.dtype, p.d).slots;
-  q.slots = (int)(frames < ctas ? frames : ctas);
+  q.N = p.L == 0 ? 0 : (int)(((long long)p.L + q.rows - 1) / q.rows);
+  const long long nt = tiles_of(p.L, q.slice, q.pitch);
+  q.frames = (size_t)std::min(most, (nt + q.per - 1) / q.per * chains);
+  q.tiles = (size_t)std::min<long long>(q.frames * q.per, nt * chains);
+  const long long ctas = tile_kernels(p.dtype, p.d).slots;
+  q.slots = (int)std::min<long long>(q.frames, ctas);
   return q;
 }
 
@@ -127,17 +137,19 @@ struct SeqWs {
   __nv_bfloat16 *phi_q, *sA, *sdA, *sW;
 };
 
-SeqWs carve_seq(Carver& cv, const Seq& q, bool bwd) {
+// spare: room for any call of fewer rows too.  One frame of short tiles per chain keeps a pair
+// and its tiles' z, more than the one frame of a slice of 33 to 64 rows.
+SeqWs carve_seq(Carver& cv, const Seq& q, bool bwd, bool spare = true) {
   SeqWs w{};
-  const size_t C = q.chains, frames = C * q.nf;
+  const size_t C = q.chains, frames = q.frames, least = spare ? C : 0;
   w.err = cv.take<int>(64);
   w.st_hi = cv.take<float>(C * q.E);
   w.st_lo = cv.take<float>(C * q.E);
   w.om_t = cv.take<float>((size_t)(q.M + 63) / 64 * 64 * q.d);
   w.om_row = cv.take<__nv_bfloat16>((size_t)3 * q.M * q.d);
   w.om_norm = cv.take<float>(q.M);
-  w.delta = cv.take<float>(frames * (q.per > 1 ? 2 : 1) * q.E);
-  if (q.per > 1) w.zdelta = cv.take<float>(C * q.nt * q.M);
+  w.delta = cv.take<float>(std::max(frames * (q.per > 1 ? 2 : 1), 2 * least) * q.E);
+  w.zdelta = cv.take<float>(std::max(q.per > 1 ? q.tiles : 0, least) * q.M);
   w.phi_k = cv.take<__nv_bfloat16>(frames * q.ns * q.M * kTile);
   if (bwd) {
     w.g_hi = cv.take<float>(C * q.E);
@@ -238,7 +250,7 @@ slim_status fwd_chains(const Problem& p, int c0, const Seq& sq, const void* q, c
                        const void* v, const float* omega, void* out, StateOut st, StateInit init,
                        void* workspace, cudaStream_t s) {
   Carver cv(workspace);
-  const SeqWs w = carve_seq(cv, sq, false);
+  const SeqWs w = carve_seq(cv, sq, false, false);
   const TileKernels& tk = tile_kernels(p.dtype, p.d);
   const size_t so = (size_t)c0 * p.M * p.d, zo = (size_t)c0 * p.M;
   st = StateOut{off(st.S, so), off(st.z, zo), off(st.S_lo, so), off(st.z_lo, zo)};
@@ -262,7 +274,7 @@ slim_status fwd_chains(const Problem& p, int c0, const Seq& sq, const void* q, c
 
 size_t fwd_bytes(const Problem& p, int chains, bool small) {
   Carver cv(nullptr);
-  carve_seq(cv, sequence(p, chains, small), false);
+  carve_seq(cv, sequence(p, chains, small), false, !small);
   return cv.bytes();
 }
 

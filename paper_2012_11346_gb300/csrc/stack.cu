@@ -270,11 +270,13 @@ struct Ws {
   void* inner;
 };
 
-// what the segment calls need: those on full slices, and those on the last one, which
-// can need more (short slices have kernels and a workspace layout of their own)
+// what the segment calls need: those on full slices, and those on a last one of fewer
+// rows, which can need more where it has kernels of its own (below 64 rows) and never
+// does otherwise.  Every last slice is counted, whatever L leaves over: a stack's
+// workspace serves every shorter sequence.
 size_t inner_bytes(const Problem& p, int Cs) {
   size_t most = 0;
-  for (int rows : {Cs, Cs > 0 ? p.L % Cs : 0}) {
+  for (int rows : {Cs, std::min(Cs, 63)}) {
     const Problem t{p.B, p.H, rows, p.d, p.M, rows, p.dtype, p.feature};
     size_t f = 0, b = 0;
     slim_fwd_workspace_size(p.B, p.H, rows, p.d, p.M, rows, p.dtype, p.feature, &f);
