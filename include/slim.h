@@ -104,7 +104,7 @@ int slim_version(void);
  * on L once L is many slices.
  *   - Tensor-core kernels (slim_path_for): linear in min(C, L) and in B*H.
  *   - fp32-compute kernels: in proportion to the frames of 64 rows that one
- *     launch sequence covers (backward: 50 to 630 KB a frame, by d, M and dtype):
+ *     launch sequence covers (backward: 50 to 770 KB a frame, by d, M and dtype):
  *     a slice of every chain, but as many slices as make 304 frames where that is
  *     more, and up to eight within 2432 frames.  So C and B*H set the size above
  *     a floor of 304 frames (backward, one chain, d = 64, M = 128, fp32: 78 MB up
@@ -425,7 +425,8 @@ slim_status slim_diag_wait_timeout(void* workspace, void* stream);
  *       4*B*H*((T + 2)*M*(d + 1) + R*(4*d + 2*M + 2 + R/T)) bytes
  *     above it (R rows of a slice in T tiles of 64; of up to 1024 rows in tiles
  *     of C when C is 16, 32 or 48).  slim_fwd_workspace_size may be larger there:
- *     the sweep then takes fewer rows and chains at a time, with the same results.
+ *     the sweep then takes as many chains and rows at a time as the scratch holds,
+ *     with the same results.
  *     Use slim_fwd with a caller workspace, or a smaller C or B*H, beyond it.
  *   - The first call on a device looks up the array's device address
  *     (cudaGetSymbolAddress) with that device current.

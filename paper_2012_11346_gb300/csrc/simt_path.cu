@@ -83,13 +83,15 @@ int tiles_of(int rows, int slice, int pitch) {
   return rows / slice * per + (int)(((long long)(rows % slice) + pitch - 1) / pitch);
 }
 
-// The sweep of `chains` chains.  small: the fewest rows per sequence; the tiles are the
-// same either way.
+// The sweep of `chains` chains, with at most `limit` frames per sequence (but a slice, or a
+// frame of short ones, of every chain at least); the tiles and the bits are the same for
+// every limit.
 //
 // The workspace is sized by the most frames that a sequence may have, not by those
 // that the even cut below leaves: it then falls neither with a shorter sequence nor with
 // fewer chains, and a buffer for the largest of several problems serves them all.
-Seq sequence(const Problem& p, int chains, bool small) {
+constexpr long long kNoLimit = kMostFrames * (1LL << 24);
+Seq sequence(const Problem& p, int chains, long long limit = kNoLimit) {
   Seq q;
   q.chains = chains;
   q.d = p.d;
@@ -104,11 +106,9 @@ Seq sequence(const Problem& p, int chains, bool small) {
   const long long frame = (long long)q.per * q.pitch;  // its rows
   // frames of one slice, or the one frame that several short ones share, of all chains
   const long long slice = Cs < kTile ? chains : (((long long)Cs + kTile - 1) / kTile) * chains;
-  long long most = slice;
-  if (!small && Cs < kTile)
-    most = std::max<long long>(kSeqFrames, (kShortRows + frame - 1) / frame * chains);
-  else if (!small)
-    most = std::max<long long>({slice, kSeqFrames, std::min<long long>(kSeqSlices * slice, kMostFrames)});
+  long long most = Cs < kTile ? (kShortRows + frame - 1) / frame * chains
+                              : std::min<long long>(kSeqSlices * slice, kMostFrames);
+  most = std::max(slice, std::min(limit, std::max<long long>(kSeqFrames, most)));
   long long rows = Cs;
   if (Cs < kTile) {
     rows = frame * (most / chains);
@@ -272,9 +272,9 @@ slim_status fwd_chains(const Problem& p, int c0, const Seq& sq, const void* q, c
   return SLIM_OK;
 }
 
-size_t fwd_bytes(const Problem& p, int chains, bool small) {
+size_t fwd_bytes(const Problem& p, int chains, long long limit) {
   Carver cv(nullptr);
-  carve_seq(cv, sequence(p, chains, small), false, !small);
+  carve_seq(cv, sequence(p, chains, limit), false, limit == kNoLimit);
   return cv.bytes();
 }
 
@@ -288,7 +288,7 @@ slim_status bwd_impl(const Problem& p, const void* q, const void* k, const void*
                      const float* omega, const void* out, const void* dout,
                      const StateIn& st, const GradIO& gio, void* dq, void* dk, void* dv,
                      float* domega, void* workspace, cudaStream_t s) {
-  const Seq sq = sequence(p, p.chains(), false);
+  const Seq sq = sequence(p, p.chains());
   Carver cv(workspace);
   const SeqWs w = carve_seq(cv, sq, true);
   const TileKernels& tk = tile_kernels(p.dtype, p.d);
@@ -325,7 +325,7 @@ slim_status bwd_impl(const Problem& p, const void* q, const void* k, const void*
 slim_status fwd_bidir_impl(const Problem& p, const void* q, const void* k, const void* v,
                            const float* omega, void* out, const StateOut& st, void* workspace,
                            cudaStream_t s) {
-  const Seq sq = sequence(p, p.chains(), false);
+  const Seq sq = sequence(p, p.chains());
   Carver cv(workspace);
   const SeqWs w = carve_seq(cv, sq, false);
   const TileKernels& tk = tile_kernels(p.dtype, p.d);
@@ -356,7 +356,7 @@ slim_status bwd_bidir_impl(const Problem& p, const void* q, const void* k, const
                            const float* omega, const void* out, const void* dout,
                            const StateIn& st, void* dq, void* dk, void* dv, float* domega,
                            void* workspace, cudaStream_t s) {
-  const Seq sq = sequence(p, p.chains(), false);
+  const Seq sq = sequence(p, p.chains());
   Carver cv(workspace);
   const SeqWs w = carve_seq(cv, sq, true);
   const TileKernels& tk = tile_kernels(p.dtype, p.d);
@@ -399,9 +399,9 @@ slim_status bwd_bidir_impl(const Problem& p, const void* q, const void* k, const
 }  // namespace
 
 size_t workspace_bytes(const Problem& p, bool bwd, bool small) {
-  if (!bwd) return fwd_bytes(p, small ? 1 : p.chains(), small);
+  if (!bwd) return small ? fwd_bytes(p, 1, 0) : fwd_bytes(p, p.chains(), kNoLimit);
   Carver cv(nullptr);
-  carve_seq(cv, sequence(p, p.chains(), false), true);
+  carve_seq(cv, sequence(p, p.chains()), true);
   return cv.bytes();
 }
 
@@ -424,34 +424,43 @@ size_t noalloc_bytes(const Problem& p) {
   return cv.bytes();
 }
 
-// With less workspace than workspace_bytes asks for, the fewest rows per
-// sequence, and as many chains at a time as fit.
+// With less workspace than workspace_bytes asks for, as many chains at a time as fit, and
+// then as many frames per sequence.  (A frame per sequence instead: one chain of 8192 rows,
+// d = 128, M = 256, bf16, C = 16 in slim_fwd_noalloc's scratch 15.0 ms against 0.37 ms.)
 slim_status fwd(const Problem& p, const void* q_ptr, const void* k, const void* v,
                 const float* omega, void* out, const StateOut& st, const StateInit& init,
                 void* workspace, size_t bytes, cudaStream_t s) {
   int batch = p.chains();
+  long long limit = kNoLimit;
   if (out && p.L <= kShortMax && p.C >= p.L) {
     // a few rows on a running state: one launch (a frame of the general kernels
     // holds 64 rows; measured 70 us for one row of 64 chains there, 13 us here)
-    const Seq q = sequence(p, 1, true);
+    const Seq q = sequence(p, 1);
     const TileArgs A = seq_args(p, q, SeqWs{}, q_ptr, k, v, omega);
     SLIM_TRY(launch_short(p, A.ks_n, A.ks_a, q_ptr, k, v, omega, out, st, init,
                           static_cast<int*>(workspace), s));
     return SLIM_OK;
   }
-  const bool small = bytes < fwd_bytes(p, batch, false);
-  if (small) {
-    const size_t one = fwd_bytes(p, 1, true), two = fwd_bytes(p, 2, true);
+  if (bytes < fwd_bytes(p, batch, kNoLimit)) {
+    const size_t one = fwd_bytes(p, 1, 0), two = fwd_bytes(p, 2, 0);
     if (bytes < one) return SLIM_ERR_WORKSPACE;
     // every chain after the first adds the same, give or take the arrays' alignment
-    while (batch > 1 && fwd_bytes(p, batch, true) > bytes) {
+    while (batch > 1 && fwd_bytes(p, batch, 0) > bytes) {
       const size_t fit = 1 + (bytes - one) / (two - one);
       batch = fit < (size_t)batch ? (int)fit : batch - 1;
+    }
+    long long most = sequence(p, batch).frames;
+    for (limit = 0; limit < most;) {
+      const long long mid = (limit + most + 1) / 2;
+      if (fwd_bytes(p, batch, mid) <= bytes)
+        limit = mid;
+      else
+        most = mid - 1;
     }
   }
   for (int c0 = 0; c0 < p.chains(); c0 += batch) {
     const int n = p.chains() - c0 < batch ? p.chains() - c0 : batch;
-    const slim_status r = fwd_chains(p, c0, sequence(p, n, small), q_ptr, k, v, omega, out, st, init,
+    const slim_status r = fwd_chains(p, c0, sequence(p, n, limit), q_ptr, k, v, omega, out, st, init,
                                      workspace, s);
     if (r != SLIM_OK) return r;
   }
