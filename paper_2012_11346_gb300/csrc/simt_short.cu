@@ -22,9 +22,9 @@ struct ShortSmem {
   static constexpr int threads = 512;
   static constexpr int xs = 2 * 16 * OP, as = NS * 16 * PA, v = NX * 16 * PV;
   // Omega, then the partial sums of the products
-  static int om(int M) { return M * OP > red() ? M * OP : red(); }
+  static constexpr int om(int M) { return M * OP > red() ? M * OP : red(); }
   static constexpr int red() { return 4 * 16 * (D + 1) + 8 * 256; }
-  static int bytes(int M) {
+  static constexpr int bytes(int M) {
     return (om(M) + xs + 2 * 16 + 16 + M) * 4 + (as + v + 2 * NS * 16 * (M + 8)) * 2;
   }
 };
@@ -140,11 +140,9 @@ __global__ void __launch_bounds__(ShortSmem<IO, D>::threads) k_short(const __gri
     const float* x = xs + side * 16 * OP;
     const float* o = om + m * OP;
     bf16* dst = (side ? Pk : Pq) + m;
-    float on = 0.f;
-    if (A.feature == SLIM_FEAT_RELU) {
-      for (int j = 0; j < D; ++j) on = fmaf(o[j], o[j], on);
-      on = sqrtf(on);
-    }
+    // |omega| in k_setup's order: the bound on a projection's error is then the same number
+    // as in the kernels of a backward that follows, and so is every decision
+    const float on = A.feature == SLIM_FEAT_RELU ? sqrtf(thread_norm2<D>(o)) : 0.f;
     for (int r0 = 0; r0 < 16; r0 += 4) {
       float acc[4] = {};
       if (r0 < A.L) {
@@ -393,6 +391,7 @@ __global__ void __launch_bounds__(ShortSmem<IO, D>::threads) k_short(const __gri
 template <typename IO, int D>
 cudaError_t run(const Problem& p, ShortArgs& A, cudaStream_t s) {
   using S = ShortSmem<IO, D>;
+  static_assert(S::bytes(256) <= kSmemMax, "shared memory");
   static bool flags[kMaxDevices] = {};
   bool* set = device_flag(flags);
   if (set == nullptr) return cudaErrorInvalidDevice;

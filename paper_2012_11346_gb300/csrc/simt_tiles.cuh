@@ -26,7 +26,6 @@ namespace slim {
 namespace simt {
 
 constexpr int kChunk = 32;     // features staged at a time by the row kernels
-constexpr int kSmemMax = 232448;
 
 // x . omega as a compensated dot product (FMA TwoProduct and TwoSum, about 48
 // bits; Ogita, Rump and Oishi's Dot2): decides ReLU's branch where the

@@ -10,6 +10,7 @@ namespace slim {
 namespace simt {
 
 constexpr int kThreads = 256;  // 8 warps
+constexpr int kSmemMax = 232448;  // shared memory of a CTA
 template <typename IO> struct Pieces;
 template <> struct Pieces<bf16> { static constexpr int NX = 1, NS = 2; };
 template <> struct Pieces<float> { static constexpr int NX = 3, NS = 3; };
@@ -85,6 +86,25 @@ __device__ __forceinline__ float warp_norm2(const float* x) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   return s;
+}
+
+// warp_norm2's sums, term for term, by one thread (16-byte aligned x)
+template <int D>
+__device__ __forceinline__ float thread_norm2(const float* x) {
+  float s[32] = {};
+#pragma unroll
+  for (int j = 0; j < D; j += 4) {
+    const float4 v = *reinterpret_cast<const float4*>(x + j);
+    s[j % 32] = fmaf(v.x, v.x, s[j % 32]);
+    s[j % 32 + 1] = fmaf(v.y, v.y, s[j % 32 + 1]);
+    s[j % 32 + 2] = fmaf(v.z, v.z, s[j % 32 + 2]);
+    s[j % 32 + 3] = fmaf(v.w, v.w, s[j % 32 + 3]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int i = 0; i < o; ++i) s[i] += s[i + o];
+  return s[0];
 }
 
 // the fp32 value of staged pieces, smallest piece first
