@@ -141,8 +141,9 @@ __global__ void __launch_bounds__(256) k_carry(const __grid_constant__ CarryArgs
           }
         }
     }
-    // the state to carry on: after the sums, or rolled back
-    if (pass == 0 || mode != CARRY_ROLLBACK) {
+    // the state to carry on: after the sums, or rolled back (a forward's last state goes to
+    // the caller alone)
+    if (pass == 0 || (mode != CARRY_ROLLBACK && !(mode == CARRY_FWD && A.out.S))) {
       hi_p[idx] = hi.v;
       lo_p[idx] = lo.v;
     }

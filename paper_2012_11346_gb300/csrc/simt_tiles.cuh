@@ -218,12 +218,16 @@ __device__ __forceinline__ void features_rows(const TileArgs& A, const Frame& f,
   for (int i = NI; i < 4; ++i) put(rt + 16 * i, fq, zero);
 }
 // A frame whose rows all lie in its first 16 (a few new rows on a running state)
-// projects those alone.
-template <int D, int W, typename Put>
+// projects those alone; HALF: so does one whose rows lie in its first 32 (k_out_short on
+// one slice of 17 to 32 rows, d = 128, M = 256: 61 -> 47 us with its second tile left out
+// too; in every kernel that variant cost 1 % of the C = 16 and quadratic steps).
+template <int D, int W, bool HALF = false, typename Put>
 __device__ __forceinline__ void features_fp(const TileArgs& A, const Frame& f, const float* xs,
                                             const float* norm2, const float* om, int c0, Put put) {
   if (f.left <= (A.pitch < 16 ? A.pitch : 16))
     features_rows<D, W, 1>(A, f, xs, norm2, om, c0, put);
+  else if (HALF && f.left <= (A.pitch < 32 ? A.pitch : 32))
+    features_rows<D, W, 2>(A, f, xs, norm2, om, c0, put);
   else
     features_rows<D, W, 4>(A, f, xs, norm2, om, c0, put);
 }
@@ -231,11 +235,11 @@ __device__ __forceinline__ void features_fp(const TileArgs& A, const Frame& f, c
 constexpr int kPF = 64 + 8;  // row pitch of the forward's 64 x 64 chunk tiles
 
 // features_fp into pieces [NS][64][kPF]
-template <int D, int NS>
+template <int D, int NS, bool HALF = false>
 __device__ __forceinline__ void features_to_pieces(const TileArgs& A, const Frame& f, const float* xs,
                                                    const float* norm2, const float* om, int c0,
                                                    bf16* dst) {
-  features_fp<D, 64>(A, f, xs, norm2, om, c0, [&](int r, int fo, const float(&v)[4]) {
+  features_fp<D, 64, HALF>(A, f, xs, norm2, om, c0, [&](int r, int fo, const float(&v)[4]) {
     uint32_t a[NS], b[NS];
     split_pair<NS>(v[0], v[1], a);
     split_pair<NS>(v[2], v[3], b);
@@ -293,8 +297,9 @@ __global__ void __launch_bounds__(kThreads, (DeltaSmem<IO, D>::ctas)) k_delta(co
   row_norms<D>(xs, norm2);
   pdl_wait();
   pdl_launch();
+  const int cstep = 64 * gridDim.y;  // a frame's chunks may be dealt to several CTAs
   if (!square) {
-    stage_omega<D, 64>(om, A.om_t, 0);
+    stage_omega<D, 64>(om, A.om_t, 64 * blockIdx.y);
     cp_commit();
   }
 
@@ -308,13 +313,13 @@ __global__ void __launch_bounds__(kThreads, (DeltaSmem<IO, D>::ctas)) k_delta(co
   float* zd = A.per == 1 ? dl + A.M * D : A.zdelta + ((size_t)f.c * A.nt + f.t0) * A.M;
   bf16* pk = A.phi_k ? A.phi_k + (size_t)frame * NS * 64 * A.M : nullptr;
   const int ntl = min(A.per, A.nt - f.t0);  // tiles of this frame
-  for (int c0 = 0; c0 < A.M; c0 += 64) {
+  for (int c0 = 64 * blockIdx.y; c0 < A.M; c0 += cstep) {
     cp_wait<0>();
     __syncthreads();
     features_to_pieces<D, NS>(A, f, xs, norm2, om, c0, Ph);
     __syncthreads();
-    if (!square && c0 + 64 < A.M) {
-      stage_omega<D, 64>(om, A.om_t, c0 + 64);
+    if (!square && c0 + cstep < A.M) {
+      stage_omega<D, 64>(om, A.om_t, c0 + cstep);
       cp_commit();
     }
     const int nf = min(64, A.M - c0);
@@ -808,7 +813,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
       }
     cp_wait<1>();
     __syncthreads();
-    features_to_pieces<D, NS>(A, f, xs, norm2, om, c0, Ph);
+    features_to_pieces<D, NS, MODE == 1>(A, f, xs, norm2, om, c0, Ph);
     if (tid < nf) {  // z at every tile of the frame
       const float* p = Pt + MD + c0 + tid;
       float zh = p[0], zl = p[plo];
@@ -831,6 +836,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
         const int gn = halves ? (A.ks_n == 4 ? s >> 1 : 0) : s & (A.ks_n - 1);
 #pragma unroll
         for (int j = 0; j < NTI; ++j) {
+          if (MODE == 1 && j >= ntl) break;
           uint32_t b[NS][4];
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
@@ -852,7 +858,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
 #pragma unroll
             for (int q = 0; q < GN; ++q)
               if (q == gn) mma_pieces<NS, NS>(num[q][rb][0], num[q][rb][1], a, b);
-            if (A.causal && j + 1 < NTI) {  // Delta^T, the pieces' products in Delta's order
+            if (A.causal && j + 1 < (MODE == 1 ? ntl : NTI)) {  // Delta^T, the pieces' products in Delta's order
               uint32_t v[NX][4], k[NS][4];
               ld_at<NX>(v, Vs, kTile * PD, PD, cb, 16 * rb);
               ld_bt<NS>(k, Kp, 64 * kPF, kPF, 16 * s, 16 * rb);
@@ -866,7 +872,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
                   }
             }
           }
-          if (A.causal && j + 1 < NTI) {
+          if (A.causal && j + 1 < (MODE == 1 ? ntl : NTI)) {
 #pragma unroll
             for (int i = 0; i < 8; ++i) pair_add(hi[s][i], lo[s][i], d[i >> 2][i & 3]);
           }
@@ -1880,7 +1886,13 @@ cudaError_t run_delta(const TileArgs& A, cudaStream_t s) {
   const double rows = (double)A.chains * A.b;
   const double proj = A.feature == SLIM_FEAT_SQUARE ? 0.0 : 2.0;
   prof::Scope ps(prof::K_TILE_DELTA, s, (2.0 + proj) * rows * D * A.M, 2.0 * rows * D * sizeof(IO));
-  return launch_pdl(k_delta<IO, D>, (unsigned)(A.chains * A.nf), kThreads, smem, s, A);
+  // Few frames leave SMs idle: their chunks of 64 features, which share nothing but the
+  // rows, then go to as many CTAs as the chip has room for (one frame of d = 128, M = 256 in
+  // fp32: 47 -> 18 us; 64 frames 55 -> 36).  A frame that has an SM to itself loads its rows once.
+  const unsigned frames = (unsigned)(A.chains * A.nf), chunks = (A.M + 63) / 64,
+                 room = kSms * DeltaSmem<IO, D>::ctas / frames;
+  const dim3 grid(frames, room < 2 ? 1 : room < chunks ? room : chunks);
+  return launch_pdl(k_delta<IO, D>, grid, kThreads, smem, s, A);
 }
 template <typename IO, int D, int MODE>
 cudaError_t run_out_short(const TileArgs& A, cudaStream_t s) {
