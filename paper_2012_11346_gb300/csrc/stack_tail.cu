@@ -1,5 +1,6 @@
-// Backward of one bf16 slice of fewer than 64 rows in the layer stack: the last
-// slice of a stack on the tensor-core path, where C does not divide L.
+// Backward of one bf16 slice of fewer than 64 rows in the layer stack, d = 64 and M 128 or
+// 256: the last slice of a stack on the tensor-core path where C does not divide L, and
+// every slice where C < 64.
 //
 // A layer's dq, dk and dv are rounded to bf16 and feed the layers below, so in a
 // stack the summation order of one short slice decides roundings that move every
@@ -9,9 +10,12 @@
 // groups() interleaved groups, group sums in order, and a 65th column in fp32 FMA.
 // The tile kernels (simt_tiles.cuh), which sum otherwise, serve every other call.
 //
-// One CTA per chain, every intermediate in L2 (310 or 510 KB a chain); one launch
-// and the sum of the chains' dOmega, where the same contractions took 33 launches.
-// A slice of one in L / C: bound by latency, not tuned further.
+// One CTA per chain, two on an SM, every intermediate in L2 (310 or 510 KB a chain); one
+// launch and the sum of the chains' dOmega, where the same contractions took 33 launches.
+// Bound by the latency of its loads, element by element.  The backward of a one-layer stack
+// of one slice, 33 launches against this kernel: 63 rows of 64 chains, M = 256, 620 -> 541
+// us; of 512 chains 1993 -> 1795; 16 rows of 64 chains 448 -> 274 (with one block of columns per
+// fragment of A 640, 2130 and 287).
 #include <math.h>
 
 #include "profiler.h"
@@ -55,21 +59,19 @@ __device__ __forceinline__ float pieces(float x) {
   return __bfloat162float(__float2bfloat16_rn(__fsub_rn(x, h))) + h;
 }
 
-// put(i, j, C(i, j)) for C = A B, A m x k (m a multiple of 16), B k x n; ends with a barrier
-template <typename Put>
-__device__ __noinline__ void product(int m, int n, int k, Mat a, Mat b, Put put) {
+// C = A B, a warp taking 16 rows and NB blocks of 8 columns at a time
+template <int NB, typename Put>
+__device__ __noinline__ void product_blocks(int m, int n, int nb, int k, int ks, Mat a, Mat b, Put put) {
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, g = lane >> 2, t = lane & 3;
-  const int ks = groups(m, n, k), steps = (k + 16 * ks - 1) / (16 * ks);
-  const bool ext = n == DP;
-  const int nb = ext ? D / 8 : (n + 7) / 8;
-  for (int u = warp; u < m / 16 * nb; u += NT / 32) {
-    const int i0 = u / nb * 16, j0 = u % nb * 8;
-    float sum[4] = {};
+  const int steps = (k + 16 * ks - 1) / (16 * ks), wide = (nb + NB - 1) / NB;
+  for (int u = warp; u < m / 16 * wide; u += NT / 32) {
+    const int i0 = u / wide * 16, j0 = u % wide * 8 * NB;
+    float sum[NB][4] = {};
     for (int gg = 0; gg < ks; ++gg) {
-      float acc[4] = {};
+      float acc[NB][4] = {};
       for (int st = 0; st < steps; ++st) {
         const int k0 = (gg + st * ks) * 16;
-        uint32_t af[4][2], bf[2][2], fa[2][4];
+        uint32_t af[4][2], fa[2][4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const float* p = a.p + (i0 + g + 8 * (i & 1)) * a.rs;
@@ -79,26 +81,50 @@ __device__ __noinline__ void product(int m, int n, int k, Mat a, Mat b, Put put)
           fa[1][i] = af[i][1];
         }
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const float* p = b.p + (j0 + g) * b.cs;
-          const int kk = k0 + 2 * (t + 4 * i);
-          const bool ok = j0 + g < n;
-          split_pair<2>(ok && kk < k ? p[kk * b.rs] : 0.f, ok && kk + 1 < k ? p[(kk + 1) * b.rs] : 0.f,
-                        bf[i]);
+        for (int q = 0; q < NB; ++q) {
+          uint32_t bf[2][2];
+          const int j = j0 + 8 * q + g;
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const float* p = b.p + j * b.cs;
+            const int kk = k0 + 2 * (t + 4 * i);
+            const bool ok = j < n;
+            split_pair<2>(ok && kk < k ? p[kk * b.rs] : 0.f, ok && kk + 1 < k ? p[(kk + 1) * b.rs] : 0.f,
+                          bf[i]);
+          }
+          mma16816(acc[q], fa[0], bf[0][1], bf[1][1]);
+          mma16816(acc[q], fa[1], bf[0][0], bf[1][0]);
+          mma16816(acc[q], fa[0], bf[0][0], bf[1][0]);
         }
-        mma16816(acc, fa[0], bf[0][1], bf[1][1]);
-        mma16816(acc, fa[1], bf[0][0], bf[1][0]);
-        mma16816(acc, fa[0], bf[0][0], bf[1][0]);
       }
 #pragma unroll
-      for (int c = 0; c < 4; ++c) sum[c] = gg ? sum[c] + acc[c] : acc[c];
+      for (int q = 0; q < NB; ++q)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) sum[q][c] = gg ? sum[q][c] + acc[q][c] : acc[q][c];
     }
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int i = i0 + g + 8 * (c >> 1), j = j0 + 2 * t + (c & 1);
-      if (j < n) put(i, j, sum[c]);
-    }
+    for (int q = 0; q < NB; ++q)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int i = i0 + g + 8 * (c >> 1), j = j0 + 8 * q + 2 * t + (c & 1);
+        if (j < min(n, 8 * nb)) put(i, j, sum[q][c]);
+      }
   }
+}
+
+// put(i, j, C(i, j)) for C = A B, A m x k (m a multiple of 16), B k x n; ends with a barrier.
+// Where every warp still has work, a fragment of A, loaded and split once, serves two
+// blocks of columns (four: no faster, and it spills in the 64 registers that two CTAs on an
+// SM leave; one CTA with four blocks is faster up to 152 chains and slower above).
+template <typename Put>
+__device__ __forceinline__ void product(int m, int n, int k, Mat a, Mat b, Put put) {
+  const int ks = groups(m, n, k), steps = (k + 16 * ks - 1) / (16 * ks);
+  const bool ext = n == DP;
+  const int nb = ext ? D / 8 : (n + 7) / 8, units = m / 16 * nb;
+  if (m > 16 && k > 16 && units >= 2 * (NT / 32))
+    product_blocks<2>(m, n, nb, k, ks, a, b, put);
+  else
+    product_blocks<1>(m, n, nb, k, ks, a, b, put);
   if (ext)
     for (int i = threadIdx.x; i < m; i += NT) {
       float sum = 0.f;
@@ -119,7 +145,7 @@ __device__ __forceinline__ float warp_sum(float s) {
   return s;
 }
 
-__global__ void __launch_bounds__(NT) k_stack_tail(const __grid_constant__ Args A) {
+__global__ void __launch_bounds__(NT, 2) k_stack_tail(const __grid_constant__ Args A) {
   __shared__ float xn2[128], rowdot[64], omn[256], den[64], usum[128];
   const int T = A.T, M = A.M, b = A.b, tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
   const size_t c = blockIdx.x, row0 = c * b;
