@@ -728,20 +728,27 @@ __global__ void __launch_bounds__(kThreads, D <= 64 ? 2 : 1)
 // at the end.  Where the columns leave half of the warps free (d = 64 and less) two
 // warps share a column block, each with every other k16 step.  Scores, den and masks as
 // in k_out, warp (r, h) with rows 16 r .. 16 r + 15 and half of the tile's keys.
-template <typename IO, int D>
+// CAUSAL false: the non-causal readout, all tiles from one state, absent tiles left out; two
+// CTAs on an SM where they fit (600 chains of 9 rows, d = 64, M = 128, bf16: 139 -> 106 us for the
+// whole forward; as an argument of the causal kernel the same cost its C = 16 step 0.4 %).
+template <typename IO, int D, bool CAUSAL>
 struct ShortSmemOut {
   static constexpr int NX = Pieces<IO>::NX, NS = Pieces<IO>::NS, PD = D + 8;
   static constexpr int xs = kTile * fp_pitch<D>() * 4, om = D * 64 * 4, ph = NS * 64 * kPF * 2,
-                       v = NX * kTile * PD * 2, zs = 4 * 64 * 4;
-  static constexpr int bytes = xs + om + 2 * ph + v + zs + 2 * kTile * 4;
+                       kp = CAUSAL ? ph : 0, v = CAUSAL ? NX * kTile * PD * 2 : 0, zs = 4 * 64 * 4;
+  static constexpr int bytes = xs + om + ph + kp + v + zs + 2 * kTile * 4;
   static constexpr int NCB = D / 16, NH = D == 128 ? 1 : 2;
   static_assert(NH == 1 || NCB * 32 * 64 * 4 <= xs + om, "the second halves' sums");
   static_assert(bytes <= kSmemMax, "shared memory");
+  // without scores and state products two CTAs fit an SM; for d < 64, and for bf16 at
+  // d = 128, they would spill (17 chains of 216 rows, C = 7, d = 128: 130 us against 114)
+  static constexpr int ctas = !CAUSAL && (D == 64 || (D == 128 && NX == 3)) ? 2 : 1;
+  static_assert(ctas == 1 || 2 * (bytes + 1024) <= 233472, "two CTAs on an SM");
 };
 
-template <typename IO, int D, int MODE>
-__global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant__ TileArgs A) {
-  using S = ShortSmemOut<IO, D>;
+template <typename IO, int D, int MODE, bool CAUSAL>
+__global__ void __launch_bounds__(kThreads, (ShortSmemOut<IO, D, CAUSAL>::ctas)) k_out_short(const __grid_constant__ TileArgs A) {
+  using S = ShortSmemOut<IO, D, CAUSAL>;
   constexpr int NX = S::NX, NS = S::NS, PD = S::PD, NCB = S::NCB, NH = S::NH;
   constexpr int GN = NH == 1 && MODE == 2 && NS == 2 ? 4 : 2;          // readout groups of a warp, at most
   constexpr int GA = MODE == 1 ? 2 : NS == 2 ? 8 : 4;                  // score groups, at most
@@ -753,7 +760,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
   float* om = xs + S::xs / 4;
   bf16* Ph = reinterpret_cast<bf16*>(om + S::om / 4);
   bf16* Kp = Ph + S::ph / 2;
-  bf16* Vs = Kp + S::ph / 2;
+  bf16* Vs = Kp + S::kp / 2;
   float* zs = reinterpret_cast<float*>(Vs + S::v / 2);  // [tile][64]: z (d >= 64: rounded to the pieces)
   float* norm2 = zs + 4 * 64;
   float* den_s = norm2 + kTile;
@@ -770,11 +777,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
   const long long plo = A.p_lo;                           // from the pair's values to its errors
   const float* zd = A.zdelta + ((size_t)f.c * A.nt + f.t0) * A.M;
   const bf16* pk = A.phi_k + (size_t)frame * NS * 64 * A.M;
+  const bool causal = CAUSAL && A.causal;
   const bool square = A.feature == SLIM_FEAT_SQUARE;
   const int k0 = MODE == 1 ? 32 * ti + 16 * h : r0;       // first key of this warp's scores
 
   auto stage_keys = [&](int c0) {
-    if (A.causal)
+    if (causal)
       stage_rows<NS>(Kp, 64 * kPF, kPF, pk + c0, (size_t)64 * A.M, A.M, 64, min(64, A.M - c0));
     cp_commit();
   };
@@ -785,7 +793,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
   stage_om(0);
   stage_keys(0);
   load_rows_fp<IO, D>(A, f, static_cast<const IO*>(A.q) + f.row0 * D, xs);
-  load_rows<IO, D>(A, f, static_cast<const IO*>(A.v) + f.row0 * D, Vs, nullptr);
+  if (CAUSAL) load_rows<IO, D>(A, f, static_cast<const IO*>(A.v) + f.row0 * D, Vs, nullptr);
   __syncthreads();
   row_norms<D>(xs, norm2);
   pdl_wait();  // the state; the rest is older
@@ -800,6 +808,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
     // the chunk's state at the frame's start: element i of step s is column cb + g + 8
     // ((i >> 1) & 1), feature c0 + 16 s + 2 t + (i & 1) + 8 (i >> 2)
     float hi[4][8], lo[4][8];
+    auto value = [&](int s, int i) { return S::ctas == 1 ? hi[s][i] + lo[s][i] : hi[s][i]; };
 #pragma unroll
     for (int s = 0; s < 4; ++s)
 #pragma unroll
@@ -807,8 +816,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
         hi[s][i] = lo[s][i] = 0.f;
         if (own(s) && 16 * s < nf) {
           const float* p = Pt + (size_t)(c0 + 16 * s + 2 * t + (i & 1) + 8 * (i >> 2)) * D + cb + g + 8 * ((i >> 1) & 1);
-          hi[s][i] = p[0];
-          lo[s][i] = p[plo];
+          if (S::ctas == 1) {
+            hi[s][i] = p[0];
+            lo[s][i] = p[plo];
+          } else {  // at once: 128 registers
+            hi[s][i] = p[0] + p[plo];
+          }
         }
       }
     cp_wait<1>();
@@ -822,7 +835,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
         if (j < ntl) {
           const float z = zh + zl;
           zs[j * 64 + tid] = ZM ? z : round_pieces<NS>(z);
-          if (A.causal) pair_add(zh, zl, zd[(size_t)j * A.M + c0 + tid]);
+          if (causal) pair_add(zh, zl, zd[(size_t)j * A.M + c0 + tid]);
         }
     }
     cp_wait<0>();
@@ -836,13 +849,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
         const int gn = halves ? (A.ks_n == 4 ? s >> 1 : 0) : s & (A.ks_n - 1);
 #pragma unroll
         for (int j = 0; j < NTI; ++j) {
-          if (MODE == 1 && j >= ntl) break;
+          if ((MODE == 1 || !CAUSAL) && j >= ntl) break;
           uint32_t b[NS][4];
 #pragma unroll
           for (int q = 0; q < 2; ++q) {
             uint32_t w0[NS], w1[NS];
-            split_pair<NS>(hi[s][2 * q] + lo[s][2 * q], hi[s][2 * q + 1] + lo[s][2 * q + 1], w0);
-            split_pair<NS>(hi[s][4 + 2 * q] + lo[s][4 + 2 * q], hi[s][5 + 2 * q] + lo[s][5 + 2 * q], w1);
+            split_pair<NS>(value(s, 2 * q), value(s, 2 * q + 1), w0);
+            split_pair<NS>(value(s, 4 + 2 * q), value(s, 5 + 2 * q), w1);
 #pragma unroll
             for (int p = 0; p < NS; ++p) {
               b[p][2 * q] = w0[p];
@@ -858,7 +871,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
 #pragma unroll
             for (int q = 0; q < GN; ++q)
               if (q == gn) mma_pieces<NS, NS>(num[q][rb][0], num[q][rb][1], a, b);
-            if (A.causal && j + 1 < (MODE == 1 ? ntl : NTI)) {  // Delta^T, the pieces' products in Delta's order
+            if (causal && j + 1 < (MODE == 1 ? ntl : NTI)) {  // Delta^T, the pieces' products in Delta's order
               uint32_t v[NX][4], k[NS][4];
               ld_at<NX>(v, Vs, kTile * PD, PD, cb, 16 * rb);
               ld_bt<NS>(k, Kp, 64 * kPF, kPF, 16 * s, 16 * rb);
@@ -872,7 +885,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
                   }
             }
           }
-          if (A.causal && j + 1 < (MODE == 1 ? ntl : NTI)) {
+          if (causal && j + 1 < (MODE == 1 ? ntl : NTI)) {
 #pragma unroll
             for (int i = 0; i < 8; ++i) pair_add(hi[s][i], lo[s][i], d[i >> 2][i & 3]);
           }
@@ -897,7 +910,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
               for (int x = 0; x <= o; ++x) mma16816(dz[q], a[x], w0[o - x], w1[o - x]);
           }
       }
-      if (A.causal) {
+      if (causal) {
         uint32_t b[NS][4];
         if (MODE == 2) {
           ld_b<NS>(b, Kp, 64 * kPF, kPF, r0, 16 * s);
@@ -952,7 +965,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
 #pragma unroll
       for (int i = 0; i < 32; ++i) red[(q * 32 + i) * 32] = num[q][i >> 3][(i >> 2) & 1][i & 3];
   }
-  if (A.causal) {
+  if (causal) {
     // masked scores as pieces, in g(Q)'s place
 #pragma unroll
     for (int q = 1; q < GA; ++q)
@@ -975,7 +988,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
       }
   }
   __syncthreads();
-  if (A.causal) {
+  if (causal) {
     if (ZM && h == 1) {
       float az[4] = {};
 #pragma unroll
@@ -1015,7 +1028,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_out_short(const __grid_constant
 #pragma unroll
   for (int rb = 0; rb < 4; ++rb) {
     float av[2][4] = {};
-    if (A.causal) {
+    if (causal) {
 #pragma unroll
       for (int kb = 0; kb < 4; ++kb)
         if (kb <= rb && kb / RB == rb / RB) {
@@ -1894,12 +1907,12 @@ cudaError_t run_delta(const TileArgs& A, cudaStream_t s) {
   const dim3 grid(frames, room < 2 ? 1 : room < chunks ? room : chunks);
   return launch_pdl(k_delta<IO, D>, grid, kThreads, smem, s, A);
 }
-template <typename IO, int D, int MODE>
+template <typename IO, int D, int MODE, bool CAUSAL>
 cudaError_t run_out_short(const TileArgs& A, cudaStream_t s) {
-  constexpr int smem = ShortSmemOut<IO, D>::bytes;
-  cudaError_t e = smem_limit<IO, D, 4 + MODE>((const void*)k_out_short<IO, D, MODE>, smem);
+  constexpr int smem = ShortSmemOut<IO, D, CAUSAL>::bytes;
+  cudaError_t e = smem_limit<IO, D, 2 + 2 * MODE + CAUSAL>((const void*)k_out_short<IO, D, MODE, CAUSAL>, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_out_short<IO, D, MODE>, (unsigned)(A.chains * A.nf), kThreads, smem, s, A);
+  return launch_pdl(k_out_short<IO, D, MODE, CAUSAL>, (unsigned)(A.chains * A.nf), kThreads, smem, s, A);
 }
 template <typename IO, int D>
 cudaError_t run_out(const TileArgs& A, cudaStream_t s) {
@@ -1907,8 +1920,8 @@ cudaError_t run_out(const TileArgs& A, cudaStream_t s) {
   const double proj = A.feature == SLIM_FEAT_SQUARE ? 0.0 : 2.0;
   prof::Scope ps(prof::K_TILE_OUT, s, (2.0 + proj) * rows * D * A.M,
                  (A.causal ? 3.0 : 2.0) * rows * D * sizeof(IO));
-  if (A.rows == 16) return run_out_short<IO, D, 2>(A, s);
-  if (A.rows == 32) return run_out_short<IO, D, 1>(A, s);
+  if (A.rows == 16) return A.causal ? run_out_short<IO, D, 2, true>(A, s) : run_out_short<IO, D, 2, false>(A, s);
+  if (A.rows == 32) return A.causal ? run_out_short<IO, D, 1, true>(A, s) : run_out_short<IO, D, 1, false>(A, s);
   constexpr int smem = OutSmem<IO, D>::bytes;
   cudaError_t e = smem_limit<IO, D, 1>((const void*)k_out<IO, D>, smem);
   if (e != cudaSuccess) return e;
