@@ -388,12 +388,15 @@ __device__ __forceinline__ void group_publish(int id) {
   tc_fence_after();
 }
 // Bounded poll of a flag by one thread: returns once *flag == want (then an
-// acquire fence).  The first polls come back to back (each is an L2 round trip
-// anyway): a sleep between them is added to every hop of a chain (bench step
-// 739 -> 732 us without it).  It gives up after kWaitLimitNs (or kWaitMaxPolls polls), or
-// early once another CTA has reported an error (checked every 64 polls, so
-// that waiting CTAs do not all hammer the error word); a wait that gives up
-// records itself through give_up(err).
+// acquire fence).  eager: the first polls come back to back (each is an L2 round trip
+// anyway), where the hops bound the launch (by_warp_hops): a sleep between them is added
+// to every hop of a chain (8 chains, L8192 C512: 451 us a step with it, 426 without).  Where
+// the tiles do, polls only take issue slots and L2 from them (64 chains, L4096: 734
+// with the sleeps, 739 without; 256 chains, L1024: 767, 775).  It gives up after
+// kWaitLimitNs (or kWaitMaxPolls polls), or early once another CTA has
+// reported an error (checked every 64 polls, so that waiting CTAs do not all hammer the
+// error word); a wait that gives up records itself through give_up(err).
+template <bool eager>
 __device__ __forceinline__ bool flag_poll(const int* flag, int want, int* err) {
   uint64_t t0 = 0;
   for (uint32_t i = 0; i < kWaitMaxPolls; ++i) {
@@ -406,7 +409,10 @@ __device__ __forceinline__ bool flag_poll(const int* flag, int want, int* err) {
       if (i == 63) t0 = globaltimer_ns();
       else if (globaltimer_ns() - t0 > kWaitLimitNs) break;
     }
-    if (i >= 64) __nanosleep(64);
+    if (!eager)
+      __nanosleep(i < 16 ? 32 : 256);
+    else if (i >= 64)
+      __nanosleep(64);
   }
   give_up(err);
   return false;
@@ -424,7 +430,7 @@ __device__ __forceinline__ bool chain_wait(const int* flag, bool seen, int want,
   if (wait && ok && (threadIdx.x & (by_warp ? 31 : GRP - 1)) == 0) {
     if (seen)
       fence_acq_rel_gpu();
-    else if (!flag_poll(flag, want, err)) {
+    else if (!flag_poll<by_warp>(flag, want, err)) {
       *fail = 1;
       ok = false;
     }
@@ -461,7 +467,7 @@ __device__ __forceinline__ bool flag_poll2(const int* f1, int w1, const int* f2,
       if (i == 63) t0 = globaltimer_ns();
       else if (globaltimer_ns() - t0 > kWaitLimitNs) break;
     }
-    if (i >= 64) __nanosleep(64);
+    __nanosleep(i < 16 ? 32 : 256);
   }
   give_up(err);
   return false;
@@ -483,7 +489,7 @@ __device__ __forceinline__ bool counter_poll(const int* ctr, int want, int* err)
       if (i == 63) t0 = globaltimer_ns();
       else if (globaltimer_ns() - t0 > kWaitLimitNs) break;
     }
-    if (i >= 64) __nanosleep(64);
+    __nanosleep(i < 16 ? 32 : 256);
   }
   give_up(err);
   return false;
@@ -1602,7 +1608,7 @@ __device__ __forceinline__ void role_bwd_kv(const BwdKVJob& J, int t, int c, uin
     for (int h = 0; h < C::MH; ++h) ld_lm16(dqp, h, cg, row, wq[h]);
     // slice n+1's dOmega sum at this position, added to after the next waits
     if (tid == POLL && !acc_first &&
-        !flag_poll(J.accflag + tf * FLAG_STRIDE, J.n + 2, J.err))
+        !flag_poll<false>(J.accflag + tf * FLAG_STRIDE, J.n + 2, J.err))
       abort_ = 1;
     TC_WAIT(sy);
     TC_WAIT(sy);
