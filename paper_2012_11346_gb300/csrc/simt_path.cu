@@ -60,8 +60,8 @@ namespace {
 // loses much of its last one.  Train steps at 304 / 1216 / 2432 frames: [4,12,8192]
 // fp32 relu, C = 512 (384 frames a slice) 6.43 / 5.46 / 5.36 ms; non-causal [8,8,4096]
 // bf16, C = 1024 (1024 frames) 2.52 / 2.52 / 2.28 ms; L = 65536, C = 16 9.17 / 8.95 /
-// 9.08 ms: short slices gain nothing from more than the first two (200 KB to 600 KB of
-// scratch a frame).
+// 9.08 ms.  Short slices stay at the first: 1 to 2 % is not worth four to eight times the
+// scratch (0.2 GB there).
 constexpr int kSeqFrames = 2 * kSms;  // two CTAs on each SM
 constexpr int kMostFrames = 16 * kSms;
 constexpr int kSeqSlices = 8;

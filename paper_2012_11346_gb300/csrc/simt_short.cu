@@ -5,8 +5,8 @@
 // four launches it took 70 us for one row of 64 chains (d = 64, M = 256, bf16), where
 // its traffic (the state in and out, 8.6 MB) is 1.3 us; in one launch it
 // takes 13 us, most of it the host's call.  The arithmetic is that of one 16-row
-// tile of the general kernels (simt_tiles.cuh), operation for operation, so the
-// results are the same bits and a backward may follow.
+// tile of the general kernels (simt_tiles.cuh), the same sums in the same order, the bound
+// of ReLU's recheck included, so the results are the same bits and a backward may follow.
 #include <math.h>
 
 #include "simt_short.h"

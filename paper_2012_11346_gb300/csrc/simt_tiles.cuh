@@ -250,7 +250,8 @@ __device__ __forceinline__ void features_to_pieces(const TileArgs& A, const Fram
 }
 
 // ------------------------------------------------------------------ Delta_t
-// One CTA per frame: g(K) and, tile by tile, Delta_t = g(K)^T [V | 1].  Features
+// One CTA per frame (several where frames are few, see run_delta): g(K) and, tile by tile,
+// Delta_t = g(K)^T [V | 1].  Features
 // are taken 64 at a time: project (FMA pipe), split into pieces in shared memory,
 // then the tile products from there.  g(K)'s pieces are kept for the kernels that
 // read the frame's keys.  The z column (sum of g(K) over the tile's rows) is a

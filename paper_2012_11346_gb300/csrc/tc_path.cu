@@ -391,8 +391,8 @@ __device__ __forceinline__ void group_publish(int id) {
 // acquire fence).  eager: the first polls come back to back (each is an L2 round trip
 // anyway), where the hops bound the launch (by_warp_hops): a sleep between them is added
 // to every hop of a chain (8 chains, L8192 C512: 451 us a step with it, 426 without).  Where
-// the tiles do, polls only take issue slots and L2 from them (64 chains, L4096: 734
-// with the sleeps, 739 without; 256 chains, L1024: 767, 775).  It gives up after
+// the tiles do, polls only take issue slots and L2 from them (256 chains, L1024: 767 with
+// the sleeps, 775 without; 64 chains, L4096: 734, and 734 to 739 by GPU).  It gives up after
 // kWaitLimitNs (or kWaitMaxPolls polls), or early once another CTA has
 // reported an error (checked every 64 polls, so that waiting CTAs do not all hammer the
 // error word); a wait that gives up records itself through give_up(err).
